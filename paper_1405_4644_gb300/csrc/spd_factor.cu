@@ -63,7 +63,7 @@ spd_status leaf_potrf(FCtx& c, int k, int nb) {
             F->W64, F->ldw, k, nb, F->Dinv64, c.mir, c.h->dst);
     } else {
         ++(c.h)->launches;
-        CUDA_TRY(c.h, launch_pdl(k_potrf_leaf32, dim3(1), dim3(256), potrf_leaf32_smem(), c.h->stream, F->W, F->ldw, k,
+        CUDA_TRY(c.h, launch_pdl(k_potrf_leaf32, dim3(1), dim3(LEAF_THREADS), potrf_leaf32_smem(), c.h->stream, F->W, F->ldw, k,
                                  nb, F->Dinv32, c.mir, c.h->dst));
     }
     LAUNCH_CHECK(c.h);

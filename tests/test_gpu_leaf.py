@@ -1,0 +1,60 @@
+"""The 128 x 128 leaf of the float32 factor: where its micro-steps, steps and
+barriers meet, the pivots that break down, and subnormal pivots."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1405_4644_gb300 as spd
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+from tests.gpu_util import check, dev_sym, factor_L  # noqa: E402
+
+
+@pytest.fixture(scope="module")
+def h():
+    import torch
+    hh = spd.spd_create(torch.cuda.current_stream())
+    yield hh
+    spd.spd_destroy(hh)
+
+
+@pytest.mark.parametrize("n", [4, 5, 32, 36, 63, 64, 65, 96, 100, 125, 126, 160, 255, 256])
+def test_leaf_edges(h, n):
+    A = W.gram_shifted(n, seed=n, shift=0.3)
+    d = 1.0 / np.sqrt(np.diag(A))
+    As = d[:, None] * A * d
+    st, F, _ = spd.spd_factor(h, dev_sym(A), "fp32")
+    check(h, st)
+    L, _, _ = factor_L(F)
+    spd.spd_factor_destroy(F)
+    # a float32 factor: ||L L^T - As|| <= c n 2^-24 ||As||, forward kappa times that
+    u, k = 2.0 ** -24, np.linalg.cond(As)
+    assert np.linalg.norm(L @ L.T - As) <= 4 * max(n, 8) ** 0.5 * u * np.linalg.norm(As)
+    R = oracle.potrf(As).T
+    assert np.max(np.abs(L - R)) <= 8 * k * max(n, 8) ** 0.5 * u * np.max(np.abs(R))
+
+
+@pytest.mark.parametrize("col", [1, 3, 4, 5, 31, 32, 35, 63, 64, 95, 96, 126, 127, 130])
+def test_breakdown_names_the_column(h, col):
+    A = np.eye(140)
+    A[col, col - 1] = A[col - 1, col] = 1.5  # pivot of `col`: 1 - 2.25
+    st, F, rep = spd.spd_factor(h, dev_sym(A), "fp32")
+    assert st == spd.SPD_ERR_NOT_SPD and F is None
+    assert rep.info == col + 1
+
+
+@pytest.mark.parametrize("col", [0, 2, 33, 127])
+def test_subnormal_pivot(h, col):
+    """Without the diagonal scaling a pivot may be subnormal in float32: its square root is still taken."""
+    n = 130
+    A = np.eye(n)
+    A[col, col] = 2.0 ** -140
+    st, F, _ = spd.spd_factor(h, dev_sym(A), "fp32", flags=0)
+    check(h, st)
+    L, _, _ = factor_L(F)
+    spd.spd_factor_destroy(F)
+    want = np.eye(n)
+    want[col, col] = 2.0 ** -70
+    assert np.max(np.abs(L - want) / np.where(want > 0, want, 1.0)) <= 2.0 ** -21
