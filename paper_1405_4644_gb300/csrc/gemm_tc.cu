@@ -227,9 +227,9 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (st->flags & (SPD_DEV_BREAKDOWN | SPD_DEV_NONFINITE | SPD_DEV_BADDIAG)) return;
     const int g = blockIdx.x;
-    const long u0 = unit_begin(g, W, G), u1 = unit_begin(g + 1, W, G);
+    const long u0 = unit_begin(g, W, G);
+    long u1 = unit_begin(g + 1, W, G);
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
             tc::mbar_init(&accempty[b], 4);
         }
         for (int w = 0; w < 4; ++w) tc::mbar_init(&cbar[w], 1);
-        *abort_flag = 0;
+        abort_flag[0] = 0;
         tc::fence_barrier_init();
         tc::prefetch_tmap(&mapA);
         tc::prefetch_tmap(&mapB);
@@ -251,10 +251,15 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
         tc::tmem_alloc(tmem_slot, TMEM_COLS);
         tc::tmem_relinquish();
     }
+    pdl_wait();  // (launched as a programmatic dependent) the operands and C are the previous kernels'
+    if (threadIdx.x == 0)  // one reader: another stream's kernel may be raising a flag just now
+        abort_flag[1] = *reinterpret_cast<volatile int*>(&st->flags) &
+                        (SPD_DEV_BREAKDOWN | SPD_DEV_NONFINITE | SPD_DEV_BADDIAG);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
     const uint32_t tmem = *tmem_slot;
+    if (abort_flag[1]) u1 = u0;  // the factorisation is over: no pieces
     bool ok = true;
 
     // pieces of [u0, u1): tile t, K tiles [kb, ke); tiles wholly above the
@@ -706,34 +711,45 @@ namespace {
 template <int BNT>
 void launch_kind(TcGemm* g, cudaStream_t s, int G, int cx0, int cy0, int M, int N, int a_row0, int b_row0, int k0,
                  int lower, float scale, int nseg, uint32_t segs, uint32_t accsel, int tiles_n, int nk, long W,
-                 float* Cpart, DevStatus* st) {
+                 float* Cpart, DevStatus* st, bool pdl) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(G);
+    cfg.blockDim = dim3(192);
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = pdl ? 1 : 0;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
     const CUtensorMap& mb = (BNT == 128 && !g->narrow) ? g->mapB128 : g->mapB;
     const uint32_t idesc = idesc_for(g->kind, BNT);
     float* Cb = g->C + (long)cy0 * g->ldc + cx0;  // the block's origin (epilogue without a tensor map)
-#define SPD_GEMM_ARGS                                                                                            \
+#define SPD_GEMM_LAUNCH(kernel, smem)                                                                            \
+    cfg.dynamicSmemBytes = smem;                                                                                 \
+    cudaLaunchKernelEx(&cfg, kernel, \
     g->mapA, mb, g->mapC, g->has_map_c ? 1 : 0, Cb, g->ldc, cx0, cy0, M, N, a_row0, b_row0, k0, lower, idesc, \
-        scale, nseg, segs, accsel, tiles_n, nk, W, G, Cpart, st
+        scale, nseg, segs, accsel, tiles_n, nk, W, G, Cpart, st)
     if constexpr (BNT <= 64) {  // narrow tiles: float32 as bf16 slices, all slices in one stage
-        k_gemm_tc<0, BNT, 3, 2, 3><<<G, 192, smem_bytes<BNT, 3, 3>(), s>>>(SPD_GEMM_ARGS);
+        SPD_GEMM_LAUNCH((k_gemm_tc<0, BNT, 3, 2, 3>), (smem_bytes<BNT, 3, 3>()));
     } else {
         switch (g->kind) {
-            case 1: k_gemm_tc<1, BNT, 4, 1><<<G, 192, smem_bytes<BNT, 4>(), s>>>(SPD_GEMM_ARGS); break;
+            case 1: SPD_GEMM_LAUNCH((k_gemm_tc<1, BNT, 4, 1>), (smem_bytes<BNT, 4>())); break;
             case 5: {  // float32 as bf16 slices: two accumulators; two CTAs per SM on 128-wide tiles
                 constexpr int ST = BNT == 128 ? 3 : 4;
-                k_gemm_tc<0, BNT, ST, 2><<<G, 192, smem_bytes<BNT, ST>(), s>>>(SPD_GEMM_ARGS);
+                SPD_GEMM_LAUNCH((k_gemm_tc<0, BNT, ST, 2>), (smem_bytes<BNT, ST>()));
                 break;
             }
-            case 4: k_gemm_tc<2, BNT, 4, 1><<<G, 192, smem_bytes<BNT, 4>(), s>>>(SPD_GEMM_ARGS); break;
-            default: k_gemm_tc<0, BNT, 4, 1><<<G, 192, smem_bytes<BNT, 4>(), s>>>(SPD_GEMM_ARGS);
+            case 4: SPD_GEMM_LAUNCH((k_gemm_tc<2, BNT, 4, 1>), (smem_bytes<BNT, 4>())); break;
+            default: SPD_GEMM_LAUNCH((k_gemm_tc<0, BNT, 4, 1>), (smem_bytes<BNT, 4>()));
         }
     }
-#undef SPD_GEMM_ARGS
+#undef SPD_GEMM_LAUNCH
 }
 
 }  // namespace
 
 spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, int N, int K, int a_row0, int b_row0,
-                          int k0, int lower, DevStatus* st, int splits, const TcSplit* sb) {
+                          int k0, int lower, DevStatus* st, int splits, const TcSplit* sb, bool pdl) {
     const int bk = g->kind == 1 ? 32 : g->kind == 4 ? 128 : 64;
     if (M <= 0 || N <= 0 || K <= 0) return SPD_OK;
     if (K % bk != 0 || (k0 * elem_bytes(g->kind)) % 16 != 0 || cx0 % 4 != 0) return SPD_ERR_ARG;
@@ -786,16 +802,16 @@ spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, in
     if (G != T && !part) return SPD_ERR_ARG;
     if (bnt == 32)
         launch_kind<32>(g, s, G, cx0, cy0, M, N, a_row0, b_row0, k0, lower, scale, nseg, segs, accsel, tiles_n, nk,
-                        W, part, st);
+                        W, part, st, pdl);
     else if (bnt == 64)
         launch_kind<64>(g, s, G, cx0, cy0, M, N, a_row0, b_row0, k0, lower, scale, nseg, segs, accsel, tiles_n, nk,
-                        W, part, st);
+                        W, part, st, pdl);
     else if (bnt == 128)
         launch_kind<128>(g, s, G, cx0, cy0, M, N, a_row0, b_row0, k0, lower, scale, nseg, segs, accsel, tiles_n, nk,
-                         W, part, st);
+                         W, part, st, pdl);
     else
         launch_kind<256>(g, s, G, cx0, cy0, M, N, a_row0, b_row0, k0, lower, scale, nseg, segs, accsel, tiles_n, nk,
-                         W, part, st);
+                         W, part, st, pdl);
     if (part) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(BM / 16, (unsigned)T);  // 16 rows of one tile per block
@@ -815,8 +831,8 @@ spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, in
 }
 
 spd_status tc_gemm_run(TcGemm* g, cudaStream_t s, int r0, int M, int c0, int N, int k0, int K, int lower,
-                       DevStatus* st, int splits, const TcSplit* sb) {
-    return tc_gemm_launch(g, s, r0, c0, M, N, K, r0, c0, k0, lower, st, splits, sb);
+                       DevStatus* st, int splits, const TcSplit* sb, bool pdl) {
+    return tc_gemm_launch(g, s, r0, c0, M, N, K, r0, c0, k0, lower, st, splits, sb, pdl);
 }
 
 void tc_gemm_destroy(TcGemm* g) { delete g; }

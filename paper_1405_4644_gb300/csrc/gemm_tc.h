@@ -25,8 +25,9 @@ spd_status tc_gemm_create(TcGemm** out, float* W, long ldw, void* Wh, long ldh, 
 // 128 x 128 floats suffice) that a dependent kernel adds to C in K order.
 // splits = 0 takes stream-K whenever it gives more CTAs than tiles (on all
 // SMs).  Otherwise (splits = 1, or without room in sb) one CTA per tile.
+// pdl: launched as a programmatic dependent of the previous kernel in s.
 spd_status tc_gemm_run(TcGemm* g, cudaStream_t s, int r0, int M, int c0, int N, int k0, int K, int lower,
-                       DevStatus* st, int splits = 1, const TcSplit* sb = nullptr);
+                       DevStatus* st, int splits = 1, const TcSplit* sb = nullptr, bool pdl = false);
 void tc_gemm_destroy(TcGemm* g);
 // General form: separate operand arrays (rows x cols, ld elements each) and
 // C (c_rows x c_cols, ldc floats, row-major).
@@ -42,4 +43,4 @@ spd_status tc_gemm_create_narrow(TcGemm** out, const void* Ah, long a_rows, long
 // C[cy0 + i][cx0 + j] -= sum_k A[a_row0 + i][k0 + k] B[b_row0 + j][k0 + k]
 // for i < M, j < N (cx0 a multiple of 4).
 spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, int N, int K, int a_row0, int b_row0,
-                          int k0, int lower, DevStatus* st, int splits = 1, const TcSplit* sb = nullptr);
+                          int k0, int lower, DevStatus* st, int splits = 1, const TcSplit* sb = nullptr, bool pdl = false);

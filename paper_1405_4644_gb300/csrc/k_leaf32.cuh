@@ -18,7 +18,7 @@
 #pragma once
 #include "common.cuh"
 
-#define LD32 129  // k_trsm_leaf32, k_block_inverse
+#define LD32 129  // k_block_inverse
 #define LDL 132   // the leaf: 16-byte rows, eight consecutive rows in distinct banks
 
 // Dinv32 for block b lives at Dinv32 + b * 4096: four row-major 32x32
@@ -317,19 +317,83 @@ __global__ void __launch_bounds__(LEAF_THREADS, 1) k_potrf_leaf32(float* __restr
 // Panel solve for rows [r0, r0 + m) against the factored diagonal block at
 // column c0 (order 128): X L^T = B, in four 32-column steps s:
 //   X_s = B_s D_s^T,   B_s' -= X_s L_s's^T  (s' > s),
-// with D_s the 32x32 inverses the leaf stored.  CTA = 64 rows; each thread
-// owns a 4-row by (2 | 6 - 2 s)-column register tile of each step.
-constexpr size_t trsm_leaf32_smem() { return (size_t)(64 * 132 + 96 * LD32 + 4 * 32 * 33) * sizeof(float); }
+// with D_s the 32x32 inverses the leaf stored.  CTA = 64 rows, two CTAs per SM.
+// Bound: the loads from shared memory (16 bytes per thread and 2.4 cycles of the
+// SM each) of a 4-row tile: thread (rows tr .. tr + 3, column class cg) owns the
+// columns cg, cg + 16, .. of each product, so that eight lanes read eight
+// consecutive rows of the right factor in distinct banks, four k at a time.
+// Measured from the leaf's end to the solve's (globaltimer stamps): 6.4 us with
+// one CTA on an SM (n = 2999; 12.4 us with scalar loads and one k at a time), 9.9
+// us with two (n = 16384; 17 us).
+#define LDB 132  // rows of B and L: 16-byte aligned, consecutive rows 4 banks apart
+#define LDD 36   // rows of D likewise
+constexpr size_t trsm_leaf32_smem() { return (size_t)(64 * LDB + 96 * LDB + 4 * 32 * LDD) * sizeof(float); }
 
-// b_ready: the previous kernel in the stream (the leaf) does not write B,
-// so B is loaded before waiting for it (programmatic dependent launch).
+// acc[j][q] += sum over four k of x[j] y[q]
+template <int NQ>
+__device__ __forceinline__ void trsm_fma4(float (&acc)[4][NQ], const float4 (&x)[4], const float4& y, int q) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        acc[j][q] = fmaf(x[j].x, y.x, acc[j][q]);
+        acc[j][q] = fmaf(x[j].y, y.y, acc[j][q]);
+        acc[j][q] = fmaf(x[j].z, y.z, acc[j][q]);
+        acc[j][q] = fmaf(x[j].w, y.w, acc[j][q]);
+    }
+}
+
+template <int S>
+__device__ __forceinline__ void trsm_step(float* Bs, const float* Ls, const float* Ds, int tr, int cg) {
+    constexpr int o = 32 * S, NQ = 6 - 2 * S;
+    const float* br = Bs + tr * LDB + o;
+    {   // X_s, columns o + cg and o + 16 + cg (D_s is lower triangular: the first ends at k = 15)
+        float x[4][2] = {};
+        const float* d0 = Ds + (o + cg) * LDD;
+#pragma unroll
+        for (int l = 0; l < 32; l += 4) {
+            float4 b[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(br + j * LDB + l);
+            if (l < 16) trsm_fma4<2>(x, b, *reinterpret_cast<const float4*>(d0 + l), 0);
+            trsm_fma4<2>(x, b, *reinterpret_cast<const float4*>(d0 + 16 * LDD + l), 1);
+        }
+        __syncthreads();  // every read of B_s done
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            Bs[(tr + j) * LDB + o + cg] = x[j][0];
+            Bs[(tr + j) * LDB + o + 16 + cg] = x[j][1];
+        }
+    }
+    __syncthreads();
+    if constexpr (S < 3) {  // columns o + 32 + cg + 16 q
+        float acc[4][NQ] = {};
+        const float* lr = Ls + (o + cg) * LDB + o;  // Ls holds rows 32 .. of L_kk
+#pragma unroll 2
+        for (int l = 0; l < 32; l += 4) {
+            float4 b[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) b[j] = *reinterpret_cast<const float4*>(br + j * LDB + l);
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                trsm_fma4<NQ>(acc, b, *reinterpret_cast<const float4*>(lr + 16 * q * LDB + l), q);
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) Bs[(tr + j) * LDB + o + 32 + 16 * q + cg] -= acc[j][q];
+        __syncthreads();
+    }
+}
+
+// b_ready: the previous kernel in the stream (the leaf) does not write B, and
+// what does was complete before the leaf passed its own wait, so B is loaded
+// before waiting (programmatic dependent launch).
 __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, long ldw, int r0, int m, int c0,
                                                      const float* __restrict__ Dinv32, Mirror mir,
                                                      const DevStatus* st, int b_ready) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* Bs = reinterpret_cast<float*>(smem_raw);  // [64][132] B, becoming X
-    float* Ls = Bs + 64 * 132;                       // [96][129] rows 32..127 of L_kk, columns 0..95
-    float* Ds = Ls + 96 * LD32;                      // [4][32][33] D_s
+    float* Ls = Bs + 64 * LDB;                       // [96][132] rows 32..127 of L_kk, columns 0..95
+    float* Ds = Ls + 96 * LDB;                       // [4][32][36] D_s
     const int tid = threadIdx.x;
     const int rb0 = r0 + blockIdx.x * 64;
     {
@@ -342,9 +406,9 @@ __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, l
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
         }
         if (b_ready) pdl_wait();  // L_kk and its inverses come from the previous kernel
-        if (st->flags & (SPD_DEV_BREAKDOWN | SPD_DEV_NONFINITE | SPD_DEV_BADDIAG)) return;
-        // the strictly-below-diagonal 32-blocks of L_kk (rows 32..127, columns
-        // 0..95) and the four 32x32 inverses: every load in flight first
+        const int flags = *reinterpret_cast<const volatile int*>(&st->flags);
+        // rows 32..127 of L_kk, columns 0..95 (the 32-blocks below the diagonal
+        // are used) and the four 32x32 inverses: every load in flight first
         float4 vl[9], vd[4];
 #pragma unroll
         for (int q = 0; q < 9; ++q) {
@@ -353,91 +417,36 @@ __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, l
         }
         const float4* dg = reinterpret_cast<const float4*>(Dinv32 + (long)(c0 / 128) * 4096);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) vd[q] = __ldg(dg + tid + q * 256);
-#pragma unroll
-        for (int q = 0; q < 9; ++q) {
-            const int e = tid + q * 256, r = e / 24, c4 = (e - r * 24) * 4;
-            float* d = Ls + r * LD32 + c4;
-            d[0] = (c4 + 0 < r + 32) ? vl[q].x : 0.f;
-            d[1] = (c4 + 1 < r + 32) ? vl[q].y : 0.f;
-            d[2] = (c4 + 2 < r + 32) ? vl[q].z : 0.f;
-            d[3] = (c4 + 3 < r + 32) ? vl[q].w : 0.f;
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int e = (tid + q * 256) * 4, i = e >> 5, c = e & 31;
-            float* d = Ds + i * 33 + c;
-            d[0] = vd[q].x;
-            d[1] = vd[q].y;
-            d[2] = vd[q].z;
-            d[3] = vd[q].w;
-        }
+        for (int q = 0; q < 4; ++q) vd[q] = dg[tid + q * 256];
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
             const int e = tid + q * 256, r = e >> 5, c4 = (e & 31) * 4;
-            *reinterpret_cast<float4*>(Bs + r * 132 + c4) = vb[q];
+            *reinterpret_cast<float4*>(Bs + r * LDB + c4) = vb[q];
         }
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            const int e = tid + q * 256, r = e / 24, c4 = (e - r * 24) * 4;
+            *reinterpret_cast<float4*>(Ls + r * LDB + c4) = vl[q];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int e = tid + q * 256, r = e >> 3, c4 = (e & 7) * 4;
+            *reinterpret_cast<float4*>(Ds + r * LDD + c4) = vd[q];
+        }
+        if (flags & (SPD_DEV_BREAKDOWN | SPD_DEV_NONFINITE | SPD_DEV_BADDIAG)) return;
     }
     __syncthreads();
-    // thread tile: rows tr..tr+3 (16 row groups) x a column group (16 groups)
-    const int tr = (tid >> 4) * 4, cgp = tid & 15;
-    for (int s = 0; s < 4; ++s) {
-        const int o = s * 32;
-        const float* D = Ds + s * 32 * 33;
-        // X_s, columns o + c, o + c + 1 (D[c][l] = 0 for l > c)
-        const int c = 2 * cgp;
-        float x[4][2];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) x[j][0] = x[j][1] = 0.f;
-        for (int l = 0; l <= c + 1; ++l) {
-            const float d0 = D[c * 33 + l], d1 = D[(c + 1) * 33 + l];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float b = Bs[(tr + j) * 132 + o + l];
-                x[j][0] = fmaf(b, d0, x[j][0]);
-                x[j][1] = fmaf(b, d1, x[j][1]);
-            }
-        }
-        __syncthreads();  // every read of B_s done
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            Bs[(tr + j) * 132 + o + c] = x[j][0];
-            Bs[(tr + j) * 132 + o + c + 1] = x[j][1];
-        }
-        __syncthreads();
-        if (s == 3) break;
-        // B_s' -= X_s L_s's^T for the 96 - 32 s columns to the right: CW each
-        const int CW = 6 - 2 * s;
-        const int cb = o + 32 + cgp * CW;  // first column (= row of L) of this thread
-        float acc[4][6];
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int q = 0; q < 6; ++q) acc[j][q] = 0.f;
-#pragma unroll 2
-        for (int l = 0; l < 32; ++l) {
-            float xv[4], lv[6];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) xv[j] = Bs[(tr + j) * 132 + o + l];
-#pragma unroll
-            for (int q = 0; q < 6; ++q) lv[q] = (q < CW) ? Ls[(cb + q - 32) * LD32 + o + l] : 0.f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int q = 0; q < 6; ++q) acc[j][q] = fmaf(xv[j], lv[q], acc[j][q]);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-#pragma unroll
-            for (int q = 0; q < 6; ++q)
-                if (q < CW) Bs[(tr + j) * 132 + cb + q] -= acc[j][q];
-        __syncthreads();
-    }
+    const int tr = (tid >> 4) * 4, cg = tid & 15;
+    trsm_step<0>(Bs, Ls, Ds, tr, cg);
+    trsm_step<1>(Bs, Ls, Ds, tr, cg);
+    trsm_step<2>(Bs, Ls, Ds, tr, cg);
+    trsm_step<3>(Bs, Ls, Ds, tr, cg);
+    if (tid == 0) pdl_trigger();  // the next block column's update may be scheduled
     for (int e = tid; e < 64 * 32; e += 256) {
         const int rr = e >> 5, c4 = (e & 31) * 4;
         const long row = rb0 + rr;
         if (row >= r0 + m) continue;
-        const float4 v = *reinterpret_cast<const float4*>(Bs + rr * 132 + c4);
+        const float4 v = *reinterpret_cast<const float4*>(Bs + rr * LDB + c4);
         *reinterpret_cast<float4*>(W + row * ldw + c0 + c4) = v;
         mirror_store4(mir, row, (long)(c0 + c4), v);
     }

@@ -89,12 +89,13 @@ spd_status leaf_trsm(FCtx& c, int r0, int m, int c0, int kb, bool b_ready = fals
     return SPD_OK;
 }
 
-// crit: a rank-128 update on the factorisation's critical path (recorded
-// as SPD_PHASE_TRAILING_LAST); otherwise a bulk update.  lower (r0 == c0):
-// only entries with row >= column are updated.
+// near: an update by the nearest block columns, on or beside the
+// factorisation's critical path (recorded as SPD_PHASE_TRAILING_LAST);
+// otherwise a bulk update.  lower (r0 == c0): only entries with row >= column
+// are updated.  pdl: a programmatic dependent of the previous kernel in strm.
 template <typename T>
 spd_status gemm(FCtx& c, int r0, int M, int c0, int N, int k0, int K, int lower, int splits = 1,
-                cudaStream_t strm = nullptr, const TcSplit* sb = nullptr, bool crit = false) {
+                cudaStream_t strm = nullptr, const TcSplit* sb = nullptr, bool near = false, bool pdl = false) {
     if (M <= 0 || N <= 0 || K <= 0) return SPD_OK;
     spd_factor_t* F = c.F;
     cudaStream_t s = strm ? strm : c.h->stream;
@@ -107,7 +108,7 @@ spd_status gemm(FCtx& c, int r0, int M, int c0, int N, int k0, int K, int lower,
     const double opsz = sizeof(T) == 8 ? 8.0
                         : c.mir.kind == 5 ? 6.0
                         : (c.mir.kind == 0 || c.mir.kind == 1 ? 4.0 : c.mir.kind == 4 ? 1.0 : 2.0);
-    const int phase = crit ? SPD_PHASE_TRAILING_LAST
+    const int phase = near ? SPD_PHASE_TRAILING_LAST
                            : (c.tc && c.mir.kind == 5) ? SPD_PHASE_TRAILING_X3 : SPD_PHASE_TRAILING;
     ProfScope ps(c.h, phase, 2.0 * celems * K,
                  2.0 * sizeof(T) * celems + opsz * (double)K * (lower ? M : (double)M + N), s);
@@ -117,7 +118,7 @@ spd_status gemm(FCtx& c, int r0, int M, int c0, int N, int k0, int K, int lower,
                                                                      k0, K, lower, c.h->dst);
     } else {
         if (c.tc) {
-            spd_status st = tc_gemm_run(c.tc, s, r0, M, c0, N, k0, K, lower, c.h->dst, splits, sb);
+            spd_status st = tc_gemm_run(c.tc, s, r0, M, c0, N, k0, K, lower, c.h->dst, splits, sb, pdl);
             if (st != SPD_OK) return set_err(c.h, st, "tensor-core trailing update failed");
             return SPD_OK;
         }
@@ -180,28 +181,32 @@ spd_status potrf_rec(FCtx& c, int n0, int nn) {
     return potrf_rec<T>(c, n0 + n1, nn - n1);
 }
 
-// Left-looking block-column schedule with a look-ahead (tensor-core
-// factors).  Block columns are taken in pairs P = (j, j+1), j even.  Block
-// column k needs every panel to its left applied:
-//   bulk (second stream): W[j:, j:j+2] -= L[j:, 0:j-1] L[j:j+2, 0:j-1]^T
-//        for the whole pair, as soon as panel j-2 is done; 256-wide tiles
-//        (entries above the diagonal are left alone);
-//   last (main stream, rank 128, on the critical path):
-//        block j:   W[j:, j:j+2] -= L[j:, j-1] L[j:j+2, j-1]^T  (both columns)
-//        block j+1: W[j+1:, j+1] -= L[j+1:, j] L[j+1, j]^T
-// each followed by the block's leaf and the panel solve below it.  The bulk
-// update of a pair, which holds nearly all of the tensor-core work, runs
-// while the previous block's last update, leaf and panel run; the bulk
-// update of pair P waits for panel j-2, the last update of block j for the
-// bulk update of its pair (both write W[j:, j:j+2]).
+// Left-looking block-column schedule (tensor-core factors).  Block column k
+// needs every panel to its left applied.  Block columns are taken in pairs
+// (j, j+1), j even; both columns of a pair get
+//   bulk: panels 0 .. j-2, W[j:, j:j+2] -= L[j:, 0:j-1] L[j:j+2, 0:j-1]^T, 256-wide
+//         tiles (entries above the diagonal are left alone), in two launches of
+//         half the panels each;
+//   near: panel j-1 (both columns), and for block j+1 panel j.
+// Step k has two streams:
+//   main:    near update, leaf, panel solve (programmatic dependents);
+//   second:  half a bulk update: of pair k+2 (k even, panels 0 .. a-1) or of pair
+//            k+1 (k odd, panels a .. k-1).
+// The panel solve takes the SMs as the bulk half leaves them.  A bulk half holds
+// all SMs but two for its whole length (equal ranges per CTA, one CTA per SM), so
+// that it has one wave and the leaf an SM: with a CTA on every SM one of them had
+// to wait for the leaf's or the near update's SM and doubled the launch's length,
+// and the leaf waited for the bulk update's end.  Measured with the faster panel
+// solve (k_trsm_leaf32): n = 16384 FP16 22.8 ms a solve (24.9 before), FP32 24.3
+// ms (25.3).
 template <typename T>
 spd_status potrf_left(FCtx& c, int n, bool lookahead) {
     spd_handle* h = c.h;
     const int NB = ceil_div(n, SPD_LEAF);
-    // without the look-ahead both parts run in order on the main stream
+    // without the look-ahead every part runs in order on the main stream
     cudaStream_t P = h->stream, U = lookahead ? h->aux : h->stream;
-    // two events per block: panel done (main), bulk update of the pair
-    // starting at this block done (second)
+    // two events per block: panel done (main), bulk update of the pair starting
+    // at this block done (second)
     const size_t need = 2 * (size_t)NB + 1;
     while (h->sync_ev.size() < need) {
         cudaEvent_t e = nullptr;
@@ -210,44 +215,45 @@ spd_status potrf_left(FCtx& c, int n, bool lookahead) {
     }
     cudaEvent_t* evPanel = h->sync_ev.data();
     cudaEvent_t* evBulk = h->sync_ev.data() + NB;
-    cudaEvent_t evStart = h->sync_ev[2 * NB];
-    CUDA_TRY(h, cudaEventRecord(evStart, P));  // the second stream starts after the conversion
-    CUDA_TRY(h, cudaStreamWaitEvent(U, evStart, 0));
+    cudaEvent_t evEnd = h->sync_ev[2 * NB];
     spd_status st = SPD_OK;
     cudaError_t e = cudaSuccess;
+    auto record = [&](cudaEvent_t ev, cudaStream_t s) {
+        if (lookahead && e == cudaSuccess) e = cudaEventRecord(ev, s);
+    };
+    auto wait = [&](cudaStream_t s, cudaEvent_t ev) {
+        if (lookahead && e == cudaSuccess) e = cudaStreamWaitEvent(s, ev, 0);
+    };
     for (int k = 0; k < NB && st == SPD_OK && e == cudaSuccess; ++k) {
-        const int r0 = k * SPD_LEAF, nb = std::min(SPD_LEAF, n - r0), M = n - r0;
-        const bool pair_start = (k % 2) == 0;
-        if (pair_start && k >= 2) e = cudaStreamWaitEvent(P, evBulk[k], 0);
-        if (e == cudaSuccess && k >= 1) {  // last: rank 128 with block column k-1
-            if (pair_start)
-                st = gemm<T>(c, r0, M, r0, std::min(2 * SPD_LEAF, M), r0 - SPD_LEAF, SPD_LEAF, 1, 1, P, nullptr, true);
-            else
-                st = gemm<T>(c, r0, M, r0, nb, r0 - SPD_LEAF, SPD_LEAF, 0, 1, P, nullptr, true);
-        }
+        const int r0 = k * SPD_LEAF, M = n - r0, nb = std::min(SPD_LEAF, M);
+        const bool first = (k & 1) == 0;    // of its pair
+        const int j = k + (first ? 2 : 1);  // the pair of this step's bulk half: panels [ka, kb)
+        const int a = (j - 1) / 2, ka = first ? 0 : a, kb = first ? a : k;
+        if (first && k >= 2) wait(P, evBulk[k]);
+        if (k > 0 && e == cudaSuccess)
+            st = gemm<T>(c, r0, M, r0, first ? std::min(2 * SPD_LEAF, M) : nb, r0 - SPD_LEAF, SPD_LEAF, first, 1, P,
+                         nullptr, true, true);
         if (e == cudaSuccess && st == SPD_OK) st = leaf_potrf<T>(c, r0, nb);
-        if (e == cudaSuccess && st == SPD_OK && r0 + nb < n)
-            st = leaf_trsm<T>(c, r0 + nb, n - r0 - nb, r0, nb, true);  // right after the leaf
-        if (e != cudaSuccess || st != SPD_OK) break;
-        e = cudaEventRecord(evPanel[k], P);
-        // bulk update of the pair starting at block k+2 on the second stream:
-        // panels 0..k
-        if (e == cudaSuccess && pair_start && k + 2 < NB) {
-            e = cudaStreamWaitEvent(U, evPanel[k], 0);
-            const int r2 = (k + 2) * SPD_LEAF, M2 = n - r2;
-            if (e == cudaSuccess)
-                st = gemm<T>(c, r2, M2, r2, std::min(2 * SPD_LEAF, M2), 0, (k + 1) * SPD_LEAF, 1,
-                             c.bulk ? -h->sms : 1, U, c.bulk);
-            if (e == cudaSuccess) e = cudaEventRecord(evBulk[k + 2], U);
+        if (e == cudaSuccess && st == SPD_OK && M > nb) st = leaf_trsm<T>(c, r0 + nb, M - nb, r0, nb, true);
+        if (j < NB && e == cudaSuccess && st == SPD_OK) {
+            if (k > 0) wait(U, evPanel[k - 1]);
+            if (kb > ka && e == cudaSuccess) {
+                const int r2 = j * SPD_LEAF, M2 = n - r2;
+                st = gemm<T>(c, r2, M2, r2, std::min(2 * SPD_LEAF, M2), ka * SPD_LEAF, (kb - ka) * SPD_LEAF, 1,
+                             c.bulk ? -std::max(1, h->sms - 2) : 1, U, c.bulk);
+            }
+            if (!first) record(evBulk[j], U);
         }
+        record(evPanel[k], P);
     }
     // join, on every path: the main stream continues (and frees the split
     // scratch) only after everything queued on the second stream
-    cudaEvent_t evEnd = h->sync_ev[2 * NB];
-    cudaError_t e2 = cudaEventRecord(evEnd, U);
-    if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(P, evEnd, 0);
-    if (e2 != cudaSuccess) cudaStreamSynchronize(U);
-    if (e == cudaSuccess) e = e2;
+    if (lookahead) {
+        cudaError_t e2 = cudaEventRecord(evEnd, U);
+        if (e2 == cudaSuccess) e2 = cudaStreamWaitEvent(P, evEnd, 0);
+        if (e2 != cudaSuccess) cudaStreamSynchronize(U);
+        if (e == cudaSuccess) e = e2;
+    }
     if (e != cudaSuccess && st == SPD_OK) st = set_err(h, SPD_ERR_CUDA, "look-ahead schedule: %s", cudaGetErrorString(e));
     return st;
 }
