@@ -14,12 +14,18 @@
 // to float32 C in global memory.
 //
 // Float32 operands given as three bf16 slices (s0 + s1 + s2) are multiplied
-// as the six slice products of order <= 2.  The products of one K tile are
-// issued back to back (K outer, slice pair inner), so the three reloads of a
-// slice tile within a K tile are served by L2 and each slice leaves HBM once;
-// the five small products go to one accumulator and s0*t0 to a second one,
-// added once in the epilogue, so no small product is ever rounded against
-// the large partial sums.
+// as the six slice products of order <= 2.  A pipeline stage holds all three
+// slices of both tiles (one TMA load each, a box three planes deep) and the six
+// products of its K are issued from it; the five small products go to one
+// accumulator and s0*t0 to a second one, added once in the epilogue, so no small
+// product is ever rounded against the large partial sums.  What bounds it is the
+// rate at which an SM takes operands from L2, 64 bytes a cycle: with one slice
+// pair per stage every slice was loaded twice (288 KB per 64 of K and 128 x 256
+// tile, 4500 cycles against 3072 of MMA); now once (144 KB).  Three slices of 64
+// of K would leave room for one stage only, so these stages are 32 deep (64-byte
+// rows, 64-byte swizzle).  A float32 solve of n = 32768 went from 99.2 to 93.5
+// ms, of n = 16384 from 24.3 to 23.7; prefetching A's tiles into L2 ahead of
+// their loads made both slower.
 //
 // Epilogue: each warp brings its 32 rows of the C tile into the (now idle)
 // stage buffers with TMA, as 32 x 32 boxes in the 128-byte swizzled layout
@@ -39,19 +45,18 @@
 namespace {
 
 constexpr int BM = 128, BN = 256;
-constexpr int A_STAGE = BM * 128;  // bytes: 128 rows x 128 B
 // The tile width BNT is 256 (trailing updates) or 128 (one block column),
-// with ST pipeline stages: 4 stages and one CTA per SM, or (128-wide tf32
-// tiles, whose six-segment float32 updates are long) 3 stages of 32 KB and
-// two CTAs per SM, so that one CTA's epilogue overlaps the other's main loop.
+// with ST pipeline stages and one CTA per SM.
 // Narrow tiles (BNT = 32 or 64, the skinny products A~ P of CG with m
 // right-hand sides) take all three slices of an A tile and of a B tile in one
 // stage (SL = 3 slices per stage, one TMA load each with a box three planes
 // deep), so that each slice tile crosses from L2 to shared memory once per K
 // tile and the six slice products are issued from the same stage.
-template <int BNT> __host__ __device__ constexpr int b_stage() { return BNT * 128; }
+// bytes of K per row in a stage: 64 for the wide tiles with all slices in a
+// stage, else 128
+template <int BNT, int SL = 1> __host__ __device__ constexpr int row_bytes() { return SL == 3 && BNT >= 128 ? 64 : 128; }
 template <int BNT, int SL = 1> __host__ __device__ constexpr int stage_bytes() {
-    return SL * (A_STAGE + b_stage<BNT>());
+    return SL * (BM + BNT) * row_bytes<BNT, SL>();
 }
 template <int BNT, int ST, int SL = 1> constexpr size_t smem_bytes() {
     return (size_t)ST * stage_bytes<BNT, SL>() + 1024 + 256;
@@ -195,21 +200,23 @@ __device__ __forceinline__ long unit_begin(int g, long W, int G) { return (long)
 // the tensor memory holds two, so the epilogue of one piece overlaps the
 // main loop of the next.
 template <int KIND, int BNT, int ST, int NACC, int SL = 1>
-__global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
+__global__ void __launch_bounds__(192, 1)
     k_gemm_tc(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
               const __grid_constant__ CUtensorMap mapC, int use_map_c, float* __restrict__ C, long ldc, int cx0,
               int cy0, int M, int N, int a_row0, int b_row0, int k0, int lower, uint32_t idesc, float scale, int nseg,
               uint32_t segs, uint32_t accsel, int tiles_n, int nk, long W, int G, float* __restrict__ Cpart,
               DevStatus* st) {
-    constexpr int BK = KindTraits<KIND>::BK;
-    constexpr int B_STAGE = b_stage<BNT>();      // one slice of a B tile
+    constexpr bool PROMOTE = SL == 3 && BNT <= 64;  // the narrow tiles
+    constexpr int ROWB = row_bytes<BNT, SL>();
+    constexpr int BK = KindTraits<KIND>::BK * ROWB / 128;
+    constexpr int A_STAGE = BM * ROWB, B_STAGE = BNT * ROWB;  // one slice of an A and a B tile
     constexpr int STAGES = ST;
     constexpr int STAGE_BYTES = stage_bytes<BNT, SL>();
     constexpr int A_ST = SL * A_STAGE, B_ST = SL * B_STAGE;  // a stage's A and B parts
     // accumulator buffers: two per tile with one accumulator (the epilogue of
-    // one piece overlaps the next); narrow tiles (SL = 3) promote every K
-    // tile's sums to float32 registers, alternating two buffers
-    constexpr int NBUF = (SL == 3 || NACC == 1) ? 2 : 1;
+    // one piece overlaps the next); narrow tiles promote every K tile's sums to
+    // float32 registers, alternating two buffers
+    constexpr int NBUF = (PROMOTE || NACC == 1) ? 2 : 1;
     constexpr uint32_t ACC_COLS = BNT * NACC;  // one tile's accumulator(s)
     constexpr uint32_t TMEM_COLS = ACC_COLS * NBUF;
     constexpr int MMA_PER_STAGE = BK / KindTraits<KIND>::KMMA;  // 32 bytes of K each
@@ -324,7 +331,34 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
                     }
                     tc::fence_after_sync();
                 }
-                if constexpr (SL == 3) {
+                if constexpr (SL == 3 && !PROMOTE) {
+                    for (int kin = kb; kin < ke; ++kin, ++kt) {
+                        const int s = kt % STAGES;
+                        const uint32_t ph = (kt / STAGES) & 1u;
+                        if (!tc::mbar_wait(&full[s], ph, abort_flag, WAIT_NS)) {
+                            ok = false;
+                            break;
+                        }
+                        tc::fence_after_sync();
+                        for (int q = 0; q < nseg; ++q) {
+                            const int za = (segs >> (4 * q)) & 3, zb = (segs >> (4 * q + 2)) & 3;
+                            const int a = (accsel >> q) & 1;
+                            const uint64_t ad = tc::sdesc_kmajor_sw64(tc::smem_u32(sA + s * A_ST + za * A_STAGE));
+                            const uint64_t bd = tc::sdesc_kmajor_sw64(tc::smem_u32(sB + s * B_ST + zb * B_STAGE));
+                            const uint32_t d = tmem + (uint32_t)(buf * ACC_COLS + a * BNT);
+                            const bool fresh = kin == kb && q == first[a];
+#pragma unroll
+                            for (int k = 0; k < MMA_PER_STAGE; ++k)
+                                tc::mma<KIND>(d, ad + 2 * k, bd + 2 * k, idesc, (fresh && k == 0) ? 0u : 1u);
+                        }
+                        tc::mma_commit(&empty[s]);
+                    }
+                    if (!ok) break;
+                    tc::mma_commit(&accfull[buf]);
+                    ++p;
+                    continue;
+                }
+                if constexpr (PROMOTE) {
                     // each K tile into a fresh accumulator pair (buffer pk & 1),
                     // which the epilogue adds to its float32 registers
                     for (int kin = kb; kin < ke; ++kin, ++kt, ++pk) {
@@ -391,12 +425,12 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
         // narrow tiles: the piece's sums, promoted K tile by K tile into
         // float32 registers (round to nearest) -- the tensor cores' own
         // float32 accumulation rounds toward zero, a bias that grows with K
-        constexpr int NR = SL == 3 ? BNT : 1;
+        constexpr int NR = PROMOTE ? BNT : 1;
         float S0[NR], S1[NR];
         SPD_FOR_PIECES {
             const int buf = p % NBUF;
             uint32_t tacc = 0;
-            if constexpr (SL == 3) {
+            if constexpr (PROMOTE) {
 #pragma unroll
                 for (int j = 0; j < NR; ++j) S0[j] = S1[j] = 0.f;
                 for (int kin = kb; kin < ke; ++kin, ++pk) {
@@ -430,7 +464,7 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
             }
             // 32 columns (chunk ch) of this thread's row of the piece's sum
             auto get = [&](int ch, float* v) {
-                if constexpr (SL == 3) {
+                if constexpr (PROMOTE) {
 #pragma unroll
                     for (int j = 0; j < 32; ++j) v[j] = S0[ch * 32 + j] + S1[ch * 32 + j];  // small + s0*t0
                 } else {
@@ -476,7 +510,7 @@ __global__ void __launch_bounds__(192, (ST == 3 && SL == 1) ? 2 : 1)
                 }
             }
             ok = __all_sync(0xffffffffu, ok);
-            if constexpr (SL != 3) {
+            if constexpr (!PROMOTE) {
                 tc::fence_before_sync();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(&accempty[buf]);
@@ -509,11 +543,11 @@ int elem_bytes(int kind) { return kind == 1 ? 4 : kind == 4 ? 1 : 2; }
 int slices_of(int kind) { return kind == 5 ? 3 : 1; }
 
 // 3-D map over `planes` row-major (rows x cols, ld elements) operand planes
-// (plane stride rows*ld) with a box of (128 bytes of K) x box_rows x box_z
-// (box_z = 1: one slice; 3: every slice of a float32 operand), 128-byte
+// (plane stride rows*ld) with a box of kbytes of K x box_rows x box_z (box_z
+// = 1: one slice; 3: every slice of a float32 operand), kbytes (128 or 64)
 // swizzle, zero fill outside.
 bool make_map(CUtensorMap* map, const void* base, int kind, long rows, long cols, long ld, int box_rows,
-              int box_z = 1) {
+              int box_z = 1, int kbytes = 128) {
     auto enc = get_encode();
     if (!enc) return false;
     CUtensorMapDataType dt = kind == 1 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32
@@ -523,11 +557,11 @@ bool make_map(CUtensorMap* map, const void* base, int kind, long rows, long cols
     const int es = elem_bytes(kind);
     cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)slices_of(kind)};
     cuuint64_t strides[2] = {(cuuint64_t)(ld * es), (cuuint64_t)(rows * ld * es)};
-    cuuint32_t box[3] = {(cuuint32_t)(128 / es), (cuuint32_t)box_rows, (cuuint32_t)box_z};
+    cuuint32_t box[3] = {(cuuint32_t)(kbytes / es), (cuuint32_t)box_rows, (cuuint32_t)box_z};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(map, dt, 3, const_cast<void*>(base), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                     CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-                     CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                     kbytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
+                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS;
 }
 
@@ -568,11 +602,11 @@ void set_attrs() {
         set_smem<0, 256, 4, 1>();
         set_smem<1, 256, 4, 1>();
         set_smem<2, 256, 4, 1>();
-        set_smem<0, 256, 4, 2>();
+        set_smem<0, 256, 3, 2, 3>();
         set_smem<0, 128, 4, 1>();
         set_smem<1, 128, 4, 1>();
         set_smem<2, 128, 4, 1>();
-        set_smem<0, 128, 3, 2>();
+        set_smem<0, 128, 4, 2, 3>();
         set_smem<0, 32, 3, 2, 3>();
         set_smem<0, 64, 3, 2, 3>();
         return true;
@@ -657,8 +691,10 @@ spd_status tc_gemm_create_maps(TcGemm** out, const void* Ah, long a_rows, long a
     if (kind < 1 || kind > 5) return SPD_ERR_UNSUPPORTED;
     TcGemm* g = new TcGemm();
     memset(g, 0, sizeof(*g));
-    if (!make_map(&g->mapA, Ah, kind, a_rows, cols, a_ld, BM) || !make_map(&g->mapB, Bh, kind, b_rows, cols, b_ld, BN) ||
-        !make_map(&g->mapB128, Bh, kind, b_rows, cols, b_ld, 128)) {
+    const int z = kind == 5 ? 3 : 1, kb = kind == 5 ? 64 : 128;
+    if (!make_map(&g->mapA, Ah, kind, a_rows, cols, a_ld, BM, z, kb) ||
+        !make_map(&g->mapB, Bh, kind, b_rows, cols, b_ld, BN, z, kb) ||
+        !make_map(&g->mapB128, Bh, kind, b_rows, cols, b_ld, 128, z, kb)) {
         delete g;
         return SPD_ERR_UNSUPPORTED;
     }
@@ -734,9 +770,9 @@ void launch_kind(TcGemm* g, cudaStream_t s, int G, int cx0, int cy0, int M, int 
     } else {
         switch (g->kind) {
             case 1: SPD_GEMM_LAUNCH((k_gemm_tc<1, BNT, 4, 1>), (smem_bytes<BNT, 4>())); break;
-            case 5: {  // float32 as bf16 slices: two accumulators; two CTAs per SM on 128-wide tiles
-                constexpr int ST = BNT == 128 ? 3 : 4;
-                SPD_GEMM_LAUNCH((k_gemm_tc<0, BNT, ST, 2>), (smem_bytes<BNT, ST>()));
+            case 5: {  // float32 as bf16 slices: two accumulators
+                constexpr int ST = BNT == 128 ? 4 : 3;
+                SPD_GEMM_LAUNCH((k_gemm_tc<0, BNT, ST, 2, 3>), (smem_bytes<BNT, ST, 3>()));
                 break;
             }
             case 4: SPD_GEMM_LAUNCH((k_gemm_tc<2, BNT, 4, 1>), (smem_bytes<BNT, 4>())); break;
@@ -750,7 +786,7 @@ void launch_kind(TcGemm* g, cudaStream_t s, int G, int cx0, int cy0, int M, int 
 
 spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, int N, int K, int a_row0, int b_row0,
                           int k0, int lower, DevStatus* st, int splits, const TcSplit* sb, bool pdl) {
-    const int bk = g->kind == 1 ? 32 : g->kind == 4 ? 128 : 64;
+    const int bk = (g->kind == 1 || (g->kind == 5 && !g->narrow)) ? 32 : g->kind == 4 ? 128 : 64;
     if (M <= 0 || N <= 0 || K <= 0) return SPD_OK;
     if (K % bk != 0 || (k0 * elem_bytes(g->kind)) % 16 != 0 || cx0 % 4 != 0) return SPD_ERR_ARG;
     const float scale = g->kind == 4 ? 1.0f / (tc_fp8_scale() * tc_fp8_scale()) : 1.0f;
@@ -773,16 +809,16 @@ spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, in
     // Data-parallel (one CTA per tile) or stream-K over `slots` CTAs, by an
     // estimate of the launch's length: waves x K tiles per CTA x the time of
     // one K tile, plus ~10 us of fix-up kernel for stream-K.  splits < 0
-    // allows stream-K on -splits SMs (two CTAs per SM for the 128-wide
-    // float32 tiles); splits = 1 keeps one CTA per tile.
+    // allows stream-K on -splits SMs; splits = 1 keeps one CTA per tile.
     int G = T;
     if ((splits < 0 || splits == 0) && sb && sb->part && !(lower && tiles_n > 1)) {
         const int sms = splits < 0 ? -splits : g->sms;
-        const int slots = (bnt == 128 && g->kind == 5 ? 2 : 1) * sms;
+        const int slots = sms;
         int Gs = (int)std::min<long>(slots, W);
-        // us per K tile (all segments); a narrow tile streams 48 KB of A
-        // slices per K tile at about an SM's share of HBM bandwidth
-        const double tk = g->narrow ? 1.0 : nseg * (bnt == 256 ? 0.40 : 0.25);
+        // us per K tile (all segments), measured inside the factorisation; a narrow
+        // tile streams 48 KB of A slices per K tile at about an SM's share of HBM
+        // bandwidth
+        const double tk = g->narrow ? 1.0 : g->kind == 5 ? (bnt == 256 ? 1.0 : 0.6) : (bnt == 256 ? 0.40 : 0.25);
         const double dp = (double)((T + slots - 1) / slots) * nk * tk;
         // stream-K over Gc CTAs: the longest range, plus the fix-up: a launch
         // (~4 us) and its partial slots read at ~3 TB/s

@@ -145,6 +145,18 @@ __device__ __forceinline__ uint64_t sdesc_kmajor_sw128(uint32_t saddr) {
     return d;
 }
 
+// The same for the 64-byte swizzled layout (8 rows x 64 bytes per atom, atoms
+// stacked every 512 bytes; layout type 4).
+__device__ __forceinline__ uint64_t sdesc_kmajor_sw64(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)1 << 16;
+    d |= (uint64_t)(512u >> 4) << 32;
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)4 << 61;
+    return d;
+}
+
 // Instruction descriptor (kind::f16 / kind::tf32 / kind::f8f6f4), dense,
 // float32 accumulator, both operands K-major: D format in [4,6), A and B
 // formats in [7,10) and [10,13), N >> 3 in [17,23), M >> 4 in [24,29).
