@@ -6,6 +6,7 @@
 // consumer CTA sums them in the same order), so runs are reproducible.
 #pragma once
 #include "common.cuh"
+#include "k_convert.cuh"
 
 #define MV_ROWS_PER_WARP 4
 #define MV_ROWS (8 * MV_ROWS_PER_WARP)
@@ -22,12 +23,15 @@ __device__ __forceinline__ float4 ld4(const __nv_bfloat16* p) {
 
 // Q[:, c0:c0+mc] = A~ Pf (float32 products and sums), A~ row-major n x ldt
 // (ldt a multiple of 4, padding columns zero), Pf float32 n x m (ld n).
-// One warp per row group; lanes stride the row 4 elements at a time.
+// One warp per row group; lanes stride the row 4 elements at a time.  With part
+// the block also writes its rows' share of p^T q (P float64): part[(x m + c) 2].
 template <typename T, int MC>
 static __global__ void __launch_bounds__(256) k_matvec_lp(const T* __restrict__ At, long ldt, int n,
                                                    const float* __restrict__ Pf, int c0, int mc,
-                                                   double* __restrict__ Q, const int* __restrict__ done) {
+                                                   double* __restrict__ Q, const double* __restrict__ P, int m,
+                                                   double* __restrict__ part) {
     __shared__ __align__(16) float ps[MC][MV_JCH];
+    __shared__ double red[8][MC];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int rbase = blockIdx.x * MV_ROWS + warp * MV_ROWS_PER_WARP;
     float acc[MV_ROWS_PER_WARP][MC];
@@ -59,14 +63,31 @@ static __global__ void __launch_bounds__(256) k_matvec_lp(const T* __restrict__ 
             }
         }
     }
+    double pq[MC];
+#pragma unroll
+    for (int c = 0; c < MC; ++c) pq[c] = 0.0;
 #pragma unroll
     for (int r = 0; r < MV_ROWS_PER_WARP; ++r) {
         const int row = rbase + r;
 #pragma unroll
         for (int c = 0; c < MC; ++c) {
             float v = warp_sum(acc[r][c]);
-            if (lane == 0 && row < n && c < mc) Q[(long)(c0 + c) * n + row] = (double)v;
+            if (lane == 0 && row < n && c < mc) {
+                Q[(long)(c0 + c) * n + row] = (double)v;
+                if (part) pq[c] = fma((double)v, P[(long)(c0 + c) * n + row], pq[c]);
+            }
         }
+    }
+    if (!part) return;
+    if (lane == 0) {
+#pragma unroll
+        for (int c = 0; c < MC; ++c) red[warp][c] = pq[c];
+    }
+    __syncthreads();
+    if (tid < mc) {
+        double t = 0.0;
+        for (int w = 0; w < 8; ++w) t += red[w][tid];
+        part[((long)blockIdx.x * m + c0 + tid) * 2] = t;
     }
 }
 
@@ -79,26 +100,17 @@ static __global__ void __launch_bounds__(256) k_matvec_lp(const T* __restrict__ 
 //
 // Slice planes of A~ (plane stride `plane`): row j, column i = the slices of
 // fl32(A(i, j)) (A symmetric), zero in the padding columns n <= i < Kp.
-static __global__ void k_convert_x3(const double* __restrict__ A, long lda, int n, int Kp,
+static __global__ void __launch_bounds__(256) k_convert_x3(const double* __restrict__ A, long lda, int n, int Kp,
                                     __nv_bfloat16* __restrict__ M, long ldo, long plane, DevStatus* st) {
-    const long total = (long)n * Kp;
-    bool bad = false;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const long j = e / Kp, i = e - j * Kp;  // column j of A = row j of the planes: coalesced both ways
-        float v = 0.f;
-        if (i < n) {
-            const double a = A[j * lda + i];
-            if (!isfinite(a)) bad = true;
-            v = (float)a;
-        }
-        __nv_bfloat16 s0, s1, s2;
-        split_bf16x3(v, s0, s1, s2);
-        __nv_bfloat16* q = M + j * ldo + i;
-        q[0] = s0;
-        q[plane] = s1;
-        q[2 * plane] = s2;
-    }
-    if (bad) dev_raise(st, SPD_DEV_NONFINITE);
+    if (for_columns(A, lda, n, Kp, [=](long j, long i, double v) {
+            __nv_bfloat16 s0, s1, s2;
+            split_bf16x3(f64_to_f32(v), s0, s1, s2);
+            __nv_bfloat16* q = M + j * ldo + i;
+            q[0] = s0;
+            q[plane] = s1;
+            q[2 * plane] = s2;
+        }))
+        dev_raise(st, SPD_DEV_NONFINITE);
 }
 
 // Rows c < m of P^T's slice planes: row c, column k = the slices of Pf[c n + k]
@@ -117,12 +129,45 @@ static __global__ void k_p_x3(const float* __restrict__ Pf, int n, int m, __nv_b
     }
 }
 
-// Q[c n + i] = -C[i ldc + c] (float64, column-major) from the narrow GEMM's C
-static __global__ void k_cf_to_q(const float* __restrict__ Cf, long ldc, int n, int m, double* __restrict__ Q) {
-    const long total = (long)n * m;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-        const long c = e / n, i = e - c * n;
-        Q[e] = -(double)Cf[i * ldc + c];
+// Q[c n + i] = -C[i ldc + c] (float64, column-major) from the narrow GEMM's C,
+// which is set back to zero for the next product, and the block's share of p^T q:
+// block (x, y) takes rows [128 x, 128 x + 128) of columns 32 y .. 32 y + 31
+// through a transposed tile (C by rows, Q and P by columns, both coalesced); part
+// holds ceil(n / 128) partials per column.
+constexpr int CFQ_ROWS = 128;
+static __global__ void __launch_bounds__(256) k_cf_to_q_dot(float* __restrict__ Cf, long ldc, int n, int m,
+                                                     const double* __restrict__ P, double* __restrict__ Q,
+                                                     double* __restrict__ part) {
+    __shared__ float tile[32][CFQ_ROWS + 1];
+    const int i0 = blockIdx.x * CFQ_ROWS, c0 = blockIdx.y * 32, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+#pragma unroll
+    for (int u = 0; u < CFQ_ROWS / 32; ++u) {  // a float4 of a row: 8 per row (ldc is a multiple of 32)
+        const int r = (tid >> 3) + 32 * u, q = (tid & 7) * 4;
+        if (i0 + r < n) {
+            float4* cf = reinterpret_cast<float4*>(Cf + (long)(i0 + r) * ldc + c0 + q);
+            const float4 v = *cf;
+            *cf = make_float4(0.f, 0.f, 0.f, 0.f);
+            tile[q][r] = v.x;
+            tile[q + 1][r] = v.y;
+            tile[q + 2][r] = v.z;
+            tile[q + 3][r] = v.w;
+        }
+    }
+    __syncthreads();
+    for (int cc = w; cc < 32 && c0 + cc < m; cc += 8) {
+        const long base = (long)(c0 + cc) * n;
+        double s = 0.0;
+#pragma unroll
+        for (int u = 0; u < CFQ_ROWS / 32; ++u) {
+            const int r = lane + 32 * u;
+            if (i0 + r < n) {
+                const double q = -(double)tile[cc][r];
+                Q[base + i0 + r] = q;
+                s = fma(P[base + i0 + r], q, s);
+            }
+        }
+        s = warp_sum(s);
+        if (lane == 0) part[((long)blockIdx.x * m + c0 + cc) * 2] = s;
     }
 }
 
@@ -200,90 +245,196 @@ struct CgCol {
     int pad;
 };
 
-// alpha_c = rho_c / (p^T q)_c (every CTA computes it identically from the
-// partials); e += alpha p; r -= alpha q; with Jacobi z = dinv .* r.
+// The vector work of a step is launched per (row chunk, column): the column's
+// scalars (a float64 division and a square root, dozens of instructions at the
+// float64 rate) are formed once per block.  With every block forming all m
+// columns' scalars, they took 73 us of a step at n = 16384, m = 32 (now 10); the
+whole solve went from 100.6 to 77.6 ms with the other fusions of the step.
+
+// alpha_c = rho_c / (p^T q)_c (every block of a column computes it identically
+// from the partials); e += alpha p; r -= alpha q; with Jacobi z = dinv .* r; with
+// part2 also the chunk's partials of r^T z and r^T r (z = r without dinv), as
+// k_dot2 forms them.  Also clears the count of active columns that the p-update
+// forms anew.
 static __global__ void __launch_bounds__(256) k_cg_update(const double* __restrict__ part, int G, int n, int m,
-                                                   CgCol* __restrict__ cols, int parity,
+                                                   CgCol* __restrict__ cols, int parity, int* __restrict__ active,
                                                    double* __restrict__ E, double* __restrict__ Rr,
                                                    const double* __restrict__ P, const double* __restrict__ Qv,
-                                                   const double* __restrict__ dinv, double* __restrict__ Z) {
-    __shared__ double s_alpha[64];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int cb = 0; cb < m; cb += 64) {
-        const int cn = min(64, m - cb);
-        __syncthreads();
-        for (int c = warp; c < cn; c += blockDim.x >> 5) {  // one warp per column
-            const double pq = warp_sum_parts(part, G, m, cb + c, 0, lane);
-            if (lane == 0) {
-                const CgCol& st = cols[cb + c];
-                s_alpha[c] = st.done ? 0.0 : st.rho[parity] / pq;
-            }
+                                                   const double* __restrict__ dinv, double* __restrict__ Z,
+                                                   double* __restrict__ part2) {
+    __shared__ double s_alpha;
+    __shared__ double red[2][8];
+    const int c = blockIdx.y, lane = threadIdx.x & 31;
+    if (blockIdx.x == 0 && c == 0 && threadIdx.x == 0) *active = 0;
+    if (threadIdx.x < 32) {
+        const double pq = warp_sum_parts(part, G, m, c, 0, lane);
+        if (lane == 0) s_alpha = cols[c].done ? 0.0 : cols[c].rho[parity] / pq;
+    }
+    __syncthreads();
+    const double a = s_alpha;
+    const int rows_per = (n + gridDim.x - 1) / gridDim.x;
+    const int i0 = blockIdx.x * rows_per, i1 = min(n, i0 + rows_per);
+    double s1 = 0.0, s2 = 0.0;
+    for (int i = i0 + threadIdx.x; i < i1; i += 256) {
+        const long k = (long)c * n + i;
+        double r = Rr[k];
+        if (a != 0.0) {
+            E[k] = fma(a, P[k], E[k]);
+            r = fma(-a, Qv[k], r);
+            Rr[k] = r;
         }
-        __syncthreads();
-        long total = (long)n * cn;
-        for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-            int cl = (int)(e / n), i = (int)(e % n);
-            int c = cb + cl;
-            double a = s_alpha[cl];
-            long k = (long)c * n + i;
-            if (a != 0.0) {
-                E[k] = fma(a, P[k], E[k]);
-                Rr[k] = fma(-a, Qv[k], Rr[k]);
-            }
-            if (dinv) Z[k] = dinv[i] * Rr[k];
+        double z = r;
+        if (dinv) {
+            z = dinv[i] * r;
+            Z[k] = z;
         }
-        if (blockIdx.x == 0 && threadIdx.x < cn) cols[cb + threadIdx.x].alpha = s_alpha[threadIdx.x];
+        s1 += r * z;
+        s2 += r * r;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) cols[c].alpha = a;
+    if (!part2) return;
+    s1 = warp_sum(s1);
+    s2 = warp_sum(s2);
+    if (lane == 0) {
+        red[0][threadIdx.x >> 5] = s1;
+        red[1][threadIdx.x >> 5] = s2;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double t1 = 0.0, t2 = 0.0;
+        for (int k = 0; k < 8; ++k) {
+            t1 += red[0][k];
+            t2 += red[1][k];
+        }
+        part2[((long)blockIdx.x * m + c) * 2 + 0] = t1;
+        part2[((long)blockIdx.x * m + c) * 2 + 1] = t2;
     }
 }
 
-// rho'_c = (r^T z)_c, rr_c = (r^T r)_c from partials; beta = rho'/rho;
-// p = z + beta p, pf = fl32(p); CTA 0 records rho' and the stop test.
+// Column c's scalars of the p-update, by one warp (lane 0's results): rho' = r^T
+// z and r^T r from the partials, beta = rho' / rho, the stop test; block 0 of the
+// column records them.
+__device__ __forceinline__ void cg_beta(const double* part, int G, int m, int c, CgCol* cols, int parity, int* active,
+                                        bool record, int lane, double& beta, int& stop_out) {
+    const double rz = warp_sum_parts(part, G, m, c, 0, lane);
+    const double rr = warp_sum_parts(part, G, m, c, 1, lane);
+    if (lane != 0) return;
+    CgCol st = cols[c];
+    const bool was_done = st.done, stop = was_done || (sqrt(rr) <= st.stop);
+    beta = stop ? 0.0 : rz / st.rho[parity];
+    stop_out = stop;
+    if (record) {
+        if (!was_done) {
+            st.iters += 1;
+            st.total += 1;
+            st.rho[parity ^ 1] = rz;
+            st.rr = rr;
+        }
+        // the column's other blocks read done before or after this write, with the
+        // same outcome; rho[parity] keeps its value
+        st.done = stop;
+        cols[c] = st;
+        if (!stop) atomicAdd(active, 1);
+    }
+}
+
+// p = z + beta p, pf = fl32(p) for a row chunk of column c; with Pm (the tensor-
+// core product) pf's three bf16 slices instead.
 static __global__ void __launch_bounds__(256) k_cg_pupdate(const double* __restrict__ part, int G, int n, int m,
                                                     CgCol* __restrict__ cols, int parity, int* __restrict__ active,
                                                     double* __restrict__ P, float* __restrict__ Pf,
-                                                    const double* __restrict__ Z) {
-    __shared__ double s_beta[64];
-    __shared__ int s_done[64];
-    __shared__ int s_active;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_active = 0;
-    for (int cb = 0; cb < m; cb += 64) {
-        const int cn = min(64, m - cb);
-        __syncthreads();
-        for (int c = warp; c < cn; c += blockDim.x >> 5) {  // one warp per column
-            const double rz = warp_sum_parts(part, G, m, cb + c, 0, lane);
-            const double rr = warp_sum_parts(part, G, m, cb + c, 1, lane);
-            if (lane != 0) continue;
-            CgCol st = cols[cb + c];
-            bool was_done = st.done;
-            bool stop = was_done || (sqrt(rr) <= st.stop);
-            s_beta[c] = stop ? 0.0 : rz / st.rho[parity];
-            s_done[c] = stop;
-            if (blockIdx.x == 0) {
-                if (!was_done) {
-                    st.iters += 1;
-                    st.total += 1;
-                    st.rho[parity ^ 1] = rz;
-                    st.rr = rr;
-                }
-                st.done = stop;
-                cols[cb + c] = st;
-                if (!stop) atomicAdd(&s_active, 1);
-            }
-        }
-        __syncthreads();
-        long total = (long)n * cn;
-        for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total; e += (long)gridDim.x * blockDim.x) {
-            int cl = (int)(e / n), i = (int)(e % n);
-            if (s_done[cl]) continue;
-            long k = (long)(cb + cl) * n + i;
-            double p = fma(s_beta[cl], P[k], Z[k]);
-            P[k] = p;
+                                                    const double* __restrict__ Z, __nv_bfloat16* __restrict__ Pm,
+                                                    long ldo, long plane) {
+    __shared__ double s_beta;
+    __shared__ int s_stop;
+    const int c = blockIdx.y;
+    if (threadIdx.x < 32) cg_beta(part, G, m, c, cols, parity, active, blockIdx.x == 0, threadIdx.x, s_beta, s_stop);
+    __syncthreads();
+    if (s_stop) return;
+    const double beta = s_beta;
+    const int rows_per = (n + gridDim.x - 1) / gridDim.x;
+    const int i0 = blockIdx.x * rows_per, i1 = min(n, i0 + rows_per);
+    for (int i = i0 + threadIdx.x; i < i1; i += 256) {
+        const long k = (long)c * n + i;
+        const double p = fma(beta, P[k], Z[k]);
+        P[k] = p;
+        if (Pm) {
+            __nv_bfloat16* q = Pm + c * ldo + i;
+            split_bf16x3((float)p, q[0], q[plane], q[2 * plane]);
+        } else {
             Pf[k] = (float)p;
         }
     }
+}
+
+// The p-update of one step and the banded product of the next in one launch
+// (block (x, c): rows [128 x, 128 x + 128) of column c): p = z + beta p for the
+// rows and the band's halo on both sides, formed again from z and the old p by
+// every block that needs them (Pold is read, Pnew written: they alternate by
+// step), q = A~ p, and the chunk's share of p^T q.  first: p = Pold as it is (the
+// first product of an inner loop).  Two threads share a row, taking every other
+// diagonal.  A step is this and k_cg_update: with five launches it took 31 us at
+// n = 16384, half-width 16, nearly all of them launches and their latencies.
+constexpr int CGB_ROWS = 128;
+constexpr int CGB_MAXBAND = 256;  // past it the halo is more work than the launches cost
+static __global__ void __launch_bounds__(256) k_cg_band_step(const double* __restrict__ part2, int G2, int n, int m,
+                                                      CgCol* __restrict__ cols, int parity, int* __restrict__ active,
+                                                      const double* __restrict__ Pold, double* __restrict__ Pnew,
+                                                      const double* __restrict__ Z, const float* __restrict__ Ab,
+                                                      int band, double* __restrict__ Q, double* __restrict__ part,
+                                                      int first) {
+    __shared__ float pf[CGB_ROWS + 2 * CGB_MAXBAND];
+    __shared__ double pd[CGB_ROWS];
+    __shared__ double red[8];
+    __shared__ double s_beta;
+    __shared__ int s_stop;
+    const int c = blockIdx.y, tid = threadIdx.x, i0 = blockIdx.x * CGB_ROWS;
+    if (first) {
+        if (tid == 0) s_stop = cols[c].done;
+    } else if (tid < 32) {
+        cg_beta(part2, G2, m, c, cols, parity, active, blockIdx.x == 0, tid, s_beta, s_stop);
+    }
     __syncthreads();
-    if (blockIdx.x == 0 && threadIdx.x == 0) *active = s_active;
+    if (s_stop) return;  // its alpha is 0 from here on
+    const double beta = s_beta;
+    for (int k = tid; k < CGB_ROWS + 2 * band; k += 256) {
+        const int i = i0 - band + k;
+        double p = 0.0;
+        if (i >= 0 && i < n) {
+            const long e = (long)c * n + i;
+            p = first ? Pold[e] : fma(beta, Pold[e], Z[e]);
+            if (k >= band && k < band + CGB_ROWS) {
+                pd[k - band] = p;
+                if (!first) Pnew[e] = p;
+            }
+        }
+        pf[k] = (float)p;
+    }
+    __syncthreads();
+    const int r = tid >> 1, h = tid & 1, i = i0 + r;
+    float acc = 0.f;
+    if (i < n) {
+        const float* ab = Ab + i;
+#pragma unroll 8
+        for (int d = h; d <= 2 * band; d += 2) {  // outside the matrix the band is zero
+            acc = fmaf(__ldg(ab + (long)d * n), pf[r + d], acc);
+        }
+    }
+    acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+    double s = 0.0;
+    if (i < n && h == 0) {
+        const double q = (double)acc;
+        Q[(long)c * n + i] = q;
+        s = pd[r] * q;
+    }
+    s = warp_sum(s);
+    if ((tid & 31) == 0) red[tid >> 5] = s;
+    __syncthreads();
+    if (tid == 0) {
+        double t = 0.0;
+        for (int k = 0; k < 8; ++k) t += red[k];
+        part[((long)blockIdx.x * m + c) * 2] = t;
+    }
 }
 
 // Start of an inner loop: e = 0, r_in = r, z = M r (Jacobi or identity),
@@ -376,9 +527,10 @@ static __global__ void k_jacobi_dinv(const double* __restrict__ A, long lda, int
 // warp w takes rows 32 w .. 32 w + 31, lane k column k, the eight warps'
 // sums added in warp order.
 static __global__ void __launch_bounds__(256) k_cg_update_wb(const double* __restrict__ part, int G2, int n, int m,
-                                                      CgCol* __restrict__ cols, int parity, double* __restrict__ E,
-                                                      double* __restrict__ Rr, const double* __restrict__ P,
-                                                      const double* __restrict__ Qv, const double* __restrict__ sdg,
+                                                      CgCol* __restrict__ cols, int parity, int* __restrict__ active,
+                                                      double* __restrict__ E, double* __restrict__ Rr,
+                                                      const double* __restrict__ P, const double* __restrict__ Qv,
+                                                      const double* __restrict__ sdg,
                                                       const double* __restrict__ dh, const double* __restrict__ Uh,
                                                       double* __restrict__ wpart) {
     static_assert(LOWRANK_RANK == 32, "one lane per column of Uh");
@@ -387,6 +539,7 @@ static __global__ void __launch_bounds__(256) k_cg_update_wb(const double* __res
     __shared__ double red[8][LOWRANK_RANK];
     const int c = blockIdx.y, x = blockIdx.x, i0 = 256 * x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (x == 0 && c == 0 && threadIdx.x == 0) *active = 0;
     if (w == 0) {
         const double pq = warp_sum_parts(part, G2, m, c, 0, lane);
         if (lane == 0) {

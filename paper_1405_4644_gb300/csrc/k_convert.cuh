@@ -67,23 +67,50 @@ static __global__ void k_add_diag(T* __restrict__ W, long ldw, int n, double sig
     if (i < n) W[(long)i * ldw + i] += (T)sigma;
 }
 
+// (float)a, rounded to nearest even, by integer operations where the result is a
+// normal float (a conversion runs at the float64 rate, a small fraction of the
+// float32 one)
+__device__ __forceinline__ float f64_to_f32(double a) {
+    const unsigned long long w = (unsigned long long)__double_as_longlong(a), b = w & 0x7FFFFFFFFFFFFFFFull;
+    const int e = (int)(b >> 52);
+    if (e < 1023 - 126 || e > 1023 + 127) return b == 0ull ? __uint_as_float((uint32_t)(w >> 32)) : (float)a;
+    const uint32_t f = (uint32_t)((b + 0x0FFFFFFFull + ((b >> 29) & 1ull)) >> 29) - 0xC0000000u;
+    return __uint_as_float(f | ((uint32_t)(w >> 32) & 0x80000000u));
+}
+__device__ __forceinline__ bool f64_nonfinite(double a) {
+    return ((unsigned long long)__double_as_longlong(a) & 0x7FF0000000000000ull) == 0x7FF0000000000000ull;
+}
+
+// Walks A by columns, 1024 rows of one column per block and step (grid: row
+// chunks x columns), four loads in flight per thread: f(j, i, a) for i < rows;
+// rows past n get a = 0.
+template <typename Fn>
+__device__ __forceinline__ bool for_columns(const double* __restrict__ A, long lda, int n, int rows, Fn f) {
+    bool bad = false;
+    const int i0 = blockIdx.x * 1024 + threadIdx.x;
+    for (int j = blockIdx.y; j < n; j += gridDim.y) {
+        const double* a = A + (long)j * lda;
+        double v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i0 + 256 * u < n ? __ldg(a + i0 + 256 * u) : 0.0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            bad = bad || f64_nonfinite(v[u]);
+            if (i0 + 256 * u < rows) f((long)j, (long)(i0 + 256 * u), v[u]);
+        }
+    }
+    return bad;
+}
+
 // Full low-precision copy A~ = fl(A) for the CG matrix-vector product:
 // row-major n x lda_out (A is symmetric, so this is also its column-major
-// copy).  T is float or __nv_bfloat16.
+// copy): element (i, j) is written to row j, column i.  T is float or
+// __nv_bfloat16.
 template <typename T>
-static __global__ void k_convert_full(const double* __restrict__ A, long lda, int n,
+static __global__ void __launch_bounds__(256) k_convert_full(const double* __restrict__ A, long lda, int n,
                                T* __restrict__ At, long ldt, DevStatus* st) {
-    long total = (long)n * n;
-    bool bad = false;
-    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < total;
-         e += (long)gridDim.x * blockDim.x) {
-        long j = e / n, i = e - j * n;  // column-major walk: coalesced reads
-        double v = A[j * lda + i];
-        if (!isfinite(v)) bad = true;
-        // symmetric: A(i, j) = A(j, i); write row j, column i of the copy
-        At[j * ldt + i] = (T)(float)v;
-    }
-    if (bad) dev_raise(st, SPD_DEV_NONFINITE);
+    if (for_columns(A, lda, n, n, [=](long j, long i, double v) { At[j * ldt + i] = (T)f64_to_f32(v); }))
+        dev_raise(st, SPD_DEV_NONFINITE);
 }
 
 // Banded low-precision copy in diagonal-major layout:
@@ -100,8 +127,8 @@ static __global__ void k_convert_band(const double* __restrict__ A, long lda, in
         float v = 0.0f;
         if (j >= 0 && j < n) {
             double a = A[(long)j * lda + i];
-            if (!isfinite(a)) bad = true;
-            v = (float)a;
+            if (f64_nonfinite(a)) bad = true;
+            v = f64_to_f32(a);
         }
         Ab[e] = v;
     }

@@ -18,6 +18,18 @@
 #define RESID_ROWS 256
 #define RESID_JT 64
 
+// |a| rounded to float32 (half up) by 32-bit integer operations without a branch:
+// a float64 -> float32 conversion runs at the float64 rate, a small fraction of
+// the float32 one; below 2^-126 counts as 0, above float range (and NaN) as
+// infinity
+__device__ __forceinline__ float f64_absf(double a) {
+    const uint32_t hi = (uint32_t)__double2hiint(a) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(a);
+    uint32_t f = __funnelshift_l(lo, hi, 3) - 0xC0000000u + ((lo >> 28) & 1u);
+    f = hi < 0x38100000u ? 0u : f;           // exponent below 1023 - 126
+    f = hi >= 0x47F00000u ? 0x7F800000u : f;  // 2^128 and up
+    return __uint_as_float(f);
+}
+
 template <int MT>
 static __global__ void __launch_bounds__(RESID_ROWS) k_resid_partial(const double* __restrict__ A, long lda, int n,
                                                               const double* __restrict__ X, long ldx, int c0,
@@ -47,7 +59,7 @@ static __global__ void __launch_bounds__(RESID_ROWS) k_resid_partial(const doubl
         __syncthreads();
         if (i < n) {
             const double* ap = Ai + (long)jb * lda;
-            if (MT == 1 && jn == RESID_JT && !rowabs) {
+            if (MT == 1 && jn == RESID_JT) {
                 // one column: four interleaved accumulators (column jj into
                 // accumulator jj % 4) and sixteen loads in flight per thread,
                 // added in a fixed order below
@@ -55,6 +67,7 @@ static __global__ void __launch_bounds__(RESID_ROWS) k_resid_partial(const doubl
                 for (int jj = 0; jj < RESID_JT; jj += 4) {
                     const double a0 = __ldg(ap + (long)jj * lda), a1 = __ldg(ap + (long)(jj + 1) * lda);
                     const double a2 = __ldg(ap + (long)(jj + 2) * lda), a3 = __ldg(ap + (long)(jj + 3) * lda);
+                    if (rowabs) asum += (f64_absf(a0) + f64_absf(a1)) + (f64_absf(a2) + f64_absf(a3));
                     q0 = fma(a0, xs[jj][0], q0);
                     q1 = fma(a1, xs[jj + 1][0], q1);
                     q2 = fma(a2, xs[jj + 2][0], q2);
@@ -64,14 +77,14 @@ static __global__ void __launch_bounds__(RESID_ROWS) k_resid_partial(const doubl
 #pragma unroll 4
                 for (int jj = 0; jj < RESID_JT; ++jj) {
                     double a = __ldg(ap + (long)jj * lda);
-                    if (rowabs) asum += fabsf((float)a);
+                    if (rowabs) asum += f64_absf(a);
 #pragma unroll
                     for (int c = 0; c < MT; ++c) acc[c] = fma(a, xs[jj][c], acc[c]);
                 }
             } else {
                 for (int jj = 0; jj < jn; ++jj) {
                     double a = __ldg(ap + (long)jj * lda);
-                    if (rowabs) asum += fabsf((float)a);
+                    if (rowabs) asum += f64_absf(a);
 #pragma unroll
                     for (int c = 0; c < MT; ++c) acc[c] = fma(a, xs[jj][c], acc[c]);
                 }
@@ -169,23 +182,34 @@ static __global__ void __launch_bounds__(256) k_colnorms(const double* __restric
     }
 }
 
-// ||A||_inf = max_i sum_s rowabs[s][i]  (single CTA, fixed order)
-static __global__ void __launch_bounds__(1024) k_anorm(const float* __restrict__ rowabs, int S, int n,
+// ||A||_inf = max_i sum_s rowabs[s][i]: one thread per row, block maxima met by an
+// integer atomicMax on the bits (non-negative doubles order like integers, so the
+// result does not depend on the order; *anorm starts at 0).  NaN rows are left
+// out, as by fmax.  One CTA alone took 83 us for 8 x 16384 sums, 300 for 64 x
+// 8191: its loads' latency, row after row.
+static __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ rowabs, int S, int n,
                                                 double* __restrict__ anorm) {
-    __shared__ double red[32];
-    double best = 0.0;
-    for (int i = threadIdx.x; i < n; i += 1024) {
-        double s = 0.0;
-        for (int k = 0; k < S; ++k) s += (double)rowabs[(long)k * n + i];
-        best = fmax(best, s);
+    __shared__ double red[8];
+    const int i = blockIdx.x * 256 + threadIdx.x;
+    double s = 0.0;
+    if (i < n) {
+        int k = 0;
+        for (; k + 8 <= S; k += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = rowabs[(long)(k + u) * n + i];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += (double)v[u];
+        }
+        for (; k < S; ++k) s += (double)rowabs[(long)k * n + i];
     }
-    best = warp_max(best);
+    const double best = warp_max(fmax(0.0, s));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;
     __syncthreads();
     if (threadIdx.x == 0) {
         double b = 0.0;
-        for (int k = 0; k < 32; ++k) b = fmax(b, red[k]);
-        *anorm = b;
+        for (int k = 0; k < 8; ++k) b = fmax(b, red[k]);
+        atomicMax(reinterpret_cast<unsigned long long*>(anorm), (unsigned long long)__double_as_longlong(b));
     }
 }
 

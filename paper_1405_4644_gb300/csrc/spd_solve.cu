@@ -277,7 +277,8 @@ spd_status resid_run(spd_handle* h, const ResidWs& w, int n, int m, const double
             LAUNCH_CHECK(h);
         }
         if (anorm) {
-            ++(h)->launches, k_anorm<<<1, 1024, 0, s>>>(w.tc->rowabs, w.tc->RS, n, anorm);
+            CUDA_TRY(h, cudaMemsetAsync(anorm, 0, sizeof(double), s));
+            ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.tc->rowabs, w.tc->RS, n, anorm);
             LAUNCH_CHECK(h);
         }
         return SPD_OK;
@@ -315,7 +316,8 @@ spd_status resid_run(spd_handle* h, const ResidWs& w, int n, int m, const double
         LAUNCH_CHECK(h);
     }
     if (anorm) {
-        ++(h)->launches, k_anorm<<<1, 1024, 0, s>>>(w.rowabs, S, n, anorm);
+        CUDA_TRY(h, cudaMemsetAsync(anorm, 0, sizeof(double), s));
+            ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.rowabs, S, n, anorm);
         LAUNCH_CHECK(h);
     }
     return SPD_OK;
@@ -692,42 +694,45 @@ struct CgSetup {
     TcSplit sk{nullptr, 0};
 };
 
-// Q = A~ P on the tensor cores (float32 operands as three bf16 slices each)
-spd_status mv_tc(spd_handle* h, const CgSetup& cs, int n, int m, const float* Pf, double* Q) {
+// Q = A~ P on the tensor cores (float32 operands as three bf16 slices each: P's
+// are in cs.Pm, cs.Cf is zero before and after), and the partials of p^T q
+spd_status mv_tc(spd_handle* h, const CgSetup& cs, int n, int m, const double* P, double* Q, double* part) {
     ProfScope ps(h, SPD_PHASE_MATVEC, 2.0 * n * (double)n * m, 6.0 * n * (double)cs.Kp);
     cudaStream_t s = h->stream;
-    const int gv = grid_for((long)n * m, 256, 8 * h->sms);
-    ++h->launches, k_p_x3<<<gv, 256, 0, s>>>(Pf, n, m, cs.Pm, cs.ldo, cs.plane_p);
-    CUDA_TRY(h, cudaMemsetAsync(cs.Cf, 0, sizeof(float) * n * cs.ldc, s));
     ++h->launches;
     const spd_status st = tc_gemm_launch(cs.tg, s, 0, 0, n, m, cs.Kp, 0, 0, 0, 0, h->dst, -h->sms, &cs.sk);
     if (st != SPD_OK) return set_err(h, st, "spd_cg: tensor-core product launch failed");
-    ++h->launches, k_cf_to_q<<<gv, 256, 0, s>>>(cs.Cf, cs.ldc, n, m, Q);
+    ++h->launches, k_cf_to_q_dot<<<dim3(ceil_div(n, CFQ_ROWS), ceil_div(m, 32)), 256, 0, s>>>(cs.Cf, cs.ldc, n, m, P, Q, part);
     return SPD_OK;
 }
 
 template <typename T, int MC>
-void mv_launch(spd_handle* h, const CgSetup& cs, int n, int m, const float* Pf, double* Q) {
+void mv_launch(spd_handle* h, const CgSetup& cs, int n, int m, const float* Pf, double* Q, const double* P, double* part) {
     ProfScope ps(h, SPD_PHASE_MATVEC, 2.0 * n * (double)n * m, (double)sizeof(T) * n * (double)n);
     int grid = ceil_div(n, MV_ROWS);
     for (int c0 = 0; c0 < m; c0 += MC) {
         int mc = std::min(MC, m - c0);
         ++(h)->launches, k_matvec_lp<T, MC><<<grid, 256, 0, h->stream>>>(static_cast<const T*>(cs.At), cs.ldt, n, Pf, c0, mc, Q,
-                                                        nullptr);
+                                                        P, m, part);
     }
 }
 
 template <typename T>
-void mv_dispatch(spd_handle* h, const CgSetup& cs, int n, int m, const float* Pf, double* Q) {
-    if (m == 1) mv_launch<T, 1>(h, cs, n, m, Pf, Q);
-    else if (m <= 4) mv_launch<T, 4>(h, cs, n, m, Pf, Q);
-    else if (m <= 8) mv_launch<T, 8>(h, cs, n, m, Pf, Q);
-    else mv_launch<T, 16>(h, cs, n, m, Pf, Q);
+void mv_dispatch(spd_handle* h, const CgSetup& cs, int n, int m, const float* Pf, double* Q, const double* P, double* part) {
+    if (m == 1) mv_launch<T, 1>(h, cs, n, m, Pf, Q, P, part);
+    else if (m <= 4) mv_launch<T, 4>(h, cs, n, m, Pf, Q, P, part);
+    else if (m <= 8) mv_launch<T, 8>(h, cs, n, m, Pf, Q, P, part);
+    else mv_launch<T, 16>(h, cs, n, m, Pf, Q, P, part);
 }
+
+// Up to this many right-hand sides the CUDA-core product writes the partials of
+// p^T q itself, ceil(n / 32) per column (past it their sums in every block of the
+// update cost more than a launch)
+constexpr int MV_DOT_MAXM = 8;
 
 struct CgWs {
     ResidWs rw;
-    double *R, *colnorms, *anorm, *b2, *target, *E, *Rr, *Z, *P, *Q, *part, *Yz;
+    double *R, *colnorms, *anorm, *b2, *target, *E, *Rr, *Z, *P, *Q, *part, *part2, *Yz;
     float* Pf;
     IrCol* cols;
     IrSummary* sum;
@@ -738,9 +743,9 @@ struct CgWs {
 
 size_t cg_plan(WsPlan& p, spd_handle* h, int n, int m, size_t* o, int* S, int* G2) {
     *S = (int)resid_plan(p, h, n, m, o);
-    // row chunks per column of the dot products: about 2 blocks per SM over
-    // all m columns, at least 256 rows each
-    *G2 = std::max(1, std::min(2 * h->sms, ceil_div(n, 256)) / std::max(m, 1));
+    // row chunks per column of the vector work: about 4 blocks per SM over all m
+    // columns, at least 256 rows each
+    *G2 = std::max(1, std::min(ceil_div(n, 256), 4 * h->sms / std::max(m, 1)));
     size_t nm = (size_t)n * m;
     o[4] = p.add<double>(nm);       // R
     o[5] = p.add<double>(3 * m);    // colnorms
@@ -752,7 +757,8 @@ size_t cg_plan(WsPlan& p, spd_handle* h, int n, int m, size_t* o, int* S, int* G
     o[11] = p.add<double>(nm);      // Z
     o[12] = p.add<double>(nm);      // P
     o[13] = p.add<double>(nm);      // Q
-    o[14] = p.add<double>((size_t)(*G2) * m * 2);  // part
+    // part: p^T q, written by k_dot2, the products (32-row blocks) or the band step
+    o[14] = p.add<double>((size_t)std::max(*G2, m <= MV_DOT_MAXM ? ceil_div(n, MV_ROWS) : ceil_div(n, CGB_ROWS)) * m * 2);
     o[15] = p.add<double>(nm);      // Yz (factor preconditioner scratch)
     o[16] = p.add<float>(nm);       // Pf
     o[17] = p.add<IrCol>(m);
@@ -760,6 +766,7 @@ size_t cg_plan(WsPlan& p, spd_handle* h, int n, int m, size_t* o, int* S, int* G
     o[19] = p.add<CgCol>(m);
     o[20] = p.add<int>(m);          // frozen
     o[21] = p.add<int>(1);          // active
+    o[22] = p.add<double>((size_t)(*G2) * m * 2);  // part2: r^T z, r^T r
     return p.bytes;
 }
 
@@ -784,6 +791,7 @@ CgWs cg_bind(spd_handle* h, int n, const size_t* o, int S, int G2) {
     w.cg = ws_at<CgCol>(h, o[19]);
     w.frozen = ws_at<int>(h, o[20]);
     w.active = ws_at<int>(h, o[21]);
+    w.part2 = ws_at<double>(h, o[22]);
     w.G2 = G2;
     return w;
 }
@@ -870,18 +878,45 @@ spd_status cg_ir_core(spd_handle* h, CgWs& w, int n, int m, const double* A, lon
             if (st != SPD_OK) return st;
             ++(h)->launches, k_copy_p<<<gv, 256, 0, s>>>(n, m, w.Z, w.P, w.Pf);
         }
-        ++(h)->launches, k_dot2<<<dim3(w.G2, m), 256, 0, s>>>(w.Rr, Zr, w.Rr, w.Rr, n, m, w.part);
-        ++(h)->launches, k_cg_init_cols<<<ceil_div(m, 4), 128, 0, s>>>(w.part, w.G2, m, w.cg, w.frozen, o.eta, w.target);
+        ++(h)->launches, k_dot2<<<dim3(w.G2, m), 256, 0, s>>>(w.Rr, Zr, w.Rr, w.Rr, n, m, w.part2);
+        ++(h)->launches, k_cg_init_cols<<<ceil_div(m, 4), 128, 0, s>>>(w.part2, w.G2, m, w.cg, w.frozen, o.eta, w.target);
         LAUNCH_CHECK(h);
+        const dim3 gvec(w.G2, m);
+        // the banded product with no preconditioner or Jacobi: one launch for the
+        // p-update and the next product, whose direction vectors alternate
+        // between P and P2 (Yz is only the factor preconditioner's scratch)
+        const bool band_fused = cs.matvec == MV_BAND && cs.band <= CGB_MAXBAND && !fac && !lowrank;
+        double* const Pb[2] = {w.P, w.Yz};
+        const int Gb = ceil_div(n, CGB_ROWS);
+        auto band_step = [&](int t, int first) {  // p of step t (after its p-update) and q
+            ProfScope ps(h, SPD_PHASE_MATVEC, 2.0 * (2.0 * cs.band + 1.0) * n * m, 4.0 * (2.0 * cs.band + 1.0) * n, s);
+            ++(h)->launches, k_cg_band_step<<<dim3(Gb, m), 256, 0, s>>>(
+                w.part2, w.G2, n, m, w.cg, (t + 1) & 1, w.active, first ? Pb[t & 1] : Pb[(t + 1) & 1], Pb[t & 1], Zr,
+                static_cast<const float*>(cs.At), cs.band, w.Q, w.part, first);
+        };
         // one inner step (products, dots, updates) at iteration t
         auto step = [&](int t) -> spd_status {
             const int par = t & 1;
             spd_status sst = SPD_OK;
+            if (band_fused) {
+                ++(h)->launches, k_cg_update<<<gvec, 256, 0, s>>>(w.part, Gb, n, m, w.cg, par, w.active, w.E, w.Rr, Pb[par],
+                                                                 w.Q, cs.pc == SPD_PC_JACOBI ? cs.dinv : nullptr, w.Z,
+                                                                 w.part2);
+                band_step(t + 1, 0);
+                LAUNCH_CHECK(h);
+                return SPD_OK;
+            }
+            // the product and the partials of p^T q (Gp per column)
+            int Gp = w.G2;
+            const bool mv_dot = m <= MV_DOT_MAXM && (cs.matvec == MV_FP32 || cs.matvec == MV_BF16);
+            double* const pq = mv_dot ? w.part : nullptr;
+            if (mv_dot) Gp = ceil_div(n, MV_ROWS);
             switch (cs.matvec) {
-                case MV_FP32: mv_dispatch<float>(h, cs, n, m, w.Pf, w.Q); break;
-                case MV_BF16: mv_dispatch<__nv_bfloat16>(h, cs, n, m, w.Pf, w.Q); break;
+                case MV_FP32: mv_dispatch<float>(h, cs, n, m, w.Pf, w.Q, w.P, pq); break;
+                case MV_BF16: mv_dispatch<__nv_bfloat16>(h, cs, n, m, w.Pf, w.Q, w.P, pq); break;
                 case MV_TC:
-                    sst = mv_tc(h, cs, n, m, w.Pf, w.Q);
+                    sst = mv_tc(h, cs, n, m, w.P, w.Q, w.part);
+                    Gp = ceil_div(n, CFQ_ROWS);
                     if (sst != SPD_OK) return sst;
                     break;
                 case MV_BAND: {  // (2b + 1) n float32 entries of the band per product
@@ -896,31 +931,39 @@ spd_status cg_ir_core(spd_handle* h, CgWs& w, int n, int m, const double* A, lon
                     if (sst != SPD_OK) return sst;
             }
             LAUNCH_CHECK(h);
-            ++(h)->launches, k_dot2<<<dim3(w.G2, m), 256, 0, s>>>(w.P, w.Q, nullptr, nullptr, n, m, w.part);
+            if (!mv_dot && cs.matvec != MV_TC)
+                ++(h)->launches, k_dot2<<<gvec, 256, 0, s>>>(w.P, w.Q, nullptr, nullptr, n, m, w.part);
+            const double* dots = w.part2;
+            int Gd = w.G2;
             if (lowrank) {
                 // the Woodbury apply fused into the update and the next dots:
                 // as many launches per step as Jacobi-PCG
                 const LowrankView v = lowrank_view(cs.LR, n, m);
-                ++(h)->launches, k_cg_update_wb<<<dim3(v.G, m), 256, 0, s>>>(w.part, w.G2, n, m, w.cg, par, w.E, w.Rr,
+                ++(h)->launches, k_cg_update_wb<<<dim3(v.G, m), 256, 0, s>>>(w.part, Gp, n, m, w.cg, par, w.active, w.E, w.Rr,
                                                                             w.P, w.Q, v.sdg, v.dh, v.Uh, v.wpart);
                 ++(h)->launches, k_wb_apply_dot<<<dim3(v.G, m), 256, 0, s>>>(w.Rr, v.sdg, v.dh, v.Uh, v.Lc, v.wpart, v.G,
                                                                             n, m, w.Z, v.dpart);
-                ++(h)->launches, k_cg_pupdate<<<gv, 256, 0, s>>>(v.dpart, v.G, n, m, w.cg, par, w.active, w.P, w.Pf, Zr);
-                LAUNCH_CHECK(h);
-                return SPD_OK;
+                dots = v.dpart;
+                Gd = v.G;
+            } else {
+                ++(h)->launches, k_cg_update<<<gvec, 256, 0, s>>>(w.part, Gp, n, m, w.cg, par, w.active, w.E, w.Rr, w.P, w.Q,
+                                               cs.pc == SPD_PC_JACOBI ? cs.dinv : nullptr, w.Z, fac ? nullptr : w.part2);
             }
-            ++(h)->launches, k_cg_update<<<gv, 256, 0, s>>>(w.part, w.G2, n, m, w.cg, par, w.E, w.Rr, w.P, w.Q,
-                                           cs.pc == SPD_PC_JACOBI ? cs.dinv : nullptr, w.Z);
             LAUNCH_CHECK(h);
             if (fac) {
                 sst = lp_apply(h, cs.F, n, m, w.Rr, n, w.Yz, w.Z, n, nullptr, 0);
                 if (sst != SPD_OK) return sst;
+                ++(h)->launches, k_dot2<<<gvec, 256, 0, s>>>(w.Rr, Zr, w.Rr, w.Rr, n, m, w.part2);
             }
-            ++(h)->launches, k_dot2<<<dim3(w.G2, m), 256, 0, s>>>(w.Rr, Zr, w.Rr, w.Rr, n, m, w.part);
-            ++(h)->launches, k_cg_pupdate<<<gv, 256, 0, s>>>(w.part, w.G2, n, m, w.cg, par, w.active, w.P, w.Pf, Zr);
+            ++(h)->launches, k_cg_pupdate<<<gvec, 256, 0, s>>>(dots, Gd, n, m, w.cg, par, w.active, w.P, w.Pf, Zr,
+                                                              cs.matvec == MV_TC ? cs.Pm : nullptr, cs.ldo, cs.plane_p);
             LAUNCH_CHECK(h);
             return SPD_OK;
         };
+        if (cs.matvec == MV_TC)
+            ++(h)->launches, k_p_x3<<<gv, 256, 0, s>>>(w.Pf, n, m, cs.Pm, cs.ldo, cs.plane_p);
+        if (band_fused) band_step(0, 1);
+        LAUNCH_CHECK(h);
         for (int t = 0; t < o.maxit_inner;) {
             if (graph_ok && (t & 1) == 0 && t + CG_GRAPH_STEPS <= o.maxit_inner) {
                 if (!cg_graph.exec) {
@@ -1001,7 +1044,7 @@ extern "C" spd_status spd_solve_ir(spd_handle* h, const spd_factor_t* F, int n, 
     if (n == 0 || m == 0) return SPD_OK;
     cudaStream_t s = h->stream;
     WsPlan p;
-    size_t o_[22];
+    size_t o_[23];
     int S, G2;
     cg_plan(p, h, n, m, o_, &S, &G2);
     TcSetup tcs;
@@ -1142,7 +1185,7 @@ extern "C" spd_status spd_solve_ir_async(spd_handle* h, const spd_factor_t* F, i
     const int kind = o.resid == SPD_RESID_TC ? SPD_RESID_TC : SPD_RESID_FP64;  // no hybrid: no host decision
     cudaStream_t s = h->stream;
     WsPlan p;
-    size_t o_[22];
+    size_t o_[23];
     int S, G2;
     cg_plan(p, h, n, m, o_, &S, &G2);
     TcSetup tcs;
@@ -1218,7 +1261,7 @@ extern "C" spd_status spd_cg(spd_handle* h, int n, int m, const double* A, int l
     if (n == 0 || m == 0) return SPD_OK;
     cudaStream_t s = h->stream;
     WsPlan p;
-    size_t o_[22];
+    size_t o_[23];
     int S, G2;
     cg_plan(p, h, n, m, o_, &S, &G2);
     CgSetup cs;
@@ -1264,7 +1307,6 @@ extern "C" spd_status spd_cg(spd_handle* h, int n, int m, const double* A, int l
     CUDA_TRY(h, cudaEventRecord(h->e0, s));
     st = tc_bind_prepare(h, tcs, n, m, A, lda, w.rw);
     if (st != SPD_OK) return st;
-    const int gbig = grid_for((long)n * n, 256, 16 * h->sms);
     struct TgGuard {  // the narrow GEMM's maps live for this call
         TcGemm*& g;
         ~TgGuard() {
@@ -1276,8 +1318,9 @@ extern "C" spd_status spd_cg(spd_handle* h, int n, int m, const double* A, int l
         cs.Pm = ws_at<__nv_bfloat16>(h, o_pm);
         cs.Cf = ws_at<float>(h, o_cf);
         cs.sk.part = ws_at<float>(h, o_sk);
-        ++(h)->launches, k_convert_x3<<<gbig, 256, 0, s>>>(A, lda, n, cs.Kp, Am, cs.ldo, (long)n * cs.ldo, h->dst);
+        ++(h)->launches, k_convert_x3<<<dim3(ceil_div(cs.Kp, 1024), std::min(n, 65535)), 256, 0, s>>>(A, lda, n, cs.Kp, Am, cs.ldo, (long)n * cs.ldo, h->dst);
         CUDA_TRY(h, cudaMemsetAsync(cs.Pm, 0, sizeof(__nv_bfloat16) * 3 * cs.plane_p, s));
+        CUDA_TRY(h, cudaMemsetAsync(cs.Cf, 0, sizeof(float) * n * cs.ldc, s));
         st = tc_gemm_create_narrow(&cs.tg, Am, n, cs.ldo, cs.Pm, cs.plane_p / cs.ldo, cs.ldo, cs.Kp, cs.Cf, n,
                                    cs.ldc, cs.ldc, bnt);
         if (st != SPD_OK) return set_err(h, st, "spd_cg: tensor maps of the product failed");
@@ -1290,13 +1333,13 @@ extern "C" spd_status spd_cg(spd_handle* h, int n, int m, const double* A, int l
     } else if (cs.matvec == MV_FP32) {
         float* At = ws_at<float>(h, o_at);
         CUDA_TRY(h, cudaMemsetAsync(At, 0, sizeof(float) * n * ldt, s));
-        ++(h)->launches, k_convert_full<float><<<gbig, 256, 0, s>>>(A, lda, n, At, ldt, h->dst);
+        ++(h)->launches, k_convert_full<float><<<dim3(ceil_div(n, 1024), std::min(n, 65535)), 256, 0, s>>>(A, lda, n, At, ldt, h->dst);
         cs.At = At;
         cs.ldt = ldt;
     } else if (cs.matvec == MV_BF16) {
         __nv_bfloat16* At = ws_at<__nv_bfloat16>(h, o_at);
         CUDA_TRY(h, cudaMemsetAsync(At, 0, sizeof(__nv_bfloat16) * n * ldt, s));
-        ++(h)->launches, k_convert_full<__nv_bfloat16><<<gbig, 256, 0, s>>>(A, lda, n, At, ldt, h->dst);
+        ++(h)->launches, k_convert_full<__nv_bfloat16><<<dim3(ceil_div(n, 1024), std::min(n, 65535)), 256, 0, s>>>(A, lda, n, At, ldt, h->dst);
         cs.At = At;
         cs.ldt = ldt;
     }
