@@ -249,7 +249,7 @@ struct CgCol {
 // scalars (a float64 division and a square root, dozens of instructions at the
 // float64 rate) are formed once per block.  With every block forming all m
 // columns' scalars, they took 73 us of a step at n = 16384, m = 32 (now 10); the
-whole solve went from 100.6 to 77.6 ms with the other fusions of the step.
+// whole solve went from 100.6 to 77.6 ms with the other fusions of the step.
 
 // alpha_c = rho_c / (p^T q)_c (every block of a column computes it identically
 // from the partials); e += alpha p; r -= alpha q; with Jacobi z = dinv .* r; with
