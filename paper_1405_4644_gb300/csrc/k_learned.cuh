@@ -19,16 +19,31 @@ static __global__ void k_features(const double* __restrict__ A, long lda, int n,
     const int i = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
     if (i >= n) return;
     const double si = sdiag[i];
-    double s1 = 0.0, s2 = 0.0, mx = 0.0;
-    for (int j = lane; j < n; j += 32) {  // row i read as column i (symmetric): coalesced
-        const double v = fabs(A[(long)i * lda + j] * si * sdiag[j]);
-        s1 += v;
-        s2 += v * v;
-        if (j != i) mx = fmax(mx, v);
+    // t_j = |a_ij| s_j; the row's own s_i multiplies the sums.  Three float64
+    // operations per entry (they bound it: 1/64 of the float32 rate); the maximum
+    // compares the bits of the non-negative t_j.  Four loads in flight.
+    double s1 = 0.0, s2 = 0.0;
+    unsigned long long mb = 0ull;
+    for (int j0 = lane; j0 < n; j0 += 128) {  // row i read as column i (symmetric): coalesced
+        double a[4], sd[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const int j = j0 + 32 * u;
+            a[u] = j < n ? A[(long)i * lda + j] : 0.0;
+            sd[u] = j < n ? sdiag[j] : 0.0;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const double t = fabs(a[u]) * sd[u];
+            s1 += t;
+            s2 = fma(t, t, s2);
+            const unsigned long long b = (unsigned long long)__double_as_longlong(t);
+            if (j0 + 32 * u != i && b > mb) mb = b;
+        }
     }
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    mx = warp_max(mx);
+    s1 = warp_sum(s1) * si;
+    s2 = warp_sum(s2) * (si * si);
+    const double mx = warp_max(__longlong_as_double((long long)mb)) * si;
     if (lane == 0) {
         const double x = coords[2 * i], y = coords[2 * i + 1];
         const double pi = 3.14159265358979323846;
@@ -55,17 +70,23 @@ static __global__ void k_features(const double* __restrict__ A, long lda, int n,
 // ---- K13: dense layers --------------------------------------------------
 // Generic strided SIMT GEMM: C[m][n] = alpha * sum_k A(m,k) B(k,n) + beta C
 // with A(m,k) = A[m*sam + k*sak], B(k,n) = B[k*sbk + n*sbn]; optional bf16
-// rounding of both operands (mixed-precision training).  64x64 tiles.
-static __global__ void __launch_bounds__(256) k_gemm_strided(int M, int N, int K, const float* __restrict__ A,
+// rounding of both operands (mixed-precision training).  64x64 tiles; with
+// gridDim.z > 1 slice z takes kslice of K and writes its product to C + z
+// czs (k_sum_slices adds them up): the weight gradients, whose K is the number
+// of rows, have a handful of tiles and left the chip idle (720 us for 33 x 256 x
+// 4096).
+static __global__ void __launch_bounds__(256) k_gemm_strided(int M, int N, int Ktot, const float* __restrict__ A,
                                                              long sam, long sak, const float* __restrict__ B,
                                                              long sbk, long sbn, float* __restrict__ C, long ldc,
-                                                             float alpha, float beta, int bf16) {
+                                                             float alpha, float beta, int bf16, int kslice, long czs) {
+    const int kbeg = blockIdx.z * kslice, K = min(Ktot, kbeg + kslice);
+    C += blockIdx.z * czs;
     __shared__ float As[16][64 + 1];
     __shared__ float Bs[16][64 + 1];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
     float acc[4][4] = {};
-    for (int k0 = 0; k0 < K; k0 += 16) {
+    for (int k0 = kbeg; k0 < K; k0 += 16) {
         for (int e = tid; e < 16 * 64; e += 256) {
             const int kk = e / 64, mm = e % 64;
             const int gm = m0 + mm, gk = k0 + kk;
@@ -107,6 +128,21 @@ static __global__ void __launch_bounds__(256) k_gemm_strided(int M, int N, int K
         }
 }
 
+// out[e] = sum of Z slices, in order
+static __global__ void k_sum_slices(const float* __restrict__ part, int Z, long count, float* __restrict__ out) {
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < count; e += (long)gridDim.x * blockDim.x) {
+        float s = 0.f;
+        for (int z0 = 0; z0 < Z; z0 += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = z0 + u < Z ? part[(z0 + u) * count + e] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += v[u];
+        }
+        out[e] = s;
+    }
+}
+
 __device__ __forceinline__ float silu(float x) { return x / (1.f + __expf(-x)); }
 __device__ __forceinline__ float silu_grad(float x) {
     const float s = 1.f / (1.f + __expf(-x));
@@ -135,13 +171,16 @@ static __global__ void k_act_back(const float* __restrict__ Z, float* __restrict
         dH[e] *= silu_grad(Z[e]);
 }
 
-// db[c] = sum_r dZ[r][c]  (one thread per column, fixed order)
-static __global__ void k_colsum(const float* __restrict__ dZ, int rows, int N, float* __restrict__ db) {
+// Column sums over row chunks: part[x][c] = sum over rows [rows x, rows (x + 1))
+// of dZ[r][c] (thread = column; k_sum_slices adds the chunks in order)
+static __global__ void k_colsum(const float* __restrict__ dZ, int rows, int N, int chunk, float* __restrict__ part) {
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
+    const int r0 = blockIdx.y * chunk, r1 = min(rows, r0 + chunk);
     float s = 0.f;
-    for (int r = 0; r < rows; ++r) s += dZ[(long)r * N + c];
-    db[c] = s;
+#pragma unroll 8
+    for (int r = r0; r < r1; ++r) s += dZ[(long)r * N + c];
+    part[(long)blockIdx.y * N + c] = s;
 }
 
 // Adam on a flat parameter vector (float32 master weights)
@@ -174,70 +213,70 @@ static __global__ void k_out_to_dU(const float* __restrict__ O, int n, double* _
 // Writes Lc (the core's Cholesky factor, row-major) and, after it, Ci = the
 // core's inverse Lc^{-T} Lc^{-1} (the Woodbury apply multiplies by it).
 // The core's Gram term over row chunks: block x (1024 threads) stages rows
-// [CORE_ROWS x, CORE_ROWS (x + 1)) of Uh and 1/dh in shared memory; thread
+// [CORE_ROWS x, CORE_ROWS (x + 1)) of Uh and Uh ./ dh in shared memory; thread
 // (a, b) writes part[x][a][b] = sum over the chunk's rows, in row order, of
-// Uh_ia Uh_ib (1/dh_i).
-#define CORE_ROWS 128
+// Uh_ia (Uh_ib / dh_i); 32 rows a block keep the float64 units of more SMs busy.
+#define CORE_ROWS 32
 static __global__ void __launch_bounds__(1024) k_core_gram(const double* __restrict__ dh, const double* __restrict__ Uh,
                                                            int n, double* __restrict__ part) {
-    __shared__ double Us[CORE_ROWS][LR_RANK];
-    __shared__ double rd[CORE_ROWS];
+    __shared__ double Us[CORE_ROWS][LR_RANK], Ud[CORE_ROWS][LR_RANK];  // Uh and Uh ./ dh
     const int i0 = blockIdx.x * CORE_ROWS, rows = min(CORE_ROWS, n - i0);
-    for (int e = threadIdx.x; e < CORE_ROWS * LR_RANK; e += 1024) {
-        const int r = e / LR_RANK, k = e % LR_RANK;
-        Us[r][k] = r < rows ? Uh[(long)(i0 + r) * LR_RANK + k] : 0.0;
+    static_assert(CORE_ROWS * LR_RANK == 1024, "one entry per thread");
+    {
+        const int r = threadIdx.x / LR_RANK, k = threadIdx.x % LR_RANK;
+        const double u = r < rows ? Uh[(long)(i0 + r) * LR_RANK + k] : 0.0;
+        Us[r][k] = u;
+        Ud[r][k] = r < rows ? u * (1.0 / dh[i0 + r]) : 0.0;
     }
-    if (threadIdx.x < CORE_ROWS) rd[threadIdx.x] = threadIdx.x < rows ? 1.0 / dh[i0 + threadIdx.x] : 0.0;
     __syncthreads();
     const int a = threadIdx.x / LR_RANK, b = threadIdx.x % LR_RANK;
     double s = 0.0;
 #pragma unroll 8
-    for (int r = 0; r < CORE_ROWS; ++r) s = fma(Us[r][a] * Us[r][b], rd[r], s);
+    for (int r = 0; r < CORE_ROWS; ++r) s = fma(Us[r][a], Ud[r][b], s);
     part[(long)blockIdx.x * LR_RANK * LR_RANK + threadIdx.x] = s;
 }
 
 // Cc = I + the G chunk partials (in chunk order), then its Cholesky factor Lc
-// and the inverse Ci = Lc^{-T} Lc^{-1}.
+// and the inverse Ci = Lc^{-T} Lc^{-1}.  One CTA, thread (a, b) one entry: every
+// step's updates are independent (a serial sum per entry took 121 us).
 static __global__ void __launch_bounds__(1024) k_core_chol(const double* __restrict__ part, int G,
                                                            double* __restrict__ Lc, int* __restrict__ bad) {
     __shared__ double Cs[LR_RANK][LR_RANK + 1];
     __shared__ double Li[LR_RANK][LR_RANK + 1];
+    __shared__ double rd[LR_RANK];
     const int a = threadIdx.x / LR_RANK, b = threadIdx.x % LR_RANK;
     double s = (a == b) ? 1.0 : 0.0;
-    for (int x = 0; x < G; ++x) s += part[(long)x * LR_RANK * LR_RANK + threadIdx.x];
+    for (int x0 = 0; x0 < G; x0 += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = x0 + u < G ? part[(long)(x0 + u) * LR_RANK * LR_RANK + threadIdx.x] : 0.0;
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s += v[u];
+    }
     Cs[a][b] = s;
+    Li[a][b] = (a == b) ? 1.0 : 0.0;
     __syncthreads();
-    if (threadIdx.x < 32) {  // warp 0: Cholesky of Cs in place, lane = row
-        const int r = threadIdx.x;
-        for (int j = 0; j < LR_RANK; ++j) {
-            if (r == j) {
-                double v = Cs[j][j];
-                for (int k = 0; k < j; ++k) v -= Cs[j][k] * Cs[j][k];
-                if (!(v > 0.0)) {
-                    *bad = 1;
-                    v = 1.0;
-                }
-                Cs[j][j] = sqrt(v);
+    for (int j = 0; j < LR_RANK; ++j) {  // right-looking, the lower triangle
+        if (threadIdx.x == 0) {
+            double v = Cs[j][j];
+            if (!(v > 0.0)) {
+                *bad = 1;
+                v = 1.0;
             }
-            __syncwarp();
-            if (r > j) {
-                double v = Cs[r][j];
-                for (int k = 0; k < j; ++k) v -= Cs[r][k] * Cs[j][k];
-                Cs[r][j] = v / Cs[j][j];
-            }
-            __syncwarp();
+            const double l = sqrt(v);
+            Cs[j][j] = l;
+            rd[j] = 1.0 / l;
         }
+        __syncthreads();
+        if (b == j && a > j) Cs[a][j] *= rd[j];
+        __syncthreads();
+        if (b > j && a >= b) Cs[a][b] = fma(-Cs[a][j], Cs[b][j], Cs[a][b]);
+        // column b of Lc^{-1}, the same way: x_j = x_j / L_jj, then x_a -= L_aj x_j
+        if (a > j && b <= j) Li[a][b] = fma(-Cs[a][j], Li[j][b] * rd[j], Li[a][b]);
+        __syncthreads();
     }
-    __syncthreads();
+    Li[a][b] = b <= a ? Li[a][b] * rd[a] : 0.0;
     Lc[a * LR_RANK + b] = (b <= a) ? Cs[a][b] : 0.0;
-    if (threadIdx.x < 32) {  // lane b: column b of Lc^{-1} by forward substitution
-        const int bb = threadIdx.x;
-        for (int r = 0; r < LR_RANK; ++r) {
-            double v = (r == bb) ? 1.0 : 0.0;
-            for (int k = bb; k < r; ++k) v -= Cs[r][k] * Li[k][bb];
-            Li[r][bb] = (r >= bb) ? v / Cs[r][r] : 0.0;
-        }
-    }
     __syncthreads();
     double ci = 0.0;
     for (int k = max(a, b); k < LR_RANK; ++k) ci += Li[k][a] * Li[k][b];

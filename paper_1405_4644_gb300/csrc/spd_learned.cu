@@ -6,6 +6,7 @@
 #include <string>
 #include "engine.cuh"
 #include "k_learned.cuh"
+#include "k_resid.cuh"
 
 struct spd_mlp {
     spd_handle* h = nullptr;
@@ -52,7 +53,27 @@ void gemm(spd_handle* h, int M, int N, int K, const float* A, long sam, long sak
           float* C, long ldc, float alpha, float beta, int bf16) {
     dim3 grid((N + 63) / 64, (M + 63) / 64);
     ++h->launches, k_gemm_strided<<<grid, 256, 0, h->stream>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, alpha, beta,
-                                                               bf16);
+                                                               bf16, K, 0);
+}
+
+// The weight gradients: C (M x N, dense) = A B over K = the rows of the batch, in
+// slices of 128 of K (at most GRAD_SLICES) added in order; part holds the slices.
+constexpr int GRAD_SLICES = 32;
+void gemm_grad(spd_handle* h, int M, int N, int K, const float* A, long sam, long sak, const float* B, long sbk,
+               long sbn, float* C, float* part) {
+    const int ks = std::max(128, (int)round_up(ceil_div(K, GRAD_SLICES), 16)), Z = ceil_div(K, ks);
+    dim3 grid((N + 63) / 64, (M + 63) / 64, Z);
+    const long cnt = (long)M * N;
+    ++h->launches, k_gemm_strided<<<grid, 256, 0, h->stream>>>(M, N, K, A, sam, sak, B, sbk, sbn, part, N, 1.f, 0.f, 0,
+                                                               ks, cnt);
+    ++h->launches, k_sum_slices<<<grid_for(cnt, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, cnt, C);
+}
+
+// out = column sums of dZ (rows x N), in row chunks added in order
+void colsum(spd_handle* h, const float* dZ, int rows, int N, float* out, float* part) {
+    const int chunk = std::max(64, ceil_div(rows, 64)), Z = ceil_div(rows, chunk);
+    ++h->launches, k_colsum<<<dim3((N + 127) / 128, Z), 128, 0, h->stream>>>(dZ, rows, N, chunk, part);
+    ++h->launches, k_sum_slices<<<grid_for(N, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, N, out);
 }
 
 spd_status ensure_acts(spd_mlp* m, int n) {
@@ -88,24 +109,28 @@ void forward(spd_mlp* m, int n, const float* F) {
 }
 
 // backward pass from dO (n x 33) into m->g
-void backward(spd_mlp* m, int n, const float* F) {
+// part: GRAD_SLICES x the largest weight matrix, and 64 x H for the column sums
+size_t backward_part(const spd_mlp* m) {
+    return std::max((size_t)GRAD_SLICES * m->H * std::max({m->H, m->O, m->F}), (size_t)64 * std::max(m->H, m->O));
+}
+void backward(spd_mlp* m, int n, const float* F, float* part) {
     spd_handle* h = m->h;
     const Lay L = layout(m);
     const int H = m->H, O = m->O;
     cudaStream_t s = h->stream;
     // layer 3
-    gemm(h, O, H, n, m->dO, 1, O, m->H2, H, 1, m->g + L.W3, H, 1.f, 0.f, 0);
-    ++h->launches, k_colsum<<<(O + 127) / 128, 128, 0, s>>>(m->dO, n, O, m->g + L.b3);
+    gemm_grad(h, O, H, n, m->dO, 1, O, m->H2, H, 1, m->g + L.W3, part);
+    colsum(h, m->dO, n, O, m->g + L.b3, part);
     gemm(h, n, H, O, m->dO, O, 1, m->p + L.W3, H, 1, m->dH2, H, 1.f, 0.f, 0);
     ++h->launches, k_act_back<<<grid_for((long)n * H, 256, 8 * h->sms), 256, 0, s>>>(m->Z2, m->dH2, (long)n * H);
     // layer 2
-    gemm(h, H, H, n, m->dH2, 1, H, m->H1, H, 1, m->g + L.W2, H, 1.f, 0.f, 0);
-    ++h->launches, k_colsum<<<(H + 127) / 128, 128, 0, s>>>(m->dH2, n, H, m->g + L.b2);
+    gemm_grad(h, H, H, n, m->dH2, 1, H, m->H1, H, 1, m->g + L.W2, part);
+    colsum(h, m->dH2, n, H, m->g + L.b2, part);
     gemm(h, n, H, H, m->dH2, H, 1, m->p + L.W2, H, 1, m->dH, H, 1.f, 0.f, 0);
     ++h->launches, k_act_back<<<grid_for((long)n * H, 256, 8 * h->sms), 256, 0, s>>>(m->Z1, m->dH, (long)n * H);
     // layer 1
-    gemm(h, H, m->F, n, m->dH, 1, H, F, m->F, 1, m->g + L.W1, m->F, 1.f, 0.f, 0);
-    ++h->launches, k_colsum<<<(H + 127) / 128, 128, 0, s>>>(m->dH, n, H, m->g + L.b1);
+    gemm_grad(h, H, m->F, n, m->dH, 1, H, F, m->F, 1, m->g + L.W1, part);
+    colsum(h, m->dH, n, H, m->g + L.b1, part);
 }
 
 __global__ void k_sdiag(const double* __restrict__ A, long lda, int n, double* __restrict__ s) {
@@ -113,50 +138,70 @@ __global__ void k_sdiag(const double* __restrict__ A, long lda, int n, double* _
     if (i < n) s[i] = 1.0 / sqrt(A[(long)i * lda + i]);
 }
 
-// Q = A P in float64 (A column-major symmetric, P n x p with ld n)
-__global__ void __launch_bounds__(256) k_gemv64(const double* __restrict__ A, long lda, int n, const double* __restrict__ P,
-                                                int p, double* __restrict__ Q) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double acc[8];
-    for (int c0 = 0; c0 < p; c0 += 8) {
-        const int pc = min(8, p - c0);
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-        for (int j = 0; j < n; ++j) {
-            const double a = A[(long)j * lda + i];
-#pragma unroll
-            for (int c = 0; c < 8; ++c)
-                if (c < pc) acc[c] = fma(a, P[(long)(c0 + c) * n + j], acc[c]);
-        }
-        for (int c = 0; c < pc; ++c) Q[(long)(c0 + c) * n + i] = acc[c];
+// Q = A P in float64 (A column-major symmetric, P n x p with ld n): the split-K
+// partial sums of the residual (k_resid_partial; bound by the float64 rate), then
+// their sum in order.  A thread per row over all of A kept ceil(n / 256) SMs busy:
+// 3.4 ms at n = 4096, p = 8.
+__global__ void k_sum_parts64(const double* __restrict__ P, int S, long count, double* __restrict__ Q) {
+    for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < count; e += (long)gridDim.x * blockDim.x) {
+        double s = 0.0;
+        for (int k = 0; k < S; ++k) s += P[k * count + e];
+        Q[e] = s;
     }
 }
+int prod64_splits(const spd_handle* h, int n) {
+    return std::max(1, std::min(ceil_div(4 * h->sms, ceil_div(n, RESID_ROWS)), n / (2 * RESID_JT)));
+}
+void prod64(spd_handle* h, const double* A, long lda, int n, const double* P, int p, double* Q, double* part) {
+    const int S = prod64_splits(h, n), jchunk = (int)round_up(ceil_div(n, S), RESID_JT);
+    const dim3 grid(ceil_div(n, RESID_ROWS), S);
+    cudaStream_t s = h->stream;
+    for (int c0 = 0; c0 < p; c0 += 16) {
+        const int pc = std::min(16, p - c0);
+        ++h->launches;
+        if (pc == 1) k_resid_partial<1><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
+        else if (pc <= 4) k_resid_partial<4><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
+        else if (pc <= 8) k_resid_partial<8><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
+        else k_resid_partial<16><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
+    }
+    ++h->launches, k_sum_parts64<<<grid_for((long)n * p, 256, 8 * h->sms), 256, 0, s>>>(part, S, (long)n * p, Q);
+}
 
-// PV[c][k] = sum_i Uh_ik V_ic  (one CTA per column, fixed order)
-__global__ void __launch_bounds__(256) k_proj(const double* __restrict__ Uh, const double* __restrict__ V, int n,
-                                              double* __restrict__ PV) {
+// PV[c][k] = sum_i Uh_ik V_ic: block (x, c) over rows [256 x, 256 x + 256) as
+// k_wb_proj (warp w rows 32 w .., lane k column k), partials added in chunk order
+// by k_proj_sum
+__global__ void __launch_bounds__(256) k_proj(const double* __restrict__ Uh, const double* __restrict__ V, int n, int p,
+                                              double* __restrict__ part) {
+    __shared__ double vs[256];
     __shared__ double red[8][LR_RANK];
-    const int c = blockIdx.x;
-    double acc[LR_RANK];
+    const int c = blockIdx.y, i0 = blockIdx.x * 256, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    vs[threadIdx.x] = i0 + threadIdx.x < n ? V[(long)c * n + i0 + threadIdx.x] : 0.0;
+    __syncthreads();
+    double u[32];
 #pragma unroll
-    for (int k = 0; k < LR_RANK; ++k) acc[k] = 0.0;
-    for (int i = threadIdx.x; i < n; i += 256) {
-        const double v = V[(long)c * n + i];
-#pragma unroll
-        for (int k = 0; k < LR_RANK; ++k) acc[k] = fma(Uh[(long)i * LR_RANK + k], v, acc[k]);
+    for (int r = 0; r < 32; ++r) {
+        const int i = i0 + 32 * w + r;
+        u[r] = i < n ? Uh[(long)i * LR_RANK + lane] : 0.0;
     }
+    double acc = 0.0;
 #pragma unroll
-    for (int k = 0; k < LR_RANK; ++k) {
-        double v = warp_sum(acc[k]);
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][k] = v;
-    }
+    for (int r = 0; r < 32; ++r) acc = fma(u[r], vs[32 * w + r], acc);
+    red[w][lane] = acc;
     __syncthreads();
     if (threadIdx.x < LR_RANK) {
         double s = 0.0;
-        for (int w = 0; w < 8; ++w) s += red[w][threadIdx.x];
-        PV[c * LR_RANK + threadIdx.x] = s;
+#pragma unroll
+        for (int v = 0; v < 8; ++v) s += red[v][threadIdx.x];
+        part[((long)blockIdx.x * p + c) * LR_RANK + threadIdx.x] = s;
     }
+}
+__global__ void k_proj_sum(const double* __restrict__ part, int G, int count, double* __restrict__ PV) {
+    const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e >= count) return;
+    double s = 0.0;
+#pragma unroll 4
+    for (int x = 0; x < G; ++x) s += part[(long)x * count + e];
+    PV[e] = s;
 }
 
 // loss pieces per column: E = Q - Z; returns per-column ||E||^2 and ||Z||^2
@@ -489,13 +534,15 @@ extern "C" spd_status spd_mlp_loss_grad(spd_mlp* m, int n, const double* A, int 
            o_w = pl.add<double>((size_t)wb_chunks(n) * LR_RANK * p),
            o_sums = pl.add<double>(2 * p + 2), o_coef = pl.add<double>(p), o_dh = pl.add<double>(n),
            o_Uh = pl.add<double>((size_t)n * LR_RANK), o_Lc = pl.add<double>(2 * LR_RANK * LR_RANK),
-           o_bad = pl.add<int>(1);
+           o_bad = pl.add<int>(1), o_parts = pl.add<double>((size_t)prod64_splits(h, n) * np),
+           o_bpart = pl.add<float>(backward_part(m));
     if ((st = ws_reserve(h, pl.bytes)) != SPD_OK) return st;
     double *sd = ws_at<double>(h, o_sd), *Y = ws_at<double>(h, o_Y), *Q = ws_at<double>(h, o_Q),
            *E = ws_at<double>(h, o_E), *G = ws_at<double>(h, o_G), *Wv = ws_at<double>(h, o_Wv),
            *Yh = ws_at<double>(h, o_Yh), *Wh = ws_at<double>(h, o_Wh), *PY = ws_at<double>(h, o_PY),
            *PW = ws_at<double>(h, o_PW), *wb = ws_at<double>(h, o_w), *sums = ws_at<double>(h, o_sums),
-           *coef = ws_at<double>(h, o_coef);
+           *coef = ws_at<double>(h, o_coef), *parts = ws_at<double>(h, o_parts);
+    float* bpart = ws_at<float>(h, o_bpart);
     spd_lowrank P;
     P.h = h;
     P.n = n;
@@ -510,9 +557,9 @@ extern "C" spd_status spd_mlp_loss_grad(spd_mlp* m, int n, const double* A, int 
     forward(m, n, F);
     if ((st = build_core(m, &P, n, dbad)) != SPD_OK) return st;
     if ((st = lowrank_apply_internal(h, &P, n, p, Zp, n, Y, n, wb)) != SPD_OK) return st;  // Y = M Z
-    ++h->launches, k_gemv64<<<ceil_div(n, 256), 256, 0, s>>>(A, lda, n, Y, p, Q);          // Q = A Y
+    prod64(h, A, lda, n, Y, p, Q, parts);                                                  // Q = A Y
     ++h->launches, k_probe_err<<<p, 256, 0, s>>>(Q, Zp, n, E, sums);                        // E = A M Z - Z
-    ++h->launches, k_gemv64<<<ceil_div(n, 256), 256, 0, s>>>(A, lda, n, E, p, G);          // G = A E
+    prod64(h, A, lda, n, E, p, G, parts);                                                  // G = A E
     // host: loss and per-column coefficients 2 / (p ||z_c||^2); supervised target norm
     std::vector<double> hs(2 * p + 2);
     double tn2 = 1.0;
@@ -541,10 +588,12 @@ extern "C" spd_status spd_mlp_loss_grad(spd_mlp* m, int n, const double* A, int 
     if ((st = lowrank_apply_internal(h, &P, n, p, G, n, Wv, n, wb)) != SPD_OK) return st;  // W = M G
     ++h->launches, k_unscale<<<gv, 256, 0, s>>>(Y, sd, n, p, Yh);
     ++h->launches, k_unscale<<<gv, 256, 0, s>>>(Wv, sd, n, p, Wh);
-    ++h->launches, k_proj<<<p, 256, 0, s>>>(P.Uh, Yh, n, PY);
-    ++h->launches, k_proj<<<p, 256, 0, s>>>(P.Uh, Wh, n, PW);
-    ++h->launches, k_loss_grad_out<<<grid_for(n, 256, 4 * h->sms), 256, 0, s>>>(Yh, Wh, n, p, P.Uh, PY, PW, m->Ob, m->dO);
-    backward(m, n, F);
+    for (int q = 0; q < 2; ++q) {
+        ++h->launches, k_proj<<<dim3(wb_chunks(n), p), 256, 0, s>>>(P.Uh, q ? Wh : Yh, n, p, wb);
+        ++h->launches, k_proj_sum<<<ceil_div(LR_RANK * p, 128), 128, 0, s>>>(wb, wb_chunks(n), LR_RANK * p, q ? PW : PY);
+    }
+    ++h->launches, k_loss_grad_out<<<grid_for(n, 32, 4 * h->sms), 32, 0, s>>>(Yh, Wh, n, p, P.Uh, PY, PW, m->Ob, m->dO);
+    backward(m, n, F, bpart);
     LAUNCH_CHECK(h);
     int hbad = 0;
     CUDA_TRY(h, cudaMemcpyAsync(&hbad, dbad, sizeof(int), cudaMemcpyDeviceToHost, s));
