@@ -8,9 +8,14 @@
 //
 // Per-CTA scratch in global memory (L2-resident): the scaled working
 // matrix W (column-major lower, ld 512, float32).  Shared memory holds the
-// 32x32 diagonal-block inverses, the current panel, and the vectors.
+// 32x32 diagonal-block inverses (packed lower triangles), the current panel, and
+// the vectors: 112 KB, so that two CTAs of 256 threads share an SM and one's
+// pivots and barriers run beside the other's products.  4096 systems of order 32
+// .. 512: 11.9 ms (20.6 with one CTA per SM, single pivots by shuffles, and a warp
+// per row in the back substitution).
 #pragma once
 #include "common.cuh"
+#include "k_leaf32.cuh"
 
 #define BMAX 512           // largest system order
 #define BLD 512            // leading dimension of the per-CTA working matrix
@@ -47,12 +52,15 @@ struct BatchArgs {
 // The panel's rows transposed: PnT[l * BLDP + i] = L[i][k0 + l] (rounded to the
 // update type), rows contiguous so that four rows are one 16-byte load.
 #define BLDP 516
+#define BTRI 528  // entries of a 32 x 32 lower triangle
+__device__ __forceinline__ constexpr int btri(int r) { return r * (r + 1) / 2; }
 constexpr size_t batch_smem_bytes() {
-    return (size_t)(BMAX / 32) * 32 * 33 * sizeof(float)  // Inv
-           + (size_t)BMAX * 33 * sizeof(float)            // panel (PnT: 32 x BLDP floats fit in it)
-           + (size_t)4 * BMAX * sizeof(double)            // x, r, d, rowabs
-           + (size_t)2 * BMAX * sizeof(float);            // y, z
+    return (size_t)(BMAX / 32) * BTRI * sizeof(float)  // Inv
+           + (size_t)32 * BLDP * sizeof(float)         // panel
+           + (size_t)3 * BMAX * sizeof(double)         // x, r, d
+           + (size_t)BMAX * sizeof(float);             // y
 }
+constexpr size_t batch_pcg_smem_bytes() { return (size_t)6 * BMAX * sizeof(double); }
 
 __device__ __forceinline__ float round_op(float v, int prec) {
     if (prec == 3) return __bfloat162float(__float2bfloat16_rn(v));  // SPD_PREC_BF16
@@ -81,111 +89,226 @@ __device__ double block_sum(double v, double* red) {
     return r;
 }
 
-// y <- (L L^T)^{-1} y in place (float32, shared memory) with the factor in W
-// and the diagonal-block inverses in Inv.
+// y <- (L L^T)^{-1} y in place (float32, shared memory, zero from n to the next
+// multiple of 32) with the factor in W and the diagonal-block inverses in Inv.
+// One thread per row for the updates; the row's 32 entries of L (forward: a
+// strided row, coalesced across threads; backward: 128 contiguous bytes of its
+// column) are in flight while warp 0 applies the block's inverse.
 template <int NT>
 __device__ void batch_lsolve(const float* W, const float* Inv, float* y, int n) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int nb = (n + 31) / 32;
     for (int kb = 0; kb < nb; ++kb) {  // forward
         const int k0 = kb * 32;
+        int i = k0 + 32 + tid;
+        float w[32];
+        if (i < n) {
+#pragma unroll
+            for (int c = 0; c < 32; ++c) w[c] = W[i + (long)(k0 + c) * BLD];
+        }
         if (warp == 0) {
-            const float* I = Inv + kb * 32 * 33;
-            float s = 0.f;
-            for (int l = 0; l <= lane; ++l) s += I[lane * 33 + l] * ((k0 + l < n) ? y[k0 + l] : 0.f);
+            const float* I = Inv + kb * BTRI + btri(lane);
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int l = 0; l < 32; l += 2) {
+                if (l <= lane) s0 = fmaf(I[l], y[k0 + l], s0);
+                if (l + 1 <= lane) s1 = fmaf(I[l + 1], y[k0 + l + 1], s1);
+            }
             __syncwarp();
-            if (k0 + lane < n) y[k0 + lane] = s;
+            if (k0 + lane < n) y[k0 + lane] = s0 + s1;
         }
         __syncthreads();
-        for (int i = k0 + 32 + tid; i < n; i += NT) {
+        while (i < n) {
             float s = 0.f;
-#pragma unroll 8
-            for (int c = 0; c < 32; ++c) s += W[i + (long)(k0 + c) * BLD] * y[k0 + c];
+#pragma unroll
+            for (int c = 0; c < 32; ++c) s = fmaf(w[c], y[k0 + c], s);
             y[i] -= s;
+            i += NT;
+            if (i < n) {
+#pragma unroll
+                for (int c = 0; c < 32; ++c) w[c] = W[i + (long)(k0 + c) * BLD];
+            }
         }
         __syncthreads();
     }
     for (int kb = nb - 1; kb >= 0; --kb) {  // backward
         const int k0 = kb * 32;
+        int i = tid;
+        float w[32];
+        auto load = [&]() {
+            const float4* p = reinterpret_cast<const float4*>(W + (long)i * BLD + k0);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float4 v = p[q];
+                w[4 * q] = v.x;
+                w[4 * q + 1] = v.y;
+                w[4 * q + 2] = v.z;
+                w[4 * q + 3] = v.w;
+            }
+            if (k0 + 32 > n) {  // rows past n hold another system's values
+#pragma unroll
+                for (int c = 0; c < 32; ++c)
+                    if (k0 + c >= n) w[c] = 0.f;
+            }
+        };
+        if (i < k0) load();
         if (warp == 0) {
-            const float* I = Inv + kb * 32 * 33;
-            float s = 0.f;
-            for (int l = lane; l < 32; ++l) s += I[l * 33 + lane] * ((k0 + l < n) ? y[k0 + l] : 0.f);
+            const float* I = Inv + kb * BTRI + lane;
+            float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+            for (int l = 0; l < 32; l += 2) {
+                if (l >= lane) s0 = fmaf(I[btri(l)], y[k0 + l], s0);
+                if (l + 1 >= lane) s1 = fmaf(I[btri(l + 1)], y[k0 + l + 1], s1);
+            }
             __syncwarp();
-            if (k0 + lane < n) y[k0 + lane] = s;
+            if (k0 + lane < n) y[k0 + lane] = s0 + s1;
         }
         __syncthreads();
-        // y_i -= sum_c L[k0+c][i] z[k0+c]: one warp per row i, lane c reading
-        // L[k0+c][i] (32 contiguous floats of W's column i), a fixed shuffle sum
-        for (int i = warp; i < k0; i += NT / 32) {
-            const float v = (k0 + lane < n) ? W[(long)i * BLD + k0 + lane] * y[k0 + lane] : 0.f;
-            const float s = warp_sum(v);
-            if (lane == 0) y[i] -= s;
+        while (i < k0) {
+            float s = 0.f;
+#pragma unroll
+            for (int c = 0; c < 32; ++c) s = fmaf(w[c], y[k0 + c], s);
+            y[i] -= s;
+            i += NT;
+            if (i < k0) load();
         }
         __syncthreads();
     }
 }
 
-// r = b - A x (float64) for one system; returns berr = ||r||_inf / (anorm ||x||_inf).
+// The Cholesky factor of a 32 x 32 diagonal block by one warp (lane = row, a[] =
+// the row's columns; micro-steps of four pivots, k_leaf32.cuh): L back into a[]
+// and, four columns at a time, into Xs (8 x 32 float4), the reciprocals of its
+// diagonal into Rs.  Returns the first non-positive pivot (INT_MAX: none).
+__device__ __forceinline__ int batch_diag32(float (&a)[32], int lane, float4* Xs, float* Rs) {
+    int bad = INT_MAX;
+    leaf_micro<0, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<1, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<2, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<3, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<4, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<5, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<6, true>(a, lane, Xs, Rs, 32, bad);
+    leaf_micro<7, true>(a, lane, Xs, Rs, 32, bad);
+    return bad;
+}
+
+// Its inverse (lane = column: x_i = (delta - sum_{l<i} L_il x_l) / L_ii): the lower
+// triangle packed into I, rows of 36 with zeros above the diagonal into D.
+__device__ __forceinline__ void batch_inverse32(int lane, const float4* Xs, const float* Rs, float* I, float* D) {
+    float x[32];
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        float s0 = (i == lane) ? 1.f : 0.f, s1 = 0.f;
+#pragma unroll
+        for (int l = 0; l < i; l += 4) {
+            const float4 t = Xs[(l >> 2) * 32 + i];
+            s0 = fmaf(-t.x, x[l], s0);
+            if (l + 1 < i) s1 = fmaf(-t.y, x[l + 1], s1);
+            if (l + 2 < i) s0 = fmaf(-t.z, x[l + 2], s0);
+            if (l + 3 < i) s1 = fmaf(-t.w, x[l + 3], s1);
+        }
+        x[i] = (s0 + s1) * Rs[i];
+        if (lane <= i) I[btri(i) + lane] = x[i];
+        D[i * 36 + lane] = lane <= i ? x[i] : 0.f;
+    }
+}
+
+// sum_j A_ij x_j (float64), and with ABS sum_j |A_ij|: four interleaved
+// accumulators (column j into j % 4), eight loads in flight, added in a fixed
+// order.  (Four threads per row, a column quarter each, so that the four
+// schedulers' float64 units have equal work, and loads one group ahead, measured
+// no faster.)
+template <bool ABS>
+__device__ __forceinline__ double batch_row_dot(const BatchSys& S, const double* x, int i, double& abs_sum) {
+    const double* Ai = S.A + i;
+    double q[4] = {0.0, 0.0, 0.0, 0.0}, a = 0.0;
+    int j = 0;
+    for (; j + 8 <= S.n; j += 8) {
+        double v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = Ai[(long)(j + u) * S.lda];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            q[u & 3] = fma(v[u], x[j + u], q[u & 3]);
+            if (ABS) a += fabs(v[u]);
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+        if (j + u < S.n) {
+            const double v = Ai[(long)(j + u) * S.lda];
+            q[u & 3] = fma(v, x[j + u], q[u & 3]);
+            if (ABS) a += fabs(v);
+        }
+    }
+    abs_sum = a;
+    return (q[0] + q[1]) + (q[2] + q[3]);
+}
+
+// The block's sum of s and maxima of m1 and m2, one pass (red: 3 NT / 32 values)
 template <int NT>
-__device__ double batch_residual(const BatchSys& S, const double* x, double* r, const double* anorm_p,
-                                 double* rowabs, bool want_anorm, double* red, double* anorm_out) {
-    const int n = S.n;
-    double rmax = 0.0, amax = 0.0, xmax = 0.0;
-    for (int i = threadIdx.x; i < n; i += NT) {
-        // four interleaved accumulators (column j into j % 4), eight loads in
-        // flight, added in a fixed order
-        double q[4] = {0.0, 0.0, 0.0, 0.0}, a = 0.0;
-        const double* Ai = S.A + i;
-        int j = 0;
-        for (; j + 8 <= n; j += 8) {
-            double v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = Ai[(long)(j + u) * S.lda];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) {
-                q[u & 3] = fma(v[u], x[j + u], q[u & 3]);
-                if (want_anorm) a += fabs(v[u]);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {  // the last n % 8 columns (j is a multiple of 8 here)
-            if (j + u < n) {
-                const double v = Ai[(long)(j + u) * S.lda];
-                q[u & 3] = fma(v, x[j + u], q[u & 3]);
-                if (want_anorm) a += fabs(v);
-            }
-        }
-        const double s = S.B[i] - ((q[0] + q[1]) + (q[2] + q[3]));
+__device__ __forceinline__ void block_sum_max2(double& s, double& m1, double& m2, double* red) {
+    constexpr int NW = NT / 32;
+    s = warp_sum(s);
+    m1 = warp_max(m1);
+    m2 = warp_max(m2);
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = s;
+        red[NW + (threadIdx.x >> 5)] = m1;
+        red[2 * NW + (threadIdx.x >> 5)] = m2;
+    }
+    __syncthreads();
+    s = m1 = m2 = 0.0;
+    for (int w = 0; w < NW; ++w) {  // fixed order
+        s += red[w];
+        m1 = fmax(m1, red[NW + w]);
+        m2 = fmax(m2, red[2 * NW + w]);
+    }
+    __syncthreads();
+}
+
+// r = b - A x (float64) for one system; returns berr = ||r||_inf / (anorm
+// ||x||_inf); with want_anorm anorm = ||A||_inf is formed first.  x is complete (a
+// barrier before the call).
+template <int NT>
+__device__ double batch_residual(const BatchSys& S, const double* x, double* r, bool want_anorm, double* red,
+                                 double* anorm) {
+    double rmax = 0.0, amax = 0.0, xmax = 0.0, none = 0.0;
+    for (int i = threadIdx.x; i < S.n; i += NT) {
+        double a = 0.0;
+        const double s = S.B[i] - (want_anorm ? batch_row_dot<true>(S, x, i, a) : batch_row_dot<false>(S, x, i, a));
         r[i] = s;
         rmax = fmax(rmax, fabs(s));
         xmax = fmax(xmax, fabs(x[i]));
-        if (want_anorm) amax = fmax(amax, a);
+        amax = fmax(amax, a);
     }
-    rmax = block_max<NT>(rmax, red);
-    xmax = block_max<NT>(xmax, red);
-    double an;
+    block_sum_max2<NT>(none, rmax, xmax, red);
     if (want_anorm) {
-        an = block_max<NT>(amax, red);
-        *anorm_out = an;
-    } else {
-        an = *anorm_p;
+        amax = block_max<NT>(amax, red);
+        if (threadIdx.x == 0) *anorm = amax;
+        __syncthreads();
     }
+    const double an = *anorm;
     return (an > 0.0 && xmax > 0.0) ? rmax / (an * xmax) : rmax;
 }
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
+__global__ void __launch_bounds__(NT, 512 / NT) k_batch_chol_ir(BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* Inv = reinterpret_cast<float*>(smem_raw);          // [16][32][33]
-    float* Pn = Inv + (BMAX / 32) * 32 * 33;                   // [512][33]
-    double* xs = reinterpret_cast<double*>(Pn + BMAX * 33);    // [512]
+    float* Inv = reinterpret_cast<float*>(smem_raw);           // [16][528]
+    float* Pn = Inv + (BMAX / 32) * BTRI;                      // [32][516]
+    double* xs = reinterpret_cast<double*>(Pn + 32 * BLDP);    // [512]
     double* rs = xs + BMAX;
     double* ds = rs + BMAX;
-    double* ra = ds + BMAX;
-    float* ys = reinterpret_cast<float*>(ra + BMAX);           // [512]
+    float* ys = reinterpret_cast<float*>(ds + BMAX);           // [512]
+    // scratch of the factor: the diagonal block's rows before the panel is
+    // formed, its inverse by rows before the solution is
+    float4* Xs = reinterpret_cast<float4*>(Pn);                // [8][32]
+    float* Rs = Pn + 8 * 32 * 4;                               // [32]
+    float* D = reinterpret_cast<float*>(xs);                   // [32][36]
     __shared__ int s_idx, s_bad;
-    __shared__ double red[NT / 32];
+    __shared__ double red[3 * NT / 32];
     __shared__ double s_anorm;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float* W = a.scratch + (long)blockIdx.x * BLD * BLD;
@@ -204,19 +327,18 @@ __global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
         }
         if (tid == 0) s_bad = 0;
         __syncthreads();
-        // (every entry of the n x n block, four per thread at a time; only
-        // the lower triangle is kept)
-        for (int e0 = tid; e0 < n * n; e0 += 4 * NT) {
-            double v[4];
+        // (a warp per column of the lower triangle, four loads in flight per lane)
+        for (int j = warp; j < n; j += NT / 32) {
+            const double dj = ds[j];
+            const double* aj = S.A + (long)j * S.lda;
+            float* wj = W + (long)j * BLD;
+            for (int i0 = j + lane; i0 < n; i0 += 128) {
+                double v[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = e0 + u * NT, j = e / n, i = e - j * n;
-                v[u] = (e < n * n && i >= j) ? S.A[i + (long)j * S.lda] : 0.0;
-            }
+                for (int u = 0; u < 4; ++u) v[u] = i0 + 32 * u < n ? aj[i0 + 32 * u] : 0.0;
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int e = e0 + u * NT, j = e / n, i = e - j * n;
-                if (e < n * n && i >= j) W[i + (long)j * BLD] = (float)(ds[i] * v[u] * ds[j]);
+                for (int u = 0; u < 4; ++u)
+                    if (i0 + 32 * u < n) wj[i0 + 32 * u] = (float)(ds[i0 + 32 * u] * v[u] * dj);
             }
         }
         __syncthreads();
@@ -231,65 +353,42 @@ __global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
                     const int r = k0 + lane, cc = k0 + c;
                     av[c] = (r < n && cc < n) ? ((c <= lane) ? W[r + (long)cc * BLD] : 0.f) : (lane == c ? 1.f : 0.f);
                 }
-                int badj = -1;
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float piv = __shfl_sync(0xffffffffu, av[j], j);
-                    if (!(piv > 0.f)) {
-                        if (badj < 0) badj = j;
-                        piv = 1.f;
-                    }
-                    const float dj = sqrtf(piv), inv = 1.f / dj;
-                    av[j] = (lane == j) ? dj : (lane > j ? av[j] * inv : av[j]);
-#pragma unroll
-                    for (int l = 0; l < 32; ++l) {
-                        if (l > j) {
-                            const float t = __shfl_sync(0xffffffffu, av[j], l);
-                            av[l] = (lane >= l) ? fmaf(-av[j], t, av[l]) : av[l];
-                        }
-                    }
-                }
+                const int badj = batch_diag32(av, lane, Xs, Rs);
 #pragma unroll
                 for (int c = 0; c < 32; ++c)
                     if (k0 + lane < n && k0 + c < n && c <= lane) W[k0 + lane + (long)(k0 + c) * BLD] = av[c];
-                if (badj >= 0 && k0 + badj < n && lane == 0) {
+                if (badj < n - k0 && lane == 0) {
                     s_bad = 1;
                     a.rep[sid].info = k0 + badj + 1;
                 }
                 __syncwarp();
-                // inverse of the 32x32 diagonal block: lane = column
-                float* I = Inv + kb * 32 * 33;
-                float xv[32];
-#pragma unroll
-                for (int i = 0; i < 32; ++i) {
-                    float s = (i == lane) ? 1.f : 0.f;
-                    const float lii = __shfl_sync(0xffffffffu, av[i], i);
-#pragma unroll
-                    for (int l = 0; l < 32; ++l)
-                        if (l < i) s = fmaf(-__shfl_sync(0xffffffffu, av[l], i), xv[l], s);
-                    xv[i] = s / lii;
-                }
-#pragma unroll
-                for (int i = 0; i < 32; ++i) I[i * 33 + lane] = xv[i];
+                batch_inverse32(lane, Xs, Rs, Inv + kb * BTRI, D);
             }
             __syncthreads();
             if (s_bad) break;
             const int R = n - k0 - 32;
             if (R <= 0) break;
-            const float* I = Inv + kb * 32 * 33;
-            // panel: rows below, X = B I^T
+            // panel: rows below, X = B D^T
             for (int i = tid; i < R; i += NT) {
                 float b[32];
 #pragma unroll
                 for (int c = 0; c < 32; ++c) b[c] = W[(k0 + 32 + i) + (long)(k0 + c) * BLD];
-#pragma unroll 4
-                for (int c = 0; c < 32; ++c) {
-                    float s = 0.f;
 #pragma unroll
-                    for (int l = 0; l < 32; ++l)
-                        if (l <= c) s = fmaf(b[l], I[c * 33 + l], s);
-                    W[(k0 + 32 + i) + (long)(k0 + c) * BLD] = s;
-                    Pn[c * BLDP + i] = round_op(s, a.prec);
+                for (int g = 0; g < 4; ++g) {  // D is zero above its diagonal
+#pragma unroll 2
+                    for (int c = 8 * g; c < 8 * g + 8; ++c) {
+                        float s0 = 0.f, s1 = 0.f;
+#pragma unroll
+                        for (int l = 0; l < 8 * g + 8; l += 4) {
+                            const float4 d = *reinterpret_cast<const float4*>(D + c * 36 + l);
+                            s0 = fmaf(b[l], d.x, s0);
+                            s1 = fmaf(b[l + 1], d.y, s1);
+                            s0 = fmaf(b[l + 2], d.z, s0);
+                            s1 = fmaf(b[l + 3], d.w, s1);
+                        }
+                        W[(k0 + 32 + i) + (long)(k0 + c) * BLD] = s0 + s1;
+                        Pn[c * BLDP + i] = round_op(s0 + s1, a.prec);
+                    }
                 }
             }
             for (int e = tid; e < 32 * 4; e += NT) Pn[(e >> 2) * BLDP + R + (e & 3)] = 0.f;  // rows R.. of the last group
@@ -346,16 +445,23 @@ __global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
             __syncthreads();
             continue;
         }
-        // refinement (Algorithm 1, lines 2-7)
-        for (int i = tid; i < n; i += NT) ys[i] = (float)(ds[i] * S.B[i]);
+        // refinement (Algorithm 1, lines 2-7); it = -1 is line 2's solve
+        for (int i = tid; i < n; i += NT) {
+            rs[i] = S.B[i];
+            xs[i] = 0.0;
+        }
         __syncthreads();
-        batch_lsolve<NT>(W, Inv, ys, n);
-        for (int i = tid; i < n; i += NT) xs[i] = ds[i] * (double)ys[i];
-        __syncthreads();
-        double berr = batch_residual<NT>(S, xs, rs, &s_anorm, ra, true, red, &s_anorm);
-        int it = 0, extra = a.polish;
+        int it = -1, extra = a.polish;
         bool conv = false;
+        double berr = 0.0;
         for (;;) {
+            for (int i = tid; i < 32 * nb; i += NT) ys[i] = i < n ? (float)(ds[i] * rs[i]) : 0.f;
+            __syncthreads();
+            batch_lsolve<NT>(W, Inv, ys, n);
+            for (int i = tid; i < n; i += NT) xs[i] += ds[i] * (double)ys[i];
+            __syncthreads();
+            berr = batch_residual<NT>(S, xs, rs, it < 0, red, &s_anorm);
+            ++it;
             if (berr <= a.tol) {
                 if (extra <= 0) {
                     conv = true;
@@ -366,13 +472,6 @@ __global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
                 extra = a.polish;
             }
             if (it >= a.maxit) break;
-            for (int i = tid; i < n; i += NT) ys[i] = (float)(ds[i] * rs[i]);
-            __syncthreads();
-            batch_lsolve<NT>(W, Inv, ys, n);
-            for (int i = tid; i < n; i += NT) xs[i] += ds[i] * (double)ys[i];
-            __syncthreads();
-            berr = batch_residual<NT>(S, xs, rs, &s_anorm, ra, false, red, nullptr);
-            ++it;
         }
         for (int i = tid; i < n; i += NT) S.X[i] = xs[i];
         if (tid == 0) {
@@ -386,9 +485,13 @@ __global__ void __launch_bounds__(NT, 1) k_batch_chol_ir(BatchArgs a) {
 
 // Jacobi-preconditioned CG in float64 per system (x0 = 0), restarted from
 // the true residual when the recursive one claims convergence but the true
-// backward error does not meet the tolerance.
+// backward error does not meet the tolerance.  Bound: the float64 rate (n^2
+// multiply-adds a step, one SM's float64 units take two a cycle); two CTAs of 256
+// threads share an SM to keep them busy through each other's reductions: 512
+// systems of order 32 .. 256 take 5.65 ms with one, 5.25 with two, 7.4 with three
+// (the systems no longer stay in the SM's L1).
 template <int NT>
-__global__ void __launch_bounds__(NT, 1) k_batch_pcg(BatchArgs a) {
+__global__ void __launch_bounds__(NT, 512 / NT) k_batch_pcg(BatchArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* xs = reinterpret_cast<double*>(smem_raw);
     double* rs = xs + BMAX;
@@ -397,7 +500,7 @@ __global__ void __launch_bounds__(NT, 1) k_batch_pcg(BatchArgs a) {
     double* qs = zs + BMAX;
     double* dinv = qs + BMAX;
     __shared__ int s_idx;
-    __shared__ double red[NT / 32];
+    __shared__ double red[3 * NT / 32];
     __shared__ double s_anorm;
     const int tid = threadIdx.x;
     for (;;) {
@@ -412,49 +515,49 @@ __global__ void __launch_bounds__(NT, 1) k_batch_pcg(BatchArgs a) {
             xs[i] = 0.0;
         }
         __syncthreads();
-        double berr = batch_residual<NT>(S, xs, rs, &s_anorm, nullptr, true, red, &s_anorm);
+        double berr = batch_residual<NT>(S, xs, rs, true, red, &s_anorm);
         int it = 0;
         bool conv = false;
         for (int restart = 0; restart < 4 && !conv; ++restart) {
-            double rho = 0.0;
+            double rho = 0.0, xmax = 0.0, rmax = 0.0;
             for (int i = tid; i < n; i += NT) {
-                zs[i] = dinv[i] * rs[i];
-                ps[i] = zs[i];
-                rho += rs[i] * zs[i];
+                const double r = rs[i], z = dinv[i] * r;
+                zs[i] = z;
+                ps[i] = z;
+                rho += r * z;
+                xmax = fmax(xmax, fabs(xs[i]));
+                rmax = fmax(rmax, fabs(r));
             }
-            rho = block_sum<NT>(rho, red);
+            block_sum_max2<NT>(rho, xmax, rmax, red);  // its barriers also publish ps
             for (; it < a.maxit; ++it) {
-                double xmax = 0.0, rmax = 0.0;
-                for (int i = tid; i < n; i += NT) {
-                    xmax = fmax(xmax, fabs(xs[i]));
-                    rmax = fmax(rmax, fabs(rs[i]));
-                }
-                xmax = block_max<NT>(xmax, red);
-                rmax = block_max<NT>(rmax, red);
                 if (xmax > 0.0 && rmax <= 0.5 * a.tol * s_anorm * xmax) break;
                 double pq = 0.0;
                 for (int i = tid; i < n; i += NT) {
-                    double s = 0.0;
-                    for (int j = 0; j < n; ++j) s = fma(S.A[i + (long)j * S.lda], ps[j], s);
+                    double none;
+                    const double s = batch_row_dot<false>(S, ps, i, none);
                     qs[i] = s;
                     pq += ps[i] * s;
                 }
                 pq = block_sum<NT>(pq, red);
                 const double alpha = rho / pq;
                 double rz = 0.0;
+                xmax = rmax = 0.0;
                 for (int i = tid; i < n; i += NT) {
-                    xs[i] = fma(alpha, ps[i], xs[i]);
-                    rs[i] = fma(-alpha, qs[i], rs[i]);
-                    zs[i] = dinv[i] * rs[i];
-                    rz += rs[i] * zs[i];
+                    const double x = fma(alpha, ps[i], xs[i]), r = fma(-alpha, qs[i], rs[i]), z = dinv[i] * r;
+                    xs[i] = x;
+                    rs[i] = r;
+                    zs[i] = z;
+                    rz += r * z;
+                    xmax = fmax(xmax, fabs(x));
+                    rmax = fmax(rmax, fabs(r));
                 }
-                rz = block_sum<NT>(rz, red);
+                block_sum_max2<NT>(rz, xmax, rmax, red);
                 const double beta = rz / rho;
                 rho = rz;
                 for (int i = tid; i < n; i += NT) ps[i] = fma(beta, ps[i], zs[i]);
                 __syncthreads();
             }
-            berr = batch_residual<NT>(S, xs, rs, &s_anorm, nullptr, false, red, nullptr);
+            berr = batch_residual<NT>(S, xs, rs, false, red, &s_anorm);
             conv = berr <= a.tol;
             if (it >= a.maxit) break;
         }

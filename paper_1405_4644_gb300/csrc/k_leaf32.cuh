@@ -230,7 +230,7 @@ __device__ __forceinline__ void leaf_inverse32(const float* S, int o, const floa
 // step.  Measured: 18.5 us per leaf launched back to back (of 31k cycles, 17.8k
 // in the four steps' pivots, 7k in the updates between them); a whole solve of
 // n = 16384 went from 27.96 to 25.26 ms against one pivot at a time, 21 us a leaf.
-__global__ void __launch_bounds__(LEAF_THREADS, 1) k_potrf_leaf32(float* __restrict__ W, long ldw, int k, int nb,
+static __global__ void __launch_bounds__(LEAF_THREADS, 1) k_potrf_leaf32(float* __restrict__ W, long ldw, int k, int nb,
                                                                float* __restrict__ Dinv32, Mirror mir, DevStatus* st) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* S = reinterpret_cast<float*>(smem_raw);           // [128][132] the block, then L
@@ -387,7 +387,7 @@ __device__ __forceinline__ void trsm_step(float* Bs, const float* Ls, const floa
 // b_ready: the previous kernel in the stream (the leaf) does not write B, and
 // what does was complete before the leaf passed its own wait, so B is loaded
 // before waiting (programmatic dependent launch).
-__global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, long ldw, int r0, int m, int c0,
+static __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, long ldw, int r0, int m, int c0,
                                                      const float* __restrict__ Dinv32, Mirror mir,
                                                      const DevStatus* st, int b_ready) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -458,7 +458,7 @@ __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict__ W, l
 // Rows past n are the identity, as in the leaf.
 constexpr size_t block_inverse_smem() { return (size_t)(2 * 128 * LD32 + 32 * 97) * sizeof(float); }
 
-__global__ void __launch_bounds__(256) k_block_inverse(const float* __restrict__ W, long ldw, int n,
+static __global__ void __launch_bounds__(256) k_block_inverse(const float* __restrict__ W, long ldw, int n,
                                                        const float* __restrict__ Dinv32, float* __restrict__ LinvT) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* S = reinterpret_cast<float*>(smem_raw);  // [128][129] L_JJ

@@ -27,11 +27,15 @@ struct spd_batch {
 
 namespace {
 
+// CTAs of a launch: 512 threads per SM (the kernels' launch bounds), no more than
+// systems
+int batch_ctas(const spd_batch* b, int nt) { return std::max(1, std::min(b->h->sms * (512 / nt), b->count)); }
+
 template <int NT>
 void launch_batch(spd_batch* b, int method, const BatchArgs& a, cudaStream_t s) {
-    const size_t smem = batch_smem_bytes();
-    if (method == 0) k_batch_chol_ir<NT><<<b->ctas, NT, smem, s>>>(a);
-    else k_batch_pcg<NT><<<b->ctas, NT, smem, s>>>(a);
+    const int ctas = batch_ctas(b, NT);
+    if (method == 0) k_batch_chol_ir<NT><<<ctas, NT, batch_smem_bytes(), s>>>(a);
+    else k_batch_pcg<NT><<<ctas, NT, batch_pcg_smem_bytes(), s>>>(a);
 }
 
 void set_batch_attrs() {
@@ -39,8 +43,6 @@ void set_batch_attrs() {
         const int smem = (int)batch_smem_bytes();
         cudaFuncSetAttribute(k_batch_chol_ir<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         cudaFuncSetAttribute(k_batch_chol_ir<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_batch_pcg<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        cudaFuncSetAttribute(k_batch_pcg<512>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         return true;
     }();
     (void)done;
@@ -78,7 +80,7 @@ extern "C" spd_status spd_batch_create(spd_handle* h, int count, const int* n, c
     b->h = h;
     b->count = count;
     b->nmax = nmax;
-    b->ctas = std::max(1, std::min(h->sms, count));
+    b->ctas = std::max(1, std::min(2 * h->sms, count));  // scratch of the largest Cholesky-IR launch
     set_batch_attrs();
     cudaError_t e = cudaMalloc(&b->sys, sizeof(BatchSys) * std::max(count, 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->order, sizeof(int) * std::max(count, 1));
@@ -280,7 +282,7 @@ extern "C" spd_status spd_batch_info(const spd_batch* b, int method, int* thread
     if (!b || (method != SPD_BATCH_CHOL_IR && method != SPD_BATCH_PCG_JACOBI)) return SPD_ERR_ARG;
     const int mi = method == SPD_BATCH_CHOL_IR ? 0 : 1;
     if (threads_per_cta) *threads_per_cta = b->threads[mi];
-    if (ctas) *ctas = b->ctas;
+    if (ctas) *ctas = batch_ctas(b, b->threads[mi] ? b->threads[mi] : 512);
     if (tune_ms) {
         tune_ms[0] = b->tune_ms[mi][0];
         tune_ms[1] = b->tune_ms[mi][1];
