@@ -143,8 +143,8 @@ typedef enum spd_resid {
                                     to contract).  report.shift gives sigma */
 #define SPD_FACTOR_BLOCK_SWEEPS 32u /* float32 factors: apply the factor
                                     with the sweeps over 128-row blocks.  By
-                                    default a factor of at least 16 blocks
-                                    also holds the inverses of its diagonal
+                                    default a factor of 2 to 8 blocks or of
+                                    at least 16 also holds the inverses of its diagonal
                                     super-blocks (8 blocks each, formed once,
                                     4 (1024)^2 bytes each) and is applied with
                                     the super-block sweeps */

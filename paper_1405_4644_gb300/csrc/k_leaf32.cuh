@@ -18,7 +18,6 @@
 #pragma once
 #include "common.cuh"
 
-#define LD32 129  // k_block_inverse
 #define LDL 132   // the leaf: 16-byte rows, eight consecutive rows in distinct banks
 
 // Dinv32 for block b lives at Dinv32 + b * 4096: four row-major 32x32
@@ -452,60 +451,108 @@ static __global__ void __launch_bounds__(256, 2) k_trsm_leaf32(float* __restrict
     }
 }
 
-// (L_JJ^{-1})^T of every 128x128 diagonal block (one CTA per block, after
-// the factorisation): X = L^{-1} by block rows, X_ii = D_i (the leaf's 32x32
-// inverses) and X_i,0:i = -D_i (L_i,0:i X_0:i,0:i); LinvT[l][c] = X[c][l].
-// Rows past n are the identity, as in the leaf.
-constexpr size_t block_inverse_smem() { return (size_t)(2 * 128 * LD32 + 32 * 97) * sizeof(float); }
+// The inverse of every 128x128 diagonal block (one CTA per block, after the
+// factorisation), X = L_JJ^{-1} by block rows: X_ii = D_i (the leaf's 32x32
+// inverses), X_i,0:i = -D_i (L_i,0:i X_0:i,0:i).  Kept transposed in shared memory,
+// so that both products are of rows with rows, four k per load (leaf_tile's
+// layout).  LinvT[l][c] = X[c][l]; with Xsb also X itself as diagonal block J mod
+// sbb of super-block J / sbb (order 128 sbb).  Rows past n are the identity.
+constexpr size_t block_inverse_smem() { return (size_t)(2 * 128 * LDL + 96 * 36 + 4 * 32 * 36) * sizeof(float); }
+
+// 4 x 4 outputs: out[r][q] = sum over k in [k0, k1) (multiples of 4) of A[i + r][k] B[j + 8 q][k]
+__device__ __forceinline__ void rowrow_tile(float (&acc)[4][4], const float* A, int lda, const float* B, int ldb, int k0,
+                                            int k1) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+#pragma unroll 2
+    for (int k = k0; k < k1; k += 4) {
+        float4 x[4], y[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r) x[r] = *reinterpret_cast<const float4*>(A + r * lda + k);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = *reinterpret_cast<const float4*>(B + 8 * q * ldb + k);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                acc[r][q] = fmaf(x[r].x, y[q].x, acc[r][q]);
+                acc[r][q] = fmaf(x[r].y, y[q].y, acc[r][q]);
+                acc[r][q] = fmaf(x[r].z, y[q].z, acc[r][q]);
+                acc[r][q] = fmaf(x[r].w, y[q].w, acc[r][q]);
+            }
+    }
+}
 
 static __global__ void __launch_bounds__(256) k_block_inverse(const float* __restrict__ W, long ldw, int n,
-                                                       const float* __restrict__ Dinv32, float* __restrict__ LinvT) {
+                                                       const float* __restrict__ Dinv32, float* __restrict__ LinvT,
+                                                       float* __restrict__ Xsb, int sbb) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* S = reinterpret_cast<float*>(smem_raw);  // [128][129] L_JJ
-    float* X = S + 128 * LD32;                      // [128][129] L_JJ^{-1}
-    float* Tmp = X + 128 * LD32;                    // [32][97]
+    float* S = reinterpret_cast<float*>(smem_raw);  // [128][132] L_JJ
+    float* XT = S + 128 * LDL;                      // [128][132] (L_JJ^{-1})^T
+    float* TT = XT + 128 * LDL;                     // [96][36] (L_i,0:i X_0:i,0:i)^T
+    float* Ds = TT + 96 * 36;                       // [4][32][36] D_i
     const int tid = threadIdx.x;
     const int J = blockIdx.x;
     const long k = (long)J * 128;
     const int nb = (int)min((long)128, n - k);
     const float* dg = Dinv32 + (long)J * 4096;
-    for (int e = tid; e < 128 * 128; e += 256) {
-        const int r = e >> 7, c = e & 127;
-        float v;
-        if (r < nb && c < nb) v = (c <= r) ? W[(k + r) * ldw + k + c] : 0.f;
-        else v = (r == c) ? 1.f : 0.f;
-        S[r * LD32 + c] = v;
-        const int br = r >> 5, bc = c >> 5;
-        X[r * LD32 + c] = (br == bc) ? dg[br * 1024 + (r & 31) * 32 + (c & 31)] : 0.f;
+    for (int e = tid; e < 128 * 32; e += 256) {
+        const int r = e >> 5, c4 = (e & 31) * 4;
+        float4 f = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r < nb && k + c4 < ldw) f = *reinterpret_cast<const float4*>(W + (k + r) * ldw + k + c4);
+        float v[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int c = c4 + q;
+            if (r >= nb || c >= nb) v[q] = (r == c) ? 1.f : 0.f;
+            else if (c > r) v[q] = 0.f;
+        }
+        *reinterpret_cast<float4*>(S + r * LDL + c4) = make_float4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<float4*>(XT + r * LDL + c4) = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+    __syncthreads();
+    for (int e = tid; e < 4096; e += 256) {  // D_b[r][c] (zeros above its diagonal)
+        const int b = e >> 10, r = (e >> 5) & 31, c = e & 31;
+        const float v = dg[e];
+        Ds[(b * 32 + r) * 36 + c] = v;
+        XT[(32 * b + c) * LDL + 32 * b + r] = v;
     }
     __syncthreads();
     for (int i = 1; i < 4; ++i) {
-        const int ri = i * 32, w = i * 32;  // rows ri..ri+31 of X, columns 0..w-1
-        for (int e = tid; e < 32 * w; e += 256) {
-            const int rr = e / w, c = e - rr * w;
-            const float* lr = S + (ri + rr) * LD32;
-            float s0 = 0.f, s1 = 0.f;
-            int l = (c >> 5) << 5;
-            for (; l + 1 < ri; l += 2) {  // two chains: shorter dependency
-                s0 = fmaf(lr[l], X[l * LD32 + c], s0);
-                s1 = fmaf(lr[l + 1], X[(l + 1) * LD32 + c], s1);
-            }
-            if (l < ri) s0 = fmaf(lr[l], X[l * LD32 + c], s0);
-            Tmp[rr * 97 + c] = s0 + s1;
+        const int ri = 32 * i;
+        float acc[4][4];
+        for (int e = tid; e < 64 * i; e += 256) {  // T[r][c]: 4 rows x columns c, c + 8, ..; k from c's block on
+            const int cb = e >> 6, r = ((e >> 3) & 7) * 4, c = 32 * cb + (e & 7);
+            rowrow_tile(acc, S + (ri + r) * LDL, LDL, XT + c * LDL, LDL, 32 * cb, ri);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<float4*>(TT + (c + 8 * q) * 36 + r) =
+                    make_float4(acc[0][q], acc[1][q], acc[2][q], acc[3][q]);
         }
         __syncthreads();
-        for (int e = tid; e < 32 * w; e += 256) {
-            const int rr = e / w, c = e - rr * w;
-            const float* ir = X + (ri + rr) * LD32 + ri;
-            float s = 0.f;
-            for (int l = 0; l <= rr; ++l) s = fmaf(ir[l], Tmp[l * 97 + c], s);
-            X[(ri + rr) * LD32 + c] = -s;
+        for (int e = tid; e < 64 * i; e += 256) {  // X[ri + r][c] = -sum_q D_i[r][q] T[q][c]
+            const int cb = e >> 6, r = ((e >> 3) & 7) * 4, c = 32 * cb + (e & 7);
+            rowrow_tile(acc, Ds + (32 * i + r) * 36, 36, TT + c * 36, 36, 0, 32);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<float4*>(XT + (c + 8 * q) * LDL + ri + r) =
+                    make_float4(-acc[0][q], -acc[1][q], -acc[2][q], -acc[3][q]);
         }
         __syncthreads();
     }
     float* out = LinvT + (long)J * 16384;
-    for (int e = tid; e < 128 * 128; e += 256) {
-        const int l = e >> 7, c = e & 127;
-        out[e] = X[c * LD32 + l];
+    for (int e = tid; e < 128 * 32; e += 256) {
+        const int l = e >> 5, c4 = (e & 31) * 4;
+        *reinterpret_cast<float4*>(out + l * 128 + c4) = *reinterpret_cast<const float4*>(XT + l * LDL + c4);
+    }
+    if (Xsb) {
+        const long ld = (long)sbb * 128;
+        float* xo = Xsb + (long)(J / sbb) * ld * ld + (long)(J % sbb) * 128 * (ld + 1);
+        for (int e = tid; e < 128 * 128; e += 256) {
+            const int r = e >> 7, c = e & 127;
+            xo[r * ld + c] = XT[c * LDL + r];
+        }
     }
 }

@@ -397,131 +397,77 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
 // ---------------------------------------------------------------------------
 // the super-block inverses, once per factor
 // ---------------------------------------------------------------------------
-// X_I = L_II^{-1} by block forward substitution: X_cc = L_cc^{-1} (the
-// transpose of LinvT's block), then for b = c+1 .. nb-1,
-// X_bc = -L_bb^{-1} (sum_{k=c}^{b-1} L_bk X_kc).  A strip of 32 columns of
-// block column c only needs the same strip of the blocks above it, so CTA
-// (4 c + s, I) forms strip s of block column c of X_I on its own.  Rows of L
-// past n are zero and LinvT's rows past n are the identity; those rows of X
-// meet only right-hand-side rows past n, which the sweeps hold at zero.
-// Products are 128 x 128 x 32 in float32 through shared memory, thread
-// (ty, tx) = (tid / 8, tid % 8) owning a 4 x 4 block of the result.
-constexpr int SB_STRIPS = 4;  // 32-column strips per block column
-constexpr size_t sb_inverse_smem() { return (size_t)(128 * 33 + 32 * 36 + 128 * 36) * sizeof(float); }
-
-static __global__ void __launch_bounds__(256) k_sb_inverse(const float* __restrict__ W, long ldw, int n, int NB,
-                                                           const float* __restrict__ LinvT, int SBB,
-                                                           float* __restrict__ X) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    float* As = reinterpret_cast<float*>(smem_raw);  // [128][33] a 128 x 32 slice of the left factor
-    float* Bs = As + 128 * 33;                       // [32][36]  a 32 x 32 slice of the right factor
-    float* Ts = Bs + 32 * 36;                        // [128][36] T = sum_k L_bk X_kc (this strip)
-    const int c = blockIdx.x / SB_STRIPS, strip = blockIdx.x % SB_STRIPS;
-    const int I = blockIdx.y, tid = threadIdx.x;
-    const int S = SBB * 128;
-    const int jb0 = I * SBB, nb = min(SBB, NB - jb0);
-    if (c >= nb) return;
+// X_I = L_II^{-1} by doubling: the 128-row diagonal blocks' inverses come from
+// k_block_inverse; with the inverses A^{-1}, C^{-1} of two neighbouring diagonal
+// blocks of order h in place, the block below the first is -C^{-1} (B A^{-1}), B
+// its block of L, for h = 128, 256, 512: two products per level, T = B A^{-1}
+// (kept in the unused block above the diagonal) and -C^{-1} T, over all pairs of
+// all super-blocks at once.  Block forward substitution down each column strip
+// was a chain of up to 35 products of 128 x 128 x 32 in one CTA: 282 us whatever
+// the order (558 at n = 16384).
+//
+// One 64 x 64 tile of the product per CTA, 4 x 4 per thread, 16 of K at a time
+// through shared memory with the next 16 in registers; a triangular operand's
+// zero half is left out.  Rows of L past n are zero and rows of the inverse past
+// n are the identity; those rows of X meet only right-hand-side rows past n,
+// which the sweeps hold at zero.
+constexpr int SBP_K = 16;
+template <bool FIRST>
+static __global__ void __launch_bounds__(256) k_sb_product(const float* __restrict__ W, long ldw, int n, int NB, int SBB,
+                                                           float* __restrict__ X, int h) {
+    __shared__ __align__(16) float As[SBP_K][68];  // [k][row]
+    __shared__ __align__(16) float Bs[SBP_K][68];  // [k][column]
+    const int S = SBB * 128, I = blockIdx.z, tid = threadIdx.x;
+    const int th = h / 64, pair = blockIdx.y;
+    const int ti = blockIdx.x / th, tj = blockIdx.x % th;  // tile of the h x h product
+    const int r0 = pair * 2 * h;                           // the pair's first row in the super-block
+    const int rows = min(SBB, NB - I * SBB) * 128;         // rows of this super-block
+    if (r0 + h + ti * 64 >= rows) return;
     float* XI = X + (long)I * S * S;
-    const int x0 = c * 128 + strip * 32;  // first column of the strip in X_I
-    const int ty = tid >> 3, tx = tid & 7;
-    // X_cc (this strip) = (LinvT block)^T
-    {
-        const float* lt = LinvT + (long)(jb0 + c) * 16384;
-        for (int e = tid; e < 128 * 32; e += 256) {
-            const int r = e >> 5, col = e & 31;
-            XI[(long)(c * 128 + r) * S + x0 + col] = lt[(strip * 32 + col) * 128 + r];
-        }
-    }
-    __syncthreads();
-    float acc[4][4];
-    // chunk q of T's K loop: block k = c + q / 4, columns kk = 32 (q % 4);
-    // the next chunk's entries wait in registers while this one is used
-    float an[16], bn[4];
-    auto load_chunk = [&](int b, int q) {
-        const int k = c + (q >> 2), kk = (q & 3) * 32;
-#pragma unroll
-        for (int i = 0; i < 16; ++i) {  // As[r][q'] = L[row r of block b][col kk + q' of block k]
-            const int e = tid + i * 256, r = e >> 5, qq = e & 31;
-            const long gr = (long)(jb0 + b) * 128 + r;
-            an[i] = gr < n ? W[gr * ldw + (long)(jb0 + k) * 128 + kk + qq] : 0.f;
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {  // Bs[q'][col] = X_kc[kk + q'][strip col]
-            const int e = tid + i * 256, qq = e >> 5, col = e & 31;
-            bn[i] = __ldcg(XI + (long)(k * 128 + kk + qq) * S + x0 + col);
-        }
+    const float* Lb = W + ((long)I * S + r0 + h) * ldw + (long)I * S + r0;  // B: rows of the second half
+    // FIRST: T[i][j] = sum_{k >= j} B[i][k] A^{-1}[k][j], to rows r0 .., columns r0 + h ..
+    // else:  X[i][j] = -sum_{k <= i} C^{-1}[i][k] T[k][j], to rows r0 + h .., columns r0 ..
+    const float* Am = XI + (long)(r0 + h) * S + r0 + h;                       // C^{-1}
+    const float* Bm = FIRST ? XI + (long)r0 * S + r0 : XI + (long)r0 * S + r0 + h;  // A^{-1} or T
+    const int klo = FIRST ? tj * 64 : 0, khi = FIRST ? h : (ti + 1) * 64;
+    const int ar = tid >> 2, ak = (tid & 3) * 4;    // A: row ar, k ak .. ak + 3
+    const int bk = tid >> 4, bc = (tid & 15) * 4;   // B: row bk, columns bc .. bc + 3
+    const long arow = ti * 64 + ar;
+    const bool aok = !FIRST || (long)I * S + r0 + h + arow < n;
+    float4 av, bv;
+    auto load = [&](int k) {
+        const float* pa = FIRST ? Lb + arow * ldw + k + ak : Am + arow * S + k + ak;
+        av = aok ? *reinterpret_cast<const float4*>(pa) : make_float4(0.f, 0.f, 0.f, 0.f);
+        bv = *reinterpret_cast<const float4*>(Bm + (long)(k + bk) * S + tj * 64 + bc);
     };
-    for (int b = c + 1; b < nb; ++b) {
-        // T = sum_{k=c}^{b-1} L_bk X_kc
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-        const int nq = (b - c) * 4;
-        load_chunk(b, 0);
-        for (int q = 0; q < nq; ++q) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int e = tid + i * 256;
-                As[(e >> 5) * 33 + (e & 31)] = an[i];
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int e = tid + i * 256;
-                Bs[(e >> 5) * 36 + (e & 31)] = bn[i];
-            }
-            __syncthreads();
-            if (q + 1 < nq) load_chunk(b, q + 1);
-#pragma unroll 8
-            for (int qq = 0; qq < 32; ++qq) {
-                float av[4], bv[4];
-#pragma unroll
-                for (int i = 0; i < 4; ++i) av[i] = As[(ty * 4 + i) * 33 + qq];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) bv[j] = Bs[qq * 36 + tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-            }
-            __syncthreads();
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) Ts[(ty * 4 + i) * 36 + tx * 4 + j] = acc[i][j];
+    float acc[4][4] = {};
+    const int tr = (tid >> 4) * 4, tc = (tid & 15) * 4;
+    load(klo);
+    for (int k = klo; k < khi; k += SBP_K) {
+        As[ak][ar] = av.x;
+        As[ak + 1][ar] = av.y;
+        As[ak + 2][ar] = av.z;
+        As[ak + 3][ar] = av.w;
+        *reinterpret_cast<float4*>(&Bs[bk][bc]) = bv;
         __syncthreads();
-        // X_bc = -L_bb^{-1} T, L_bb^{-1}[r][q] = LinvT_b[q][r]
-        const float* lt = LinvT + (long)(jb0 + b) * 16384;
+        if (k + SBP_K < khi) load(k + SBP_K);
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int q = 0; q < SBP_K; ++q) {
+            const float4 x = *reinterpret_cast<const float4*>(&As[q][tr]), y = *reinterpret_cast<const float4*>(&Bs[q][tc]);
+            const float xr[4] = {x.x, x.y, x.z, x.w}, yc[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-        for (int kk = 0; kk < 128; kk += 32) {
-            for (int e = tid; e < 128 * 32; e += 256) {  // As[r][q] = L_bb^{-1}[r][kk + q]
-                const int r = e >> 5, q = e & 31;
-                As[r * 33 + q] = lt[(kk + q) * 128 + r];
-            }
-            __syncthreads();
-#pragma unroll 8
-            for (int q = 0; q < 32; ++q) {
-                float av[4], bv[4];
+            for (int i = 0; i < 4; ++i)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) av[i] = As[(ty * 4 + i) * 33 + q];
-#pragma unroll
-                for (int j = 0; j < 4; ++j) bv[j] = Ts[(kk + q) * 36 + tx * 4 + j];
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
-            }
-            __syncthreads();
+                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(xr[i], yc[j], acc[i][j]);
         }
+        __syncthreads();
+    }
+    float* out = FIRST ? XI + (long)(r0 + ti * 64 + tr) * S + r0 + h + tj * 64 + tc
+                       : XI + (long)(r0 + h + ti * 64 + tr) * S + r0 + tj * 64 + tc;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-                XI[(long)(b * 128 + ty * 4 + i) * S + x0 + tx * 4 + j] = -acc[i][j];
-        __syncthreads();  // X_bc is read (through L2) by the next b
+    for (int i = 0; i < 4; ++i) {
+        const float4 v = FIRST ? make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3])
+                               : make_float4(-acc[i][0], -acc[i][1], -acc[i][2], -acc[i][3]);
+        *reinterpret_cast<float4*>(out + (long)i * S) = v;
     }
 }

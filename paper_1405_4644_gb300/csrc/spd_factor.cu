@@ -26,6 +26,13 @@
 
 namespace {
 
+// Whether a float32 factor of nb 128-row blocks is applied with the super-block
+// sweeps: with one super-block a sweep is its triangular product, with no chain at
+// all (14 us a pair at n = 1024, one right-hand side, against 57 under ncu); from two
+// full ones on the chain is short enough.  Between, the
+// 128-block sweeps stay.
+inline bool sb_sweeps(int nb) { return (nb >= 2 && nb <= SPD_SB_BLOCKS) || nb >= 2 * SPD_SB_BLOCKS; }
+
 struct FCtx {
     spd_handle* h;
     spd_factor_t* F;
@@ -435,7 +442,7 @@ spd_status factor_once(spd_handle* h, int n, const double* A, int lda, int prec,
         if (prec == SPD_PREC_FP64) req += sizeof(double) * (std::max<size_t>(nW, 1) + 4096 * nb);
         else req += sizeof(float) * (std::max<size_t>(nW, 1) + (1 + 4 + 0.25) * 16384 * nb) +
                     (kind ? mirror_elem(kind) * std::max<size_t>(nW, 1) : 0) +
-                    (nb >= 2 * SPD_SB_BLOCKS && !(flags & SPD_FACTOR_BLOCK_SWEEPS)
+                    (sb_sweeps((int)nb) && !(flags & SPD_FACTOR_BLOCK_SWEEPS)
                          ? sizeof(float) * (size_t)ceil_div((long)nb, SPD_SB_BLOCKS) * SPD_SB_BLOCKS * 128 *
                                SPD_SB_BLOCKS * 128
                          : 0);
@@ -523,36 +530,32 @@ spd_status factor_once(spd_handle* h, int n, const double* A, int lda, int prec,
             st = potrf_rec<float>(c, 0, n);
         }
         if (st == SPD_OK && prec != SPD_PREC_FP64) {
-            // per-block inverses and sweep couplings: off the factorisation's
-            // critical path, all blocks at once
-            ProfScope pinv(h, SPD_PHASE_INVERSES, (double)F->nblk128 * 128.0 * 128.0 * 128.0 / 3.0,
-                           (double)F->nblk128 * (8.0 * 16384.0 + 16384.0));
-            ++h->launches, k_block_inverse<<<F->nblk128, 256, block_inverse_smem(), s>>>(F->W, F->ldw, n, F->Dinv32,
-                                                                                        F->LinvT);
-            if (cudaGetLastError() != cudaSuccess) st = set_err(h, SPD_ERR_CUDA, "block inverse launch failed");
-        }
-        if (st == SPD_OK && prec != SPD_PREC_FP64 && !(flags & SPD_FACTOR_BLOCK_SWEEPS) &&
-            F->nblk128 >= 2 * SPD_SB_BLOCKS) {
-            // inverses of the diagonal super-blocks for the super-block sweeps
-            F->sbb = SPD_SB_BLOCKS;
-            F->nsb = ceil_div(F->nblk128, F->sbb);
-            const size_t S = (size_t)F->sbb * 128;
-            if (cudaMallocAsync(&F->Xsb, sizeof(float) * S * S * F->nsb, s) != cudaSuccess) {
-                cudaGetLastError();
-                F->Xsb = nullptr;  // the 128-block sweeps serve instead
-                F->sbb = F->nsb = 0;
-            } else {
-                static const bool attr = [] {
-                    cudaFuncSetAttribute(k_sb_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sb_inverse_smem());
-                    return true;
-                }();
-                (void)attr;
-                ProfScope pinv(h, SPD_PHASE_INVERSES, (double)F->nsb * S * S * S / 3.0, 4.0 * F->nsb * S * S);
-                ++h->launches, k_sb_inverse<<<dim3(F->sbb * SB_STRIPS, F->nsb), 256, sb_inverse_smem(), s>>>(
-                    F->W, F->ldw, n, F->nblk128, F->LinvT, F->sbb, F->Xsb);
-                if (cudaGetLastError() != cudaSuccess) st = set_err(h, SPD_ERR_CUDA, "super-block inverse launch failed");
+            // inverses of the diagonal blocks and of the diagonal super-blocks (for
+            // the super-block sweeps): off the factorisation's critical path, all
+            // blocks at once
+            if (!(flags & SPD_FACTOR_BLOCK_SWEEPS) && sb_sweeps(F->nblk128)) {
+                F->sbb = SPD_SB_BLOCKS;
+                F->nsb = ceil_div(F->nblk128, F->sbb);
+                const size_t S = (size_t)F->sbb * 128;
+                if (cudaMallocAsync(&F->Xsb, sizeof(float) * S * S * F->nsb, s) != cudaSuccess) {
+                    cudaGetLastError();
+                    F->Xsb = nullptr;  // the 128-block sweeps serve instead
+                    F->sbb = F->nsb = 0;
+                }
             }
+            const double S = (double)F->sbb * 128.0;
+            ProfScope pinv(h, SPD_PHASE_INVERSES, (double)F->nblk128 * 128.0 * 128.0 * 128.0 / 3.0 + F->nsb * S * S * S / 3.0,
+                           (double)F->nblk128 * (8.0 * 16384.0 + 16384.0) + 4.0 * F->nsb * S * S);
+            ++h->launches, k_block_inverse<<<F->nblk128, 256, block_inverse_smem(), s>>>(F->W, F->ldw, n, F->Dinv32,
+                                                                                        F->LinvT, F->Xsb, F->sbb);
+            for (int hh = 128; F->Xsb && hh < F->sbb * 128; hh *= 2) {
+                if (F->nblk128 * 128 <= hh) break;  // one block of this order or less
+                const int th = hh / 64;
+                const dim3 grid(th * th, F->sbb * 64 / hh, F->nsb);
+                ++h->launches, k_sb_product<true><<<grid, 256, 0, s>>>(F->W, F->ldw, n, F->nblk128, F->sbb, F->Xsb, hh);
+                ++h->launches, k_sb_product<false><<<grid, 256, 0, s>>>(F->W, F->ldw, n, F->nblk128, F->sbb, F->Xsb, hh);
+            }
+            if (cudaGetLastError() != cudaSuccess) st = set_err(h, SPD_ERR_CUDA, "block inverse launch failed");
         }
         // the 128-block sweeps' couplings, only where they will run
         if (st == SPD_OK && prec != SPD_PREC_FP64 && !F->Xsb) st = factor_couplings(h, F);

@@ -58,3 +58,24 @@ def test_subnormal_pivot(h, col):
     want = np.eye(n)
     want[col, col] = 2.0 ** -70
     assert np.max(np.abs(L - want) / np.where(want > 0, want, 1.0)) <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("n", [129, 200, 256, 257, 383, 385, 512, 640, 769, 897, 1023, 1024])
+@pytest.mark.parametrize("m", [1, 2, 17])
+def test_one_super_block(h, n, m):
+    """Orders of one super-block: the sweep is the product with its inverse, formed by doubling."""
+    import torch
+    A = W.gram_shifted(n, seed=n, shift=0.1)
+    At = dev_sym(A)
+    st, F, _ = spd.spd_factor(h, At, "fp32")
+    check(h, st)
+    L, d, _ = factor_L(F)
+    R = torch.from_numpy(W.gaussian_rhs(n, m, 3).T.copy()).to(At.device).t()
+    Z = torch.zeros_like(R)
+    check(h, spd.spd_factor_solve(h, F, R, Z))
+    spd.spd_factor_destroy(F)
+    Lt = np.linalg.inv(L)
+    want = d[:, None] * (Lt.T @ (Lt @ (d[:, None] * R.cpu().numpy())))
+    # float32 products with an explicit float32 inverse: n^1/2 2^-24 times cond(L) squared
+    tol = 8 * n ** 0.5 * 2.0 ** -24 * np.linalg.cond(L) ** 2
+    assert np.linalg.norm(Z.cpu().numpy() - want) <= tol * np.linalg.norm(want)
