@@ -47,7 +47,7 @@ struct spd_handle {
     const int* async_gate = nullptr;
     int* async_epoch_dev = nullptr;
     int async_rel = 0, async_total = 0;
-    void* sb_buf = nullptr;     // super-block sweeps: partial tiles, then two barrier words
+    void* sb_buf = nullptr;     // super-block sweeps: partial tiles and slots, one sweep's result, barrier words
     size_t sb_bytes = 0;
     size_t mem_cap = 0;         // largest device request of one call (0 = no cap): spd_set_memory_cap
 };

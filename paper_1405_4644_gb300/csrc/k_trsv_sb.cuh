@@ -50,6 +50,11 @@ struct SbArgs {
     unsigned long long wait_ns;
     DevStatus* st;
     const int* gate;      // (may be NULL) return at once when *gate == 0
+    // column groups of MC columns swept side by side (blockIdx.y = group): the
+    // columns of all groups from c0 / oc0 on, and the groups' strides of P, P2, bar
+    int mtot;
+    long pstride, p2stride;
+    int barstride;
 };
 
 // Grid-wide barrier: the k-th barrier of a launch waits for k * gridDim.x
@@ -210,6 +215,11 @@ constexpr size_t trsv_sb_smem() {
 // tile index of the pair (p, q), q <= p, in the order (0,0), (1,0), (1,1), ...
 __device__ __forceinline__ int sb_tri(int p, int q) { return p * (p + 1) / 2 + q; }
 
+// Columns go in groups of MC, up to SB_GROUPS of them side by side in one launch,
+// each on its share of the CTAs with barriers of its own: a sweep is mostly its
+// chain of grid-wide phases, which the groups then run at the same time, and they
+// read the same tiles of L within a short time of each other.
+constexpr int SB_GROUPS = 4;
 template <int MC, bool FWD>
 __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -220,6 +230,15 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
     const int tid = threadIdx.x;
     const int tq = tid >> 3, ts = tid & 7;
     const int G = gridDim.x, g = blockIdx.x;
+    if (gridDim.y > 1) {
+        const int y = blockIdx.y;
+        a.c0 += y * MC;
+        a.oc0 += y * MC;
+        a.mc = min(MC, a.mtot - y * MC);
+        a.P += y * a.pstride;
+        a.P2 += y * a.p2stride;
+        a.bar += y * a.barstride;
+    }
     if (tid == 0) s_abort = 0;
     __syncthreads();
     int nbar = 0;

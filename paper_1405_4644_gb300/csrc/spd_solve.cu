@@ -470,30 +470,32 @@ namespace {
 // One forward and one backward super-block sweep of columns [c0, c0 + mc)
 // (k_trsv_sb.cuh): the barrier words are cleared before each launch (a
 // stream-ordered memset, so that a captured graph clears them on replay).
-// The scratch (partial tiles, partial slots, barrier words) is sized once
-// per handle; the first call on a handle must not be captured.
+// The scratch (partial tiles, partial slots, barrier words) is sized for
+// SB_GROUPS groups of 16 columns whatever this call has, so that it grows with the
+// order alone; the first call on a handle must not be captured.  mc columns: groups
+// of MC, side by side.
 template <int MC>
 spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, int c0, int mc) {
     const size_t smem = trsv_sb_smem<MC>();
     auto fwd = k_trsv_sb<MC, true>;
     auto bwd = k_trsv_sb<MC, false>;
-    static const int per_sm = [&] {  // once per instantiation, thread-safe
+    static const bool attr = [&] {  // once per instantiation, thread-safe
         cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         cudaFuncSetAttribute(bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        int a = 0, b = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, fwd, 256, smem);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, bwd, 256, smem);
-        return std::max(1, std::min(a, b));
+        return true;
     }();
+    (void)attr;
     const size_t ntile = (size_t)F->sbb * (F->sbb + 1) / 2;
-    // every SM streams the panel updates: one CTA per resident slot
-    const int G = std::min(per_sm * h->sms, TV_SLOTS);
-    const size_t pbytes = (size_t)round_up((long)(sizeof(float) * ntile * 128 * 16), 256);
-    const size_t p2bytes = (size_t)round_up((long)(sizeof(float) * 2 * (size_t)G * 128 * 16), 256);
-    const size_t zbytes = (size_t)round_up((long)(sizeof(float) * (size_t)n * 16), 256);
-    const int nbar = 2 + F->nsb * F->sbb;  // barrier words, then the block-row tile counts
-    const size_t bbytes = (size_t)round_up((long)(sizeof(int) * nbar), 256);
-    const size_t need = pbytes + p2bytes + zbytes + bbytes;
+    // every SM streams the panel updates: one CTA each (its registers fill the SM),
+    // shared out among the column groups
+    const int ng = ceil_div(mc, MC), slots = std::max(SB_GROUPS, std::min(h->sms, TV_SLOTS));
+    const int G = slots / ng;
+    const size_t pbytes = sizeof(float) * ntile * 128 * 16;                // per group
+    const size_t p2bytes = sizeof(float) * 2 * (size_t)G * 128 * MC;       // per group
+    const size_t p2all = sizeof(float) * 2 * (size_t)slots * 128 * 16;  // ng G <= slots
+    const size_t zbytes = (size_t)round_up((long)(sizeof(float) * (size_t)n * 16 * SB_GROUPS), 256);
+    const int nbar = 2 + F->nsb * F->sbb;  // per group: barrier words, then the block-row tile counts
+    const size_t need = SB_GROUPS * pbytes + p2all + zbytes + sizeof(int) * (size_t)nbar * SB_GROUPS;
     if (h->sb_bytes < need) {
         if (h->sb_buf) {
             CUDA_TRY(h, cudaStreamSynchronize(h->stream));
@@ -506,35 +508,67 @@ spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, i
     }
     char* base = static_cast<char*>(h->sb_buf);
     float* P = reinterpret_cast<float*>(base);
-    float* P2 = reinterpret_cast<float*>(base + pbytes);
-    float* Z = reinterpret_cast<float*>(base + pbytes + p2bytes);  // the forward sweep's result
-    int* bar = reinterpret_cast<int*>(base + pbytes + p2bytes + zbytes);
+    float* P2 = reinterpret_cast<float*>(base + SB_GROUPS * pbytes);
+    float* Z = reinterpret_cast<float*>(base + SB_GROUPS * pbytes + p2all);  // the forward sweep's result
+    int* bar = reinterpret_cast<int*>(base + SB_GROUPS * pbytes + p2all + zbytes);
     for (int dir = 0; dir < 2; ++dir) {
         // forward: Y (columns c0..) reduced, result to Z; backward: Z reduced, result to Y
         SbArgs a{F->W, F->ldw, n, F->nblk128, F->Xsb, F->sbb * 128, F->sbb, F->nsb,
                  dir == 0 ? Y : Z, dir == 0 ? c0 : 0, mc, dir == 0 ? Z : Y, dir == 0 ? 0 : c0, P, P2, bar,
-                 h->wait_ns, h->dst, h->async_on ? h->async_gate : nullptr};
+                 h->wait_ns, h->dst, h->async_on ? h->async_gate : nullptr,
+                 mc, (long)(pbytes / sizeof(float)), (long)(p2bytes / sizeof(float)), nbar};
         void* args[] = {&a};
-        CUDA_TRY(h, cudaMemsetAsync(bar, 0, sizeof(int) * nbar, h->stream));
+        CUDA_TRY(h, cudaMemsetAsync(bar, 0, sizeof(int) * nbar * ng, h->stream));
         ++h->launches;
-        CUDA_TRY(h, coop_launch(dir == 0 ? (const void*)fwd : (const void*)bwd, dim3(G), dim3(256), args, smem,
+        CUDA_TRY(h, coop_launch(dir == 0 ? (const void*)fwd : (const void*)bwd, dim3(G, ng), dim3(256), args, smem,
                                 h->stream));
     }
     return SPD_OK;
 }
 
+// Columns per group and per pass of the super-block sweeps for m right-hand sides:
+// groups of w columns, up to SB_GROUPS side by side.  A pass of g groups takes
+// about c + a n + (b + (g - 1) d) n^2 us, n in thousands: the chain of phases (its
+// links grow with w), a group's share of the panel products, and what another
+// group adds (it reads the panel again and has its own products).  Coefficients
+// fitted to sweep pairs at n = 2100, 8191 and 16384 (one group of 16: 158, 501,
+// 1225 us; of 8: 113, 349, 830; two groups of 8: 115, 418, 1213; four of 16: 177,
+// 924, 3075 against 557, 1938, 4715 one after another).
+void sb_groups(int n, int m, int* w_out, int* per_out) {
+    static const struct {
+        int w;
+        double c, a, b, d;
+    } T[] = {{1, 35, 27.2, 0.48, 0.60}, {2, 37, 27.3, 0.62, 0.75}, {4, 36, 28.3, 0.78, 0.95},
+             {8, 38, 34.5, 0.98, 1.30}, {16, 52, 47.6, 1.66, 2.20}};
+    const double x = n * 1e-3;
+    double best = INFINITY;
+    for (const auto& t : T) {
+        const int total = ceil_div(m, t.w), passes = ceil_div(total, SB_GROUPS), g = ceil_div(total, passes);
+        const double us = passes * (t.c + t.a * x + (t.b + (g - 1) * t.d) * x * x);
+        if (us < best) {
+            best = us;
+            *w_out = t.w;
+            *per_out = t.w * g;
+        }
+    }
+}
+
 // Y <- (L L^T)^{-1} Y for a float32 factor (n x m, ld n).
 spd_status lp_sweeps32(spd_handle* h, const spd_factor_t* F, int n, int m, float* Y) {
     ProfScope ps(h, SPD_PHASE_SOLVE, 2.0 * n * (double)n * m, 4.0 * n * (double)n);
-    for (int c0 = 0; c0 < m && F->Xsb; c0 += 16) {  // super-block sweeps
-        const int mc = std::min(16, m - c0);
-        spd_status st;
-        if (mc == 1) st = trsv_sb_pass<1>(h, F, Y, n, c0, mc);
-        else if (mc <= 2) st = trsv_sb_pass<2>(h, F, Y, n, c0, mc);
-        else if (mc <= 4) st = trsv_sb_pass<4>(h, F, Y, n, c0, mc);
-        else if (mc <= 8) st = trsv_sb_pass<8>(h, F, Y, n, c0, mc);
-        else st = trsv_sb_pass<16>(h, F, Y, n, c0, mc);
-        if (st != SPD_OK) return st;
+    if (F->Xsb) {  // super-block sweeps
+        int mcw, per;
+        sb_groups(n, m, &mcw, &per);
+        for (int c0 = 0; c0 < m; c0 += per) {
+            const int mc = std::min(per, m - c0);
+            spd_status st;
+            if (mcw == 1) st = trsv_sb_pass<1>(h, F, Y, n, c0, mc);
+            else if (mcw == 2) st = trsv_sb_pass<2>(h, F, Y, n, c0, mc);
+            else if (mcw == 4) st = trsv_sb_pass<4>(h, F, Y, n, c0, mc);
+            else if (mcw == 8) st = trsv_sb_pass<8>(h, F, Y, n, c0, mc);
+            else st = trsv_sb_pass<16>(h, F, Y, n, c0, mc);
+            if (st != SPD_OK) return st;
+        }
     }
     for (int c0 = 0; c0 < m && !F->Xsb; c0 += 16) {
         const int mc = std::min(16, m - c0);
