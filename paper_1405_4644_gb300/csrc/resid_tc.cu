@@ -8,7 +8,7 @@
 //   k_tcr_digits_a  64x64 tiles of column-major A transposed through shared
 //                   memory into ten row-major digit planes.
 //   k_tcr_digits_x  column exponent and ten digit planes of every column of X.
-//   k_tcr_mma       persistent: work items (column block, row block, K chunk)
+//   k_tcr_mma       persistent: work items (column blocks, row block, K chunk)
 //                   in contiguous ranges per CTA.  Warp 0 feeds A and X digit
 //                   tiles by TMA; warp 1 issues tcgen05.mma (M 128, K 16,
 //                   N 16 (10 - p) for A's digit plane p against X's planes
@@ -29,16 +29,18 @@ namespace {
 constexpr int TCR_S = 10;           // digits per value (70 bits below 2^e)
 constexpr int TCR_TMAX = 11;        // products of digits p, q (1-based) with p + q <= TCR_TMAX
 constexpr int TCR_NG = TCR_TMAX - 1;  // groups t = 2..TCR_TMAX
-constexpr int TCR_BK = 64;          // K per tile: 128 bytes of bf16
-constexpr int TCR_KC = 1;           // K tiles per exactly accumulated chunk: 10 x 64^2 x 64 <= 2^22
-constexpr int TCR_NA = 10;          // A ring: one digit plane tile (128 x 64) per stage
-constexpr int TCR_NX = 2;           // X ring: ten plane tiles (16 x 64) per stage
+constexpr int TCR_BK = 64;          // K per tile: 128 bytes of bf16; exactly accumulated: 10 x 64^2 x 64 <= 2^22
+// by CB, the 16-column blocks that share an A tile:
+constexpr int tcr_na(int CB) { return CB == 1 ? 10 : 8; }  // A ring: one digit plane tile (128 x 64) per stage
+constexpr int tcr_nx(int CB) { return 2 * CB; }            // X ring: ten plane tiles (16 x 64) per stage
+constexpr int tcr_threads(int CB) { return 64 + 256 * CB; }
 constexpr int TCR_A_BYTES = 128 * 128;
 constexpr int TCR_XP_BYTES = 16 * 128;
 constexpr int TCR_X_BYTES = TCR_S * TCR_XP_BYTES;
-constexpr int TCR_THREADS = 320;
 constexpr uint32_t TCR_TMEM_COLS = 512;  // two buffers of 10 groups x 16 columns
-constexpr size_t TCR_SMEM = (size_t)TCR_NA * TCR_A_BYTES + (size_t)TCR_NX * TCR_X_BYTES + 1024 + 256;
+constexpr size_t tcr_smem(int CB) {
+    return (size_t)tcr_na(CB) * TCR_A_BYTES + (size_t)tcr_nx(CB) * TCR_X_BYTES + 1024 + 256;
+}
 constexpr uint64_t TCR_WAIT_NS = 2000000000ull;
 constexpr int TCR_RS = 64;          // column splits of the row scan
 constexpr int TCR_NONFINITE = INT_MIN;
@@ -320,27 +322,39 @@ __global__ void __launch_bounds__(256) k_tcr_digits_x(const double* __restrict__
 // ---------------------------------------------------------------------------
 // the digit products
 // ---------------------------------------------------------------------------
-// Work item t: g = t / Nkc (segment: column block g / RB, row block g % RB)
-// and K tile t % Nkc.  CTA b takes items [b T / G, (b+1) T / G).  At the end
-// of each segment, and every TCR_FLUSH items, its 32-bit sums (at most
+// Work item t: g = t / Nkc (segment: column group g / RB of CB column blocks, row
+// block g % RB) and K tile t % Nkc.  CTA b takes items [b T / G, (b+1) T / G).  At
+// the end of each segment, and every TCR_FLUSH items, its 32-bit sums (at most
 // TCR_FLUSH x 2^21.3 in magnitude) are added to the 64-bit integer sums
-// part[g][group][column][row] (integer atomics: the order does not matter).
+// part[column block RB + row block][group][column][row] (integer atomics: the order
+// does not matter).
+// The kernel is bound by the stream of A's digit planes (20 bytes an entry, from HBM
+// once they exceed L2), not by the products: 160 KB a tile are 7300 cycles of an SM's
+// share of the bandwidth, the 880 columns of one column block's products 1760 cycles
+// of its tensor core.  So for more than 16 columns two column blocks (CB = 2) are
+// multiplied with each A tile while it is in shared memory: each has one of the two
+// accumulator buffers and eight read-out warps (with CB = 1 the buffers alternate
+// from tile to tile).  The wait for the read-out before the next tile's first product
+// costs the tensor core, not the stream of A, which the ring covers.
 constexpr int TCR_FLUSH = 256;
-__global__ void __launch_bounds__(TCR_THREADS, 1)
+template <int CB>
+__global__ void __launch_bounds__(tcr_threads(CB), 1)
     k_tcr_mma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapX, int n, int RB,
-              int Nkc, long T, unsigned long long* __restrict__ part, DevStatus* st, const int* __restrict__ gate) {
+              int NCB, int Nkc, long T, unsigned long long* __restrict__ part, DevStatus* st,
+              const int* __restrict__ gate) {
     if (gate && *gate == 0) return;  // before any barrier or tensor memory
+    constexpr int NA = tcr_na(CB), NX = tcr_nx(CB);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
     unsigned char* sA = base;
-    unsigned char* sX = base + TCR_NA * TCR_A_BYTES;
-    uint64_t* afull = reinterpret_cast<uint64_t*>(sX + TCR_NX * TCR_X_BYTES);
-    uint64_t* aempty = afull + TCR_NA;
-    uint64_t* xfull = aempty + TCR_NA;
-    uint64_t* xempty = xfull + TCR_NX;
-    uint64_t* tfull = xempty + TCR_NX;  // [2] chunk accumulated (tcgen05.commit)
-    uint64_t* tfree = tfull + 2;        // [2] chunk read out (8 epilogue warps)
+    unsigned char* sX = base + NA * TCR_A_BYTES;
+    uint64_t* afull = reinterpret_cast<uint64_t*>(sX + NX * TCR_X_BYTES);
+    uint64_t* aempty = afull + NA;
+    uint64_t* xfull = aempty + NA;
+    uint64_t* xempty = xfull + NX;
+    uint64_t* tfull = xempty + NX;  // [2] chunk accumulated (tcgen05.commit)
+    uint64_t* tfree = tfull + 2;    // [2] chunk read out (8 epilogue warps)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfree + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -350,11 +364,11 @@ __global__ void __launch_bounds__(TCR_THREADS, 1)
     const int nitems = (int)(t1 - t0);
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < TCR_NA; ++s) {
+        for (int s = 0; s < NA; ++s) {
             tc::mbar_init(&afull[s], 1);
             tc::mbar_init(&aempty[s], 1);
         }
-        for (int s = 0; s < TCR_NX; ++s) {
+        for (int s = 0; s < NX; ++s) {
             tc::mbar_init(&xfull[s], 1);
             tc::mbar_init(&xempty[s], 1);
         }
@@ -383,33 +397,29 @@ __global__ void __launch_bounds__(TCR_THREADS, 1)
             for (int u = 0; u < nitems && ok; ++u) {
                 const long t = t0 + u;
                 const long g = t / Nkc;
-                const int kc = (int)(t - g * Nkc);
-                const int cb = (int)(g / RB), rb = (int)(g - (long)cb * RB);
-                for (int kt = 0; kt < TCR_KC && ok; ++kt) {
-                    const int k = (kc * TCR_KC + kt) * TCR_BK;
-                    if (k >= n) break;
-                    {
-                        const int s = ix % TCR_NX;
-                        if (ix >= TCR_NX && !tc::mbar_wait(&xempty[s], ((ix / TCR_NX) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
-                            ok = false;
-                            break;
-                        }
-                        tc::mbar_arrive_expect_tx(&xfull[s], TCR_X_BYTES);
+                const int k = (int)(t - g * Nkc) * TCR_BK;
+                const int cb = (int)(g / RB) * CB, rb = (int)(g % RB);
+                for (int c = 0; c < CB && cb + c < NCB; ++c) {
+                    const int s = ix % NX;
+                    if (ix >= NX && !tc::mbar_wait(&xempty[s], ((ix / NX) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::mbar_arrive_expect_tx(&xfull[s], TCR_X_BYTES);
 #pragma unroll
-                        for (int q = 0; q < TCR_S; ++q)
-                            tc::tma_load_3d(sX + s * TCR_X_BYTES + q * TCR_XP_BYTES, &mapX, k, cb * 16, q, &xfull[s]);
-                        ++ix;
+                    for (int q = 0; q < TCR_S; ++q)
+                        tc::tma_load_3d(sX + s * TCR_X_BYTES + q * TCR_XP_BYTES, &mapX, k, (cb + c) * 16, q, &xfull[s]);
+                    ++ix;
+                }
+                for (int p = 0; p < TCR_S && ok; ++p) {
+                    const int s = ia % NA;
+                    if (ia >= NA && !tc::mbar_wait(&aempty[s], ((ia / NA) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
+                        ok = false;
+                        break;
                     }
-                    for (int p = 0; p < TCR_S; ++p) {
-                        const int s = ia % TCR_NA;
-                        if (ia >= TCR_NA && !tc::mbar_wait(&aempty[s], ((ia / TCR_NA) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
-                            ok = false;
-                            break;
-                        }
-                        tc::mbar_arrive_expect_tx(&afull[s], TCR_A_BYTES);
-                        tc::tma_load_3d(sA + s * TCR_A_BYTES, &mapA, k, rb * 128, p, &afull[s]);
-                        ++ia;
-                    }
+                    tc::mbar_arrive_expect_tx(&afull[s], TCR_A_BYTES);
+                    tc::tma_load_3d(sA + s * TCR_A_BYTES, &mapA, k, rb * 128, p, &afull[s]);
+                    ++ia;
                 }
             }
         }
@@ -419,89 +429,100 @@ __global__ void __launch_bounds__(TCR_THREADS, 1)
             int ia = 0, ix = 0;
             bool ok = true;
             for (int u = 0; u < nitems && ok; ++u) {
-                const int buf = u & 1;
-                if (u >= 2 && !tc::mbar_wait(&tfree[buf], ((u >> 1) - 1) & 1u, abort_flag, TCR_WAIT_NS)) break;
-                tc::fence_after_sync();
-                const uint32_t dbase = tmem + (uint32_t)(buf * TCR_NG * 16);
-                const long t = t0 + u;
-                const int kc = (int)(t % Nkc);
-                for (int kt = 0; kt < TCR_KC && ok; ++kt) {
-                    const int k = (kc * TCR_KC + kt) * TCR_BK;
-                    if (k >= n) break;
-                    const int sx = ix % TCR_NX;
-                    if (!tc::mbar_wait(&xfull[sx], (ix / TCR_NX) & 1u, abort_flag, TCR_WAIT_NS)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
+                const int cb = (int)((t0 + u) / Nkc / RB) * CB, nb = CB == 1 ? 1 : min(CB, NCB - cb);
+                const int buf0 = CB == 1 ? (u & 1) : 0;
+                uint64_t bd[CB];
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    if (c >= nb || !ok) break;
+                    const int buf = buf0 + c, sx = (ix + c) % NX;
+                    const int uses = CB == 1 ? u >> 1 : u;  // a missing block stays missing
+                    if (uses && !tc::mbar_wait(&tfree[buf], (uses - 1) & 1u, abort_flag, TCR_WAIT_NS)) ok = false;
+                    if (ok && !tc::mbar_wait(&xfull[sx], ((ix + c) / NX) & 1u, abort_flag, TCR_WAIT_NS)) ok = false;
                     // the X stage holds planes q = 0..9 as one K-major tile of
                     // 160 rows (16 per plane); its first 16 (10 - p) rows
                     // against A plane p give the products (p, q), q <= 9 - p, as
                     // one N = 16 (10 - p) instruction whose columns are the
                     // accumulators of groups p .. 9 (group g at columns 16 g)
-                    const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(sX + sx * TCR_X_BYTES));
-                    for (int p = 0; p < TCR_S; ++p) {
-                        const int sa = ia % TCR_NA;
-                        if (!tc::mbar_wait(&afull[sa], (ia / TCR_NA) & 1u, abort_flag, TCR_WAIT_NS)) {
-                            ok = false;
-                            break;
-                        }
-                        tc::fence_after_sync();
-                        const uint64_t ad = tc::sdesc_kmajor_sw128(tc::smem_u32(sA + sa * TCR_A_BYTES));
-                        const uint32_t idesc = tc::idesc_f32acc(1, 128, 16 * (TCR_TMAX - 1 - p));  // bf16 -> f32
-#pragma unroll
-                        for (int kk = 0; kk < TCR_BK / 16; ++kk)  // +32 bytes of K = +2 in the address field
-                            tc::mma<0>(dbase + (uint32_t)(p * 16), ad + 2 * kk, bd + 2 * kk, idesc,
-                                       (kt > 0 || p > 0 || kk > 0) ? 1u : 0u);
-                        tc::mma_commit(&aempty[sa]);
-                        ++ia;
-                    }
-                    if (!ok) break;
-                    tc::mma_commit(&xempty[sx]);
-                    ++ix;
+                    bd[c] = tc::sdesc_kmajor_sw128(tc::smem_u32(sX + sx * TCR_X_BYTES));
                 }
                 if (!ok) break;
-                tc::mma_commit(&tfull[buf]);
+                tc::fence_after_sync();
+                for (int p = 0; p < TCR_S; ++p) {
+                    const int sa = ia % NA;
+                    if (!tc::mbar_wait(&afull[sa], (ia / NA) & 1u, abort_flag, TCR_WAIT_NS)) {
+                        ok = false;
+                        break;
+                    }
+                    tc::fence_after_sync();
+                    const uint64_t ad = tc::sdesc_kmajor_sw128(tc::smem_u32(sA + sa * TCR_A_BYTES));
+                    const uint32_t idesc = tc::idesc_f32acc(1, 128, 16 * (TCR_TMAX - 1 - p));  // bf16 -> f32
+#pragma unroll
+                    for (int c = 0; c < CB; ++c) {
+                        if (c >= nb) break;
+                        const uint32_t dcol = tmem + (uint32_t)((buf0 + c) * TCR_NG * 16 + p * 16);
+#pragma unroll
+                        for (int kk = 0; kk < TCR_BK / 16; ++kk)  // +32 bytes of K = +2 in the address field
+                            tc::mma<0>(dcol, ad + 2 * kk, bd[c] + 2 * kk, idesc, (p > 0 || kk > 0) ? 1u : 0u);
+                    }
+                    tc::mma_commit(&aempty[sa]);
+                    ++ia;
+                }
+                if (!ok) break;
+#pragma unroll
+                for (int c = 0; c < CB; ++c) {
+                    if (c >= nb) break;
+                    tc::mma_commit(&xempty[ix % NX]);
+                    ++ix;
+                    tc::mma_commit(&tfull[buf0 + c]);
+                }
             }
         }
         __syncwarp();
-    } else {  // warps 2..9: chunk read-out, lane quarter warp % 4, columns EW h .. EW h + EW - 1
+    } else {
+        // chunk read-out by eight warps a column block: lane quarter warp % 4,
+        // columns EW h .. EW h + EW - 1
         constexpr int EW = TCR_NG * 16 / 2;  // 80: groups 5 h .. 5 h + 4
-        const int quarter = warp & 3, h = (warp - 2) >> 2;
-        int acc[EW];
+        const int quarter = warp & 3, h = ((warp - 2) >> 2) & 1, c = (warp - 2) >> 3;
+        bool ok = true;
+        for (int u = 0; u < nitems && ok;) {
+            // a run of items of one segment, at most TCR_FLUSH
+            const long g = (t0 + u) / Nkc;
+            const int blk = (int)(g / RB) * CB + c;
+            if (CB > 1 && blk >= NCB) break;  // the last group's missing block
+            const int u0 = u, u1 = (int)min(min((g + 1) * Nkc - t0, (long)nitems), (long)u + TCR_FLUSH);
+            int acc[EW];
 #pragma unroll
-        for (int j = 0; j < EW; ++j) acc[j] = 0;
-        int seg_items = 0;
-        for (int u = 0; u < nitems; ++u) {
-            const int buf = u & 1;
-            bool ok = tc::mbar_wait(&tfull[buf], (u >> 1) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
-            ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
-            if (!ok) break;
-            tc::fence_after_sync();
-            const uint32_t ta = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(buf * TCR_NG * 16 + h * EW);
+            for (int j = 0; j < EW; ++j) acc[j] = 0;
+#pragma unroll 1
+            for (; u < u1; ++u) {
+                const int buf = CB == 1 ? (u & 1) : c;
+                ok = tc::mbar_wait(&tfull[buf], (CB == 1 ? u >> 1 : u) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
+                ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
+                if (!ok) break;
+                tc::fence_after_sync();
+                const uint32_t ta = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(buf * TCR_NG * 16 + h * EW);
 #pragma unroll
-            for (int q = 0; q < EW / 16; ++q) {
-                float v[16];
-                tc::tmem_ld_32x32b_x16(ta + q * 16, v);
+                for (int q = 0; q < EW / 16; ++q) {
+                    float v[16];
+                    tc::tmem_ld_32x32b_x16(ta + q * 16, v);
 #pragma unroll
-                for (int j = 0; j < 16; ++j) acc[q * 16 + j] += __float_as_int(v[j] + TCR_MAGIC);
-            }
-            tc::fence_before_sync();
-            __syncwarp();
-            if (lane == 0) tc::mbar_arrive(&tfree[buf]);
-            ++seg_items;
-            const long t = t0 + u;
-            if (u == nitems - 1 || (t + 1) % Nkc == 0 || seg_items == TCR_FLUSH) {
-                // entry (group 5 h + j / 16, column j % 16, row r) at (h EW + j) 128 + r
-                unsigned long long* out = part + (t / Nkc) * (TCR_NG * 16 * 128) + h * EW * 128 + quarter * 32 + lane;
-                const uint32_t bias = (uint32_t)seg_items * TCR_MAGIC_BITS;
-#pragma unroll
-                for (int j = 0; j < EW; ++j) {
-                    const long long v = (int)((uint32_t)acc[j] - bias);
-                    atomicAdd(out + j * 128, (unsigned long long)v);
-                    acc[j] = 0;
+                    for (int j = 0; j < 16; ++j) acc[q * 16 + j] += __float_as_int(v[j] + TCR_MAGIC);
                 }
-                seg_items = 0;
+                tc::fence_before_sync();
+                __syncwarp();
+                if (lane == 0) tc::mbar_arrive(&tfree[buf]);
+            }
+            if (!ok) break;
+            // entry (group 5 h + j / 16, column j % 16, row r) at (h EW + j) 128 + r
+            unsigned long long* out = part + ((long)blk * RB + g % RB) * (TCR_NG * 16 * 128) + h * EW * 128 + quarter * 32 + lane;
+            const uint32_t bias = (uint32_t)(u1 - u0) * TCR_MAGIC_BITS;
+#pragma unroll
+            for (int j = 0; j < EW; ++j) {
+                // in steps, or the compiler widens all sums before the first atomic (spills)
+                if (j % 8 == 0) __syncwarp();
+                const long long v = (int)((uint32_t)acc[j] - bias);
+                atomicAdd(out + j * 128, (unsigned long long)v);
             }
         }
     }
@@ -635,16 +656,19 @@ bool tcr_map_a64(CUtensorMap* map, const double* A, int n, long lda) {
 }
 
 struct TcrSchedule {
-    int RB, CB, Nkc, G;
+    int RB, CB, Nkc, G, per;
     long T;
 };
+
+// Column blocks per A tile: two from 17 columns on.
 
 TcrSchedule tcr_schedule(spd_handle* h, int n, int m) {
     TcrSchedule s;
     s.RB = ceil_div(n, 128);
     s.CB = ceil_div(m, 16);
-    s.Nkc = ceil_div(n, TCR_BK * TCR_KC);
-    s.T = (long)s.CB * s.RB * s.Nkc;
+    s.Nkc = ceil_div(n, TCR_BK);
+    s.per = m > 16 ? 2 : 1;
+    s.T = (long)ceil_div(s.CB, s.per) * s.RB * s.Nkc;
     s.G = (int)std::min<long>(std::max(1, h->sms), s.T);
     return s;
 }
@@ -679,6 +703,7 @@ spd_status tc_resid_bind(spd_handle* h, TcResidWs* w, int n, int m, const size_t
     w->CB = s.CB;
     w->Nkc = s.Nkc;
     w->G = s.G;
+    w->per = s.per;
     w->T = s.T;
     if (!tcr_map(&w->mapA, w->Ad, TCR_S, n, n, w->ldp, 128) || !tcr_map(&w->mapX, w->Xd, TCR_S, m, n, w->ldp, 16))
         return set_err(h, SPD_ERR_UNSUPPORTED, "tensor-core residual: tensor map encoding failed");
@@ -716,7 +741,8 @@ spd_status tc_resid_prepare(spd_handle* h, TcResidWs* w, const double* A, long l
 spd_status tc_resid_run(spd_handle* h, const TcResidWs* w, const double* B, long ldb, const double* X, long ldx,
                         double* R, long ldr, double* NP, int mode, const int* gate) {
     static const bool attr = [] {  // once per process, thread-safe
-        cudaFuncSetAttribute(k_tcr_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TCR_SMEM);
+        cudaFuncSetAttribute(k_tcr_mma<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcr_smem(1));
+        cudaFuncSetAttribute(k_tcr_mma<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tcr_smem(2));
         return true;
     }();
     (void)attr;
@@ -725,8 +751,13 @@ spd_status tc_resid_run(spd_handle* h, const TcResidWs* w, const double* B, long
     ++(h)->launches, k_tcr_digits_x<<<m, 256, 0, s>>>(X, ldx, n, m, w->xe, w->Xd, w->ldp, gate);
     LAUNCH_CHECK(h);
     CUDA_TRY(h, cudaMemsetAsync(w->part, 0, sizeof(unsigned long long) * (size_t)w->CB * w->RB * TCR_NG * 16 * 128, s));
-    ++(h)->launches, k_tcr_mma<<<w->G, TCR_THREADS, TCR_SMEM, s>>>(w->mapA, w->mapX, n, w->RB, w->Nkc, w->T, w->part,
-                                                                   h->dst, gate);
+    ++h->launches;
+    if (w->per == 2)
+        k_tcr_mma<2><<<w->G, tcr_threads(2), tcr_smem(2), s>>>(w->mapA, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
+                                                               w->part, h->dst, gate);
+    else
+        k_tcr_mma<1><<<w->G, tcr_threads(1), tcr_smem(1), s>>>(w->mapA, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
+                                                               w->part, h->dst, gate);
     LAUNCH_CHECK(h);
     ++(h)->launches, k_tcr_final<<<dim3(ceil_div(n, 256), m), 256, 0, s>>>(
         w->rowmax, w->xe, w->part, n, m, w->RB, mode == 0 ? B : nullptr, ldb, X, ldx, R,

@@ -27,8 +27,8 @@ struct TcResidWs {
     int* xe = nullptr;           // m: column exponents of X (INT_MIN: non-finite)
     unsigned long long* part = nullptr;  // (CB RB) x 10 x 16 x 128: 64-bit integer group sums
     long ldp = 0;
-    int n = 0, m = 0, RS = 1, RB = 0, CB = 0, Nkc = 0, G = 0;
-    long T = 0;                  // work items (column block, row block, K chunk)
+    int n = 0, m = 0, RS = 1, RB = 0, CB = 0, Nkc = 0, G = 0, per = 1;  // per: column blocks per work item
+    long T = 0;                  // work items (column blocks, row block, K chunk)
 };
 
 // Workspace layout for an n x n matrix and m right-hand sides (6 offsets).
