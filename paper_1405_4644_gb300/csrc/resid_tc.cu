@@ -6,18 +6,19 @@
 //   k_tcr_rowscan   bits of max_j |a_ij| per row (atomicMax) and partial row
 //                   sums of |a_ij| for ||A||_inf; A read once, coalesced.
 //   k_tcr_digits_a  64x64 tiles of column-major A transposed through shared
-//                   memory into ten row-major digit planes.
+//                   memory into ten digit planes, tile by tile.
 //   k_tcr_digits_x  column exponent and ten digit planes of every column of X.
 //   k_tcr_mma       persistent: work items (column blocks, row block, K chunk)
 //                   in contiguous ranges per CTA.  Warp 0 feeds A and X digit
-//                   tiles by TMA; warp 1 issues tcgen05.mma (M 128, K 16,
+//                   tiles by bulk copies; warp 1 issues tcgen05.mma (M 128, K 16,
 //                   N 16 (10 - p) for A's digit plane p against X's planes
 //                   0 .. 9 - p stacked) for the 55 digit products with
 //                   p + q <= 11, into ten group accumulators in tensor memory
-//                   (two buffers, one per chunk parity); warps 2..9 move each finished chunk to
-//                   32-bit integer sums and add them to 64-bit integer sums
-//                   at the end of every (row block, column block) segment.
-//   k_tcr_final     combines the groups with their scales in double-double,
+//                   (two buffers); the other warps move each finished chunk
+//                   to 32-bit integer sums and add them to 64-bit integer
+//                   sums at the end of every (row block, column block)
+//                   segment.
+//   k_tcr_final     combines the groups with their scales as a 128-bit integer,
 //                   R = B - AX rounded once, block partial norms.
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
@@ -32,14 +33,13 @@ constexpr int TCR_NG = TCR_TMAX - 1;  // groups t = 2..TCR_TMAX
 constexpr int TCR_BK = 64;          // K per tile: 128 bytes of bf16; exactly accumulated: 10 x 64^2 x 64 <= 2^22
 // by CB, the 16-column blocks that share an A tile:
 constexpr int tcr_na(int CB) { return CB == 1 ? 10 : 8; }  // A ring: one digit plane tile (128 x 64) per stage
-constexpr int tcr_nx(int CB) { return 2 * CB; }            // X ring: ten plane tiles (16 x 64) per stage
+constexpr int TCR_NX = 2;                                  // X ring: ten plane tiles (16 CB x 64) per stage
 constexpr int tcr_threads(int CB) { return 64 + 256 * CB; }
 constexpr int TCR_A_BYTES = 128 * 128;
-constexpr int TCR_XP_BYTES = 16 * 128;
-constexpr int TCR_X_BYTES = TCR_S * TCR_XP_BYTES;
-constexpr uint32_t TCR_TMEM_COLS = 512;  // two buffers of 10 groups x 16 columns
+constexpr int tcr_xp_bytes(int CB) { return 16 * CB * 128; }
+constexpr uint32_t TCR_TMEM_COLS = 512;  // 10 groups x 16 CB columns: two buffers (CB = 1), one (CB = 2)
 constexpr size_t tcr_smem(int CB) {
-    return (size_t)tcr_na(CB) * TCR_A_BYTES + (size_t)tcr_nx(CB) * TCR_X_BYTES + 1024 + 256;
+    return (size_t)tcr_na(CB) * TCR_A_BYTES + (size_t)TCR_NX * TCR_S * tcr_xp_bytes(CB) + 1024 + 256;
 }
 constexpr uint64_t TCR_WAIT_NS = 2000000000ull;
 constexpr int TCR_RS = 64;          // column splits of the row scan
@@ -244,6 +244,17 @@ __global__ void __launch_bounds__(256) k_tcr_rowscan_tma(const __grid_constant__
     }
 }
 
+// Digit planes of A, in the order in which they are read: for each 128-row block and
+// 64-column tile the ten planes of that tile one after another, each a K-major tile
+// of min(128, n - 128 rb) rows of 128 bytes in the 128-byte swizzle.  A work item of
+// k_tcr_mma is then one contiguous stretch of up to 160 KB (row-major planes gave
+// 128-byte pieces a row pitch apart; n = 8191: k_tcr_digits_a 365 -> 350 us,
+// k_tcr_mma 312 -> 308).
+__device__ __forceinline__ int tcr_rows(int n, int rb) { return min(128, n - rb * 128); }
+__device__ __forceinline__ long tcr_tile(int n, long ldp, int rb, int kc) {
+    return TCR_S * (rb * 128 * ldp + (long)kc * tcr_rows(n, rb) * TCR_BK);
+}
+
 // 64 x 64 tile: element (i0 + r, j0 + c) of column-major A goes to
 // tile[r][c] (coalesced along r, odd pitch: conflict-free); warp w then
 // takes rows w, w + 8, ... and lane l the columns 2 l, 2 l + 1, so each
@@ -262,6 +273,9 @@ __global__ void __launch_bounds__(256) k_tcr_digits_a(const double* __restrict__
     }
     __syncthreads();
     const int w = tid >> 5, lane = tid & 31;
+    const int rb = i0 >> 7;
+    const long plane = (long)tcr_rows(n, rb) * (TCR_BK / 2);  // 32-bit words
+    uint32_t* out = reinterpret_cast<uint32_t*>(Ad + tcr_tile(n, ldp, rb, blockIdx.y));
     for (int r = w; r < 64; r += 8) {
         const int i = i0 + r;
         if (i >= n) break;
@@ -269,10 +283,10 @@ __global__ void __launch_bounds__(256) k_tcr_digits_a(const double* __restrict__
         const bool zero = e == TCR_NONFINITE;
         uint32_t pk[TCR_S];
         tcr_digits2(zero ? 0.0 : tile[r][2 * lane], zero ? 0.0 : tile[r][2 * lane + 1], zero ? 0 : e, pk);
-        // ldp is a multiple of 64, so the tile's columns are inside the row pitch
-        uint32_t* dst = reinterpret_cast<uint32_t*>(Ad + (long)i * ldp + j0) + lane;
+        // 16-byte chunk c of row r is at chunk c ^ (r % 8)
+        uint32_t* dst = out + (i & 127) * (TCR_BK / 2) + (((lane >> 2) ^ (r & 7)) << 2) + (lane & 3);
 #pragma unroll
-        for (int p = 0; p < TCR_S; ++p) dst[(long)p * n * ldp / 2] = pk[p];
+        for (int p = 0; p < TCR_S; ++p) dst[p * plane] = pk[p];
     }
 }
 
@@ -329,32 +343,38 @@ __global__ void __launch_bounds__(256) k_tcr_digits_x(const double* __restrict__
 // part[column block RB + row block][group][column][row] (integer atomics: the order
 // does not matter).
 // The kernel is bound by the stream of A's digit planes (20 bytes an entry, from HBM
-// once they exceed L2), not by the products: 160 KB a tile are 7300 cycles of an SM's
-// share of the bandwidth, the 880 columns of one column block's products 1760 cycles
-// of its tensor core.  So for more than 16 columns two column blocks (CB = 2) are
-// multiplied with each A tile while it is in shared memory: each has one of the two
-// accumulator buffers and eight read-out warps (with CB = 1 the buffers alternate
-// from tile to tile).  The wait for the read-out before the next tile's first product
-// costs the tensor core, not the stream of A, which the ring covers.
+// once they exceed L2): 160 KB a tile are 7300 cycles of an SM's share of the
+// bandwidth.  So for more than 16 columns two column blocks (CB = 2) are multiplied
+// with each A tile while it is in shared memory, as one block of 32 columns: an
+// instruction costs at least about 128 cycles here whatever its N (one block's 40
+// instructions a tile hide behind the stream, two blocks' 80 do not), so the 320 and
+// 288 columns of p = 0, 1 are split in two and the others go as one (n = 8191 / 16384,
+// m = 32: one block at a time 373 / 1440 us, two with instructions of their own
+// 308 / 1150, as one 259 / 956; the planes' stream alone 197 / 790).  With
+// one accumulator buffer of 320 columns, the wait for the read-out before the next
+// tile's first product costs the tensor core, not the stream of A, which the ring
+// covers.
 constexpr int TCR_FLUSH = 256;
 template <int CB>
 __global__ void __launch_bounds__(tcr_threads(CB), 1)
-    k_tcr_mma(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapX, int n, int RB,
+    k_tcr_mma(const uint16_t* __restrict__ Ad, long ldp, const __grid_constant__ CUtensorMap mapX, int n, int RB,
               int NCB, int Nkc, long T, unsigned long long* __restrict__ part, DevStatus* st,
               const int* __restrict__ gate) {
     if (gate && *gate == 0) return;  // before any barrier or tensor memory
-    constexpr int NA = tcr_na(CB), NX = tcr_nx(CB);
+    constexpr int NA = tcr_na(CB), NX = TCR_NX, W = 16 * CB;
+    constexpr int NB = CB == 1 ? 2 : 1;  // accumulator buffers
+    constexpr int XP = tcr_xp_bytes(CB), XB = TCR_S * XP;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                            ~static_cast<uintptr_t>(1023));
     unsigned char* sA = base;
     unsigned char* sX = base + NA * TCR_A_BYTES;
-    uint64_t* afull = reinterpret_cast<uint64_t*>(sX + NX * TCR_X_BYTES);
+    uint64_t* afull = reinterpret_cast<uint64_t*>(sX + NX * XB);
     uint64_t* aempty = afull + NA;
     uint64_t* xfull = aempty + NA;
     uint64_t* xempty = xfull + NX;
     uint64_t* tfull = xempty + NX;  // [2] chunk accumulated (tcgen05.commit)
-    uint64_t* tfree = tfull + 2;    // [2] chunk read out (8 epilogue warps)
+    uint64_t* tfree = tfull + 2;    // [2] chunk read out (8 CB epilogue warps)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfree + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -374,11 +394,10 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
         }
         for (int s = 0; s < 2; ++s) {
             tc::mbar_init(&tfull[s], 1);
-            tc::mbar_init(&tfree[s], 8);
+            tc::mbar_init(&tfree[s], 8 * CB);
         }
         *abort_flag = 0;
         tc::fence_barrier_init();
-        tc::prefetch_tmap(&mapA);
         tc::prefetch_tmap(&mapX);
     }
     if (warp == 1) {
@@ -392,33 +411,30 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
 
     if (warp == 0) {
         if (lane == 0) {  // TMA producer
-            int ia = 0, ix = 0;
+            int ia = 0;
             bool ok = true;
             for (int u = 0; u < nitems && ok; ++u) {
                 const long t = t0 + u;
                 const long g = t / Nkc;
-                const int k = (int)(t - g * Nkc) * TCR_BK;
-                const int cb = (int)(g / RB) * CB, rb = (int)(g % RB);
-                for (int c = 0; c < CB && cb + c < NCB; ++c) {
-                    const int s = ix % NX;
-                    if (ix >= NX && !tc::mbar_wait(&xempty[s], ((ix / NX) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::mbar_arrive_expect_tx(&xfull[s], TCR_X_BYTES);
+                const int kc = (int)(t - g * Nkc), k = kc * TCR_BK;
+                const int cg = (int)(g / RB), rb = (int)(g % RB);
+                const uint16_t* a = Ad + tcr_tile(n, ldp, rb, kc);
+                const int sx = u % NX;
+                if (u >= NX && !tc::mbar_wait(&xempty[sx], ((u / NX) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) break;
+                tc::mbar_arrive_expect_tx(&xfull[sx], XB);
 #pragma unroll
-                    for (int q = 0; q < TCR_S; ++q)
-                        tc::tma_load_3d(sX + s * TCR_X_BYTES + q * TCR_XP_BYTES, &mapX, k, (cb + c) * 16, q, &xfull[s]);
-                    ++ix;
-                }
+                for (int q = 0; q < TCR_S; ++q)
+                    tc::tma_load_3d(sX + sx * XB + q * XP, &mapX, k, cg * W, q, &xfull[sx]);
                 for (int p = 0; p < TCR_S && ok; ++p) {
                     const int s = ia % NA;
                     if (ia >= NA && !tc::mbar_wait(&aempty[s], ((ia / NA) & 1u) ^ 1u, abort_flag, TCR_WAIT_NS)) {
                         ok = false;
                         break;
                     }
-                    tc::mbar_arrive_expect_tx(&afull[s], TCR_A_BYTES);
-                    tc::tma_load_3d(sA + s * TCR_A_BYTES, &mapA, k, rb * 128, p, &afull[s]);
+                    // rows past n keep what the stage held: they reach only their own, unread, sums
+                    const uint32_t bytes = (uint32_t)tcr_rows(n, rb) * 128;
+                    tc::mbar_arrive_expect_tx(&afull[s], bytes);
+                    tc::bulk_g2s(sA + s * TCR_A_BYTES, a + (long)p * (bytes / 2), bytes, &afull[s]);
                     ++ia;
                 }
             }
@@ -426,28 +442,20 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
         __syncwarp();
     } else if (warp == 1) {
         if (lane == 0) {  // MMA issuer
-            int ia = 0, ix = 0;
+            int ia = 0;
             bool ok = true;
             for (int u = 0; u < nitems && ok; ++u) {
-                const int cb = (int)((t0 + u) / Nkc / RB) * CB, nb = CB == 1 ? 1 : min(CB, NCB - cb);
-                const int buf0 = CB == 1 ? (u & 1) : 0;
-                uint64_t bd[CB];
-#pragma unroll
-                for (int c = 0; c < CB; ++c) {
-                    if (c >= nb || !ok) break;
-                    const int buf = buf0 + c, sx = (ix + c) % NX;
-                    const int uses = CB == 1 ? u >> 1 : u;  // a missing block stays missing
-                    if (uses && !tc::mbar_wait(&tfree[buf], (uses - 1) & 1u, abort_flag, TCR_WAIT_NS)) ok = false;
-                    if (ok && !tc::mbar_wait(&xfull[sx], ((ix + c) / NX) & 1u, abort_flag, TCR_WAIT_NS)) ok = false;
-                    // the X stage holds planes q = 0..9 as one K-major tile of
-                    // 160 rows (16 per plane); its first 16 (10 - p) rows
-                    // against A plane p give the products (p, q), q <= 9 - p, as
-                    // one N = 16 (10 - p) instruction whose columns are the
-                    // accumulators of groups p .. 9 (group g at columns 16 g)
-                    bd[c] = tc::sdesc_kmajor_sw128(tc::smem_u32(sX + sx * TCR_X_BYTES));
-                }
-                if (!ok) break;
+                const int buf = u % NB, sx = u % NX;
+                if (u >= NB && !tc::mbar_wait(&tfree[buf], (u / NB - 1) & 1u, abort_flag, TCR_WAIT_NS)) break;
+                if (!tc::mbar_wait(&xfull[sx], (u / NX) & 1u, abort_flag, TCR_WAIT_NS)) break;
                 tc::fence_after_sync();
+                const uint32_t dbase = tmem + (uint32_t)(buf * TCR_NG * W);
+                // the X stage holds planes q = 0..9 as one K-major tile of 10 W
+                // rows (W per plane); its first W (10 - p) rows against A
+                // plane p give the products (p, q), q <= 9 - p, as instructions
+                // of N = W (10 - p) in all, whose columns are the accumulators
+                // of groups p .. 9 (group g at columns W g)
+                const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(sX + sx * XB));
                 for (int p = 0; p < TCR_S; ++p) {
                     const int sa = ia % NA;
                     if (!tc::mbar_wait(&afull[sa], (ia / NA) & 1u, abort_flag, TCR_WAIT_NS)) {
@@ -456,52 +464,44 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
                     }
                     tc::fence_after_sync();
                     const uint64_t ad = tc::sdesc_kmajor_sw128(tc::smem_u32(sA + sa * TCR_A_BYTES));
-                    const uint32_t idesc = tc::idesc_f32acc(1, 128, 16 * (TCR_TMAX - 1 - p));  // bf16 -> f32
-#pragma unroll
-                    for (int c = 0; c < CB; ++c) {
-                        if (c >= nb) break;
-                        const uint32_t dcol = tmem + (uint32_t)((buf0 + c) * TCR_NG * 16 + p * 16);
+                    const int cols = W * (TCR_S - p), parts = cols > 256 ? 2 : 1, N = cols / parts;
+                    const uint32_t idesc = tc::idesc_f32acc(1, 128, N);  // bf16 -> f32
+                    for (int v = 0; v < parts; ++v) {
+                        const uint32_t dcol = dbase + (uint32_t)(p * W + v * N);
+                        const uint64_t bv = bd + (uint64_t)(v * N * 128 >> 4);
 #pragma unroll
                         for (int kk = 0; kk < TCR_BK / 16; ++kk)  // +32 bytes of K = +2 in the address field
-                            tc::mma<0>(dcol, ad + 2 * kk, bd[c] + 2 * kk, idesc, (p > 0 || kk > 0) ? 1u : 0u);
+                            tc::mma<0>(dcol, ad + 2 * kk, bv + 2 * kk, idesc, (p > 0 || kk > 0) ? 1u : 0u);
                     }
                     tc::mma_commit(&aempty[sa]);
                     ++ia;
                 }
                 if (!ok) break;
-#pragma unroll
-                for (int c = 0; c < CB; ++c) {
-                    if (c >= nb) break;
-                    tc::mma_commit(&xempty[ix % NX]);
-                    ++ix;
-                    tc::mma_commit(&tfull[buf0 + c]);
-                }
+                tc::mma_commit(&xempty[sx]);
+                tc::mma_commit(&tfull[buf]);
             }
         }
         __syncwarp();
     } else {
-        // chunk read-out by eight warps a column block: lane quarter warp % 4,
-        // columns EW h .. EW h + EW - 1
-        constexpr int EW = TCR_NG * 16 / 2;  // 80: groups 5 h .. 5 h + 4
-        const int quarter = warp & 3, h = ((warp - 2) >> 2) & 1, c = (warp - 2) >> 3;
+        // chunk read-out: lane quarter warp % 4, columns EW h .. EW h + EW - 1
+        constexpr int EW = TCR_NG * 16 / 2;  // 80
+        const int quarter = warp & 3, h = (warp - 2) >> 2;
         bool ok = true;
         for (int u = 0; u < nitems && ok;) {
             // a run of items of one segment, at most TCR_FLUSH
             const long g = (t0 + u) / Nkc;
-            const int blk = (int)(g / RB) * CB + c;
-            if (CB > 1 && blk >= NCB) break;  // the last group's missing block
             const int u0 = u, u1 = (int)min(min((g + 1) * Nkc - t0, (long)nitems), (long)u + TCR_FLUSH);
             int acc[EW];
 #pragma unroll
             for (int j = 0; j < EW; ++j) acc[j] = 0;
 #pragma unroll 1
             for (; u < u1; ++u) {
-                const int buf = CB == 1 ? (u & 1) : c;
-                ok = tc::mbar_wait(&tfull[buf], (CB == 1 ? u >> 1 : u) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
+                const int buf = u % NB;
+                ok = tc::mbar_wait(&tfull[buf], (u / NB) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
                 ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
                 if (!ok) break;
                 tc::fence_after_sync();
-                const uint32_t ta = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(buf * TCR_NG * 16 + h * EW);
+                const uint32_t ta = tmem + (static_cast<uint32_t>(quarter * 32) << 16) + (uint32_t)(buf * TCR_NG * W + h * EW);
 #pragma unroll
                 for (int q = 0; q < EW / 16; ++q) {
                     float v[16];
@@ -514,15 +514,19 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
                 if (lane == 0) tc::mbar_arrive(&tfree[buf]);
             }
             if (!ok) break;
-            // entry (group 5 h + j / 16, column j % 16, row r) at (h EW + j) 128 + r
-            unsigned long long* out = part + ((long)blk * RB + g % RB) * (TCR_NG * 16 * 128) + h * EW * 128 + quarter * 32 + lane;
+            // accumulator column h EW + j: group / W, column of the group % W
+            const int cb = (int)(g / RB) * CB, ncb = min(CB, NCB - cb);
+            unsigned long long* out = part + ((long)cb * RB + g % RB) * (TCR_NG * 16 * 128) + quarter * 32 + lane;
             const uint32_t bias = (uint32_t)(u1 - u0) * TCR_MAGIC_BITS;
 #pragma unroll
             for (int j = 0; j < EW; ++j) {
                 // in steps, or the compiler widens all sums before the first atomic (spills)
                 if (j % 8 == 0) __syncwarp();
                 const long long v = (int)((uint32_t)acc[j] - bias);
-                atomicAdd(out + j * 128, (unsigned long long)v);
+                const int col = h * EW + j, gr = col / W, cc = col % W;
+                if (CB == 1 || (cc >> 4) < ncb)  // the last group may lack a block
+                    atomicAdd(out + (long)(cc >> 4) * RB * (TCR_NG * 16 * 128) + (gr * 16 + (cc & 15)) * 128,
+                              (unsigned long long)v);
             }
         }
     }
@@ -541,7 +545,43 @@ __device__ __forceinline__ void tcr_two_sum(double a, double b, double& s, doubl
     e = (a - (s - bb)) + (b - bb);
 }
 
-// thread: row i of column c = blockIdx.y; block partial norms as k_resid_final
+// 2^e2 times the 128-bit integer S as an unevaluated sum hi + lo of the same sign:
+// hi its first 53 bits, lo the next 53 (S of up to 106 bits, so n below 2^30, loses
+// none).  The bits are put together by integer instructions; one conversion.
+__device__ __forceinline__ void tcr_int128(__int128 S, int e2, double& hi, double& lo) {
+    const bool neg = S < 0;
+    const unsigned __int128 M = neg ? -(unsigned __int128)S : (unsigned __int128)S;
+    const unsigned long long m1 = (unsigned long long)(M >> 64), m0 = (unsigned long long)M;
+    hi = lo = 0.0;
+    if ((m1 | m0) == 0ull) return;
+    const int lz = m1 ? __clzll((long long)m1) : 64 + __clzll((long long)m0);
+    const unsigned __int128 N = M << lz;  // leading bit at 127
+    const unsigned long long n1 = (unsigned long long)(N >> 64), n0 = (unsigned long long)N;
+    const unsigned long long sign = neg ? 1ull << 63 : 0ull;
+    // 1.f = 2^-63 n1 without its last 11 bits
+    hi = ldexp(__longlong_as_double((long long)(sign | (1023ull << 52) | ((n1 >> 11) & 0xFFFFFFFFFFFFFull))),
+               127 - lz + e2);
+    const long long l = (long long)(((n1 & 0x7FFull) << 42) | (n0 >> 22));
+    lo = ldexp((double)(neg ? -l : l), 22 - lz + e2);
+}
+
+// the larger of two non-negative doubles over the warp by their bits; NaN counts as 0
+__device__ __forceinline__ double tcr_warp_max(double a) {
+    unsigned long long v = (unsigned long long)__double_as_longlong(a);
+    if (v > 0x7FF0000000000000ull) v = 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
+        v = w > v ? w : v;
+    }
+    return __longlong_as_double((long long)v);
+}
+
+// thread: row i of column c = blockIdx.y; block partial norms as k_resid_final.
+// Bound by the float64 units: the groups are summed as a 128-bit integer
+// (sum_t G_t 2^{-7t} = 2^-77 sum_k G_{k+2} 2^{7 (9 - k)}, exact), which left 16 float64
+// operations an entry of 140 (double-double sums and a conversion per group, maxima
+// by comparison of doubles): n = 8191, m = 32 64 -> 24 us.
 __global__ void __launch_bounds__(256) k_tcr_final(const unsigned long long* __restrict__ rowmax,
                                                    const int* __restrict__ xe,
                                                    const unsigned long long* __restrict__ part, int n, int m, int RB,
@@ -566,17 +606,11 @@ __global__ void __launch_bounds__(256) k_tcr_final(const unsigned long long* __r
         if (er == TCR_NONFINITE || fc == TCR_NONFINITE) {
             r = __longlong_as_double(0x7FF8000000000000ll);
         } else {
-            // sum_t G_t 2^{-7t}, smallest group first, in double-double (each
-            // term is exact: |G_t| < 2^53 for n < 2^30)
-            double hi = 0.0, lo = 0.0;
+            __int128 S = 0;  // |G_t| < 2^53 for n < 2^30: below 2^117
 #pragma unroll
-            for (int k = TCR_NG - 1; k >= 0; --k) {  // 2^{-7(k+2)}: a constant, the product exact
-                double e;
-                tcr_two_sum(hi, (double)gs[k] * __longlong_as_double((long long)(1023 - 7 * (k + 2)) << 52), hi, e);
-                lo += e;
-            }
-            hi = ldexp(hi, er + fc);
-            lo = ldexp(lo, er + fc);
+            for (int k = 0; k < TCR_NG; ++k) S = (S << 7) + gs[k];
+            double hi, lo;
+            tcr_int128(S, er + fc - 7 * TCR_TMAX, hi, lo);
             if (mode == 0) {
                 double s, e;
                 tcr_two_sum(B[(long)c * ldb + i], -hi, s, e);
@@ -590,9 +624,9 @@ __global__ void __launch_bounds__(256) k_tcr_final(const unsigned long long* __r
         r2 = r * r;
         if (X) xmax = fabs(X[(long)c * ldx + i]);
     }
-    rmax = warp_max(rmax);
+    rmax = tcr_warp_max(rmax);
     r2 = warp_sum(r2);
-    xmax = warp_max(xmax);
+    xmax = tcr_warp_max(xmax);
     const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
     if (l == 0) {
         red[0][w] = rmax;
@@ -660,7 +694,8 @@ struct TcrSchedule {
     long T;
 };
 
-// Column blocks per A tile: two from 17 columns on.
+// Column blocks per A tile: two from 17 columns on (m = 32: n = 8191 259 us against
+// 373 with one, n = 16384 956 against 1440; 16 columns take 803 there with one).
 
 TcrSchedule tcr_schedule(spd_handle* h, int n, int m) {
     TcrSchedule s;
@@ -705,7 +740,7 @@ spd_status tc_resid_bind(spd_handle* h, TcResidWs* w, int n, int m, const size_t
     w->G = s.G;
     w->per = s.per;
     w->T = s.T;
-    if (!tcr_map(&w->mapA, w->Ad, TCR_S, n, n, w->ldp, 128) || !tcr_map(&w->mapX, w->Xd, TCR_S, m, n, w->ldp, 16))
+    if (!tcr_map(&w->mapX, w->Xd, TCR_S, m, n, w->ldp, 16 * s.per))
         return set_err(h, SPD_ERR_UNSUPPORTED, "tensor-core residual: tensor map encoding failed");
     return SPD_OK;
 }
@@ -753,10 +788,10 @@ spd_status tc_resid_run(spd_handle* h, const TcResidWs* w, const double* B, long
     CUDA_TRY(h, cudaMemsetAsync(w->part, 0, sizeof(unsigned long long) * (size_t)w->CB * w->RB * TCR_NG * 16 * 128, s));
     ++h->launches;
     if (w->per == 2)
-        k_tcr_mma<2><<<w->G, tcr_threads(2), tcr_smem(2), s>>>(w->mapA, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
+        k_tcr_mma<2><<<w->G, tcr_threads(2), tcr_smem(2), s>>>(w->Ad, w->ldp, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
                                                                w->part, h->dst, gate);
     else
-        k_tcr_mma<1><<<w->G, tcr_threads(1), tcr_smem(1), s>>>(w->mapA, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
+        k_tcr_mma<1><<<w->G, tcr_threads(1), tcr_smem(1), s>>>(w->Ad, w->ldp, w->mapX, n, w->RB, w->CB, w->Nkc, w->T,
                                                                w->part, h->dst, gate);
     LAUNCH_CHECK(h);
     ++(h)->launches, k_tcr_final<<<dim3(ceil_div(n, 256), m), 256, 0, s>>>(

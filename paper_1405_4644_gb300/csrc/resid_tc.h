@@ -10,7 +10,7 @@
 // t = p + q <= 11 (55 products) the tensor cores form sum_j D_p(i,j) E_q(j,c)
 // exactly: each 64-wide chunk of j is accumulated in float32 (at most
 // 10 x 64 x 64^2 < 2^22 in magnitude: exact integers) and added to integer
-// sums.  The groups are combined in double-double with their scales
+// sums.  The groups are combined as a 128-bit integer with their scales
 // 2^{e_i + f_c - 7t}, and b - (A X) is rounded once.  Per term the dropped
 // products (t >= 12) and the truncation are below 2^-64.5 max_j|a_ij| max|x_c|.
 #pragma once
@@ -19,8 +19,8 @@
 #include "engine.cuh"
 
 struct TcResidWs {
-    CUtensorMap mapA, mapX;      // digit planes of A (rows) and of X (columns)
-    uint16_t* Ad = nullptr;      // [10][n][ldp] bf16 digits of A's rows
+    CUtensorMap mapX;            // digit planes of X (columns)
+    uint16_t* Ad = nullptr;      // 10 n ldp bf16 digits of A's rows, by tiles
     uint16_t* Xd = nullptr;      // [10][m][ldp] bf16 digits of X's columns
     unsigned long long* rowmax = nullptr;  // n: bits of max_j |a_ij|
     float* rowabs = nullptr;     // RS x n: partial sums of |a_ij| (float32)
