@@ -51,7 +51,12 @@ constexpr int BM = 128, BN = 256;
 // right-hand sides) take all three slices of an A tile and of a B tile in one
 // stage (SL = 3 slices per stage, one TMA load each with a box three planes
 // deep), so that each slice tile crosses from L2 to shared memory once per K
-// tile and the six slice products are issued from the same stage.
+// tile.  The three slices of the B tile lie one after another, so a slice of A is
+// multiplied with all the slices of B it meets in one instruction (N = 3, 2 and 1
+// times BNT) whose columns are the accumulators of the products' orders: a tensor
+// instruction of M = 128 costs about as much for 32 columns as for 96, and with six of
+// them per K step they, not the stream of A, bounded the product (n = 16384, 32
+// columns: 303 -> 243 us; A's slices alone 237).
 // bytes of K per row in a stage: 64 for the wide tiles with all slices in a
 // stage, else 128
 template <int BNT, int SL = 1> __host__ __device__ constexpr int row_bytes() { return SL == 3 && BNT >= 128 ? 64 : 128; }
@@ -217,8 +222,8 @@ __global__ void __launch_bounds__(192, 1)
     // one piece overlaps the next); narrow tiles promote every K tile's sums to
     // float32 registers, alternating two buffers
     constexpr int NBUF = (PROMOTE || NACC == 1) ? 2 : 1;
-    constexpr uint32_t ACC_COLS = BNT * NACC;  // one tile's accumulator(s)
-    constexpr uint32_t TMEM_COLS = ACC_COLS * NBUF;
+    constexpr uint32_t ACC_COLS = BNT * (PROMOTE ? 3 : NACC);  // one tile's accumulator(s)
+    constexpr uint32_t TMEM_COLS = PROMOTE ? 8 * BNT : ACC_COLS * NBUF;  // a power of two
     constexpr int MMA_PER_STAGE = BK / KindTraits<KIND>::KMMA;  // 32 bytes of K each
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -359,7 +364,7 @@ __global__ void __launch_bounds__(192, 1)
                     continue;
                 }
                 if constexpr (PROMOTE) {
-                    // each K tile into a fresh accumulator pair (buffer pk & 1),
+                    // each K tile into fresh accumulators (buffer pk & 1), one an order,
                     // which the epilogue adds to its float32 registers
                     for (int kin = kb; kin < ke; ++kin, ++kt, ++pk) {
                         const int b2 = pk & 1;
@@ -377,16 +382,18 @@ __global__ void __launch_bounds__(192, 1)
                             break;
                         }
                         tc::fence_after_sync();
-                        for (int q = 0; q < nseg; ++q) {
-                            const int za = (segs >> (4 * q)) & 3, zb = (segs >> (4 * q + 2)) & 3;
-                            const int a = (accsel >> q) & 1;
+                        // slice za of A against the slices 0 .. 2 - za of B, which
+                        // lie one after another: products of order za .. 2
+                        const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(sB + s * B_ST));
+#pragma unroll
+                        for (int za = 0; za < 3; ++za) {
                             const uint64_t ad = tc::sdesc_kmajor_sw128(tc::smem_u32(sA + s * A_ST + za * A_STAGE));
-                            const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(sB + s * B_ST + zb * B_STAGE));
-                            const uint32_t d = tmem + (uint32_t)(b2 * ACC_COLS + a * BNT);
-                            const bool fresh = q == first[a];
+                            const uint32_t d = tmem + (uint32_t)(b2 * ACC_COLS + za * BNT);
+                            constexpr uint32_t bf16 = 1;
+                            const uint32_t id = tc::idesc_f32acc(bf16, BM, (3 - za) * BNT);
 #pragma unroll
                             for (int k = 0; k < MMA_PER_STAGE; ++k)
-                                tc::mma<KIND>(d, ad + 2 * k, bd + 2 * k, idesc, (fresh && k == 0) ? 0u : 1u);
+                                tc::mma<KIND>(d, ad + 2 * k, bd + 2 * k, id, (za == 0 && k == 0) ? 0u : 1u);
                         }
                         tc::mma_commit(&empty[s]);
                         tc::mma_commit(&accfull[b2]);
@@ -445,10 +452,13 @@ __global__ void __launch_bounds__(192, 1)
                         float v[32];
                         tc::tmem_ld_32x32b_x32(ta + ch * 32, v);
 #pragma unroll
+                        for (int j = 0; j < 32; ++j) S1[ch * 32 + j] += v[j];
+                        tc::tmem_ld_32x32b_x32(ta + 2 * BNT + ch * 32, v);
+#pragma unroll
                         for (int j = 0; j < 32; ++j) S0[ch * 32 + j] += v[j];
                         tc::tmem_ld_32x32b_x32(ta + BNT + ch * 32, v);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) S1[ch * 32 + j] += v[j];
+                        for (int j = 0; j < 32; ++j) S0[ch * 32 + j] += v[j];
                     }
                     tc::fence_before_sync();
                     __syncwarp();
