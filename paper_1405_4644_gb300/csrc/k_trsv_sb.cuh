@@ -124,9 +124,40 @@ __device__ __forceinline__ void sb_pending(const SbArgs& a, int ns, int slot_lo,
     }
 }
 
-// Yk[l][c] = Y[r0 + l, c0 + c] (zero past n or past mc), minus the block
+// 64 tile entries into registers as tv_tile, but with 16-byte loads of whole lines in
+// the forward sweep too: thread (q, s) takes the columns 32 l + 4 s + e (l, e < 4)
+// of its rows, v[j * 16 + 4 l + e], so that eight adjacent lanes read the 128 bytes of
+// a row's line (columns s + 8 l' one by one were 32-byte pieces of four lines a load,
+// four times the L1 passes: PLACEHOLDER).  sb_pos is where row k of the staged
+// right-hand sides goes so that the product finds it at s + 8 (4 l + e).
+template <bool FWD>
+__device__ __forceinline__ int sb_pos(int k) {
+    return FWD ? (k & ~31) | ((k & 3) << 3) | ((k >> 2) & 7) : k;
+}
+template <bool FWD>
+__device__ __forceinline__ void sb_tile(float (&v)[64], const float* W, long ldw, int n, int J, int K, int q, int s) {
+    if constexpr (FWD) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const long gr = (long)J * 128 + 4 * q + j;
+            const float4* src = reinterpret_cast<const float4*>(W + gr * ldw + (long)K * 128) + s;
+#pragma unroll
+            for (int l = 0; l < 4; ++l) {
+                const float4 t = gr < n ? __ldg(src + 8 * l) : make_float4(0.f, 0.f, 0.f, 0.f);
+                v[j * 16 + 4 * l] = t.x;
+                v[j * 16 + 4 * l + 1] = t.y;
+                v[j * 16 + 4 * l + 2] = t.z;
+                v[j * 16 + 4 * l + 3] = t.w;
+            }
+        }
+    } else {
+        tv_tile<false>(v, W, ldw, n, J, K, q, s);
+    }
+}
+
+// Yk[sb_pos(l)][c] = Y[r0 + l, c0 + c] (zero past n or past mc), minus the block
 // row's pending partial sum when ns > 0
-template <int MC>
+template <int MC, bool FWD>
 __device__ __forceinline__ void sb_stage(float* Yk, const SbArgs& a, long r0, int ns = 0, int slot_lo = 0,
                                          int glo = 0) {
     constexpr int PER = (128 * MC + 255) / 256;
@@ -149,13 +180,13 @@ __device__ __forceinline__ void sb_stage(float* Yk, const SbArgs& a, long r0, in
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
         const int e = threadIdx.x + u * 256, l = e & 127, c = e >> 7;
-        if (e < 128 * MC) Yk[l * tv_ys<MC>() + c] = v[u];
+        if (e < 128 * MC) Yk[sb_pos<FWD>(l) * tv_ys<MC>() + c] = v[u];
     }
 }
 
 // Blocks [cs0, cs1) of y_I (from the output vector O) into YI (block c at
 // YI + c 128 tv_ys), loads issued eight per thread at a time
-template <int MC>
+template <int MC, bool FWD>
 __device__ __forceinline__ void sb_stage_range(float* YI, const SbArgs& a, int jb0, int cs0, int cs1) {
     constexpr int BATCH = 8;
     const int total = (cs1 - cs0) * 128 * MC;
@@ -177,7 +208,7 @@ __device__ __forceinline__ void sb_stage_range(float* YI, const SbArgs& a, int j
             const int e = base + k * 256;
             if (e < total) {
                 const int blk = cs0 + e / (128 * MC), rem = e - (blk - cs0) * 128 * MC;
-                YI[(blk * 128 + (rem & 127)) * tv_ys<MC>() + (rem >> 7)] = v[k];
+                YI[(blk * 128 + sb_pos<FWD>(rem & 127)) * tv_ys<MC>() + (rem >> 7)] = v[k];
             }
         }
     }
@@ -204,6 +235,47 @@ __device__ __forceinline__ void sb_prefetch_unit(const SbArgs& a, const SbPanel&
     const int J = pn.J0 + (int)(u / pn.nb), K = jb0 + (int)(u % pn.nb);
     if (FWD) sb_prefetch_tile(a.W, a.ldw, a.n, (long)J * 128, (long)K * 128);
     else sb_prefetch_tile(a.W, a.ldw, a.n, (long)K * 128, (long)J * 128);
+}
+
+// Sum over the eight reduction slices (adjacent lanes): each exchange halves the
+// values a lane still holds (7 MC / 2 shuffles instead of 12 MC), so that lane s ends
+// with row j = s / 2 of the quad, columns (s % 2) MC / 2 .. in acc[0][0 ..] (MC = 1: the
+// column, in both lanes of the pair), and the results are written by all lanes.
+template <int MC>
+__device__ __forceinline__ void sb_reduce(float (&acc)[4][MC], float (&out)[MC > 1 ? MC / 2 : 1], int s) {
+    float v[4 * MC];
+#pragma unroll
+    for (int i = 0; i < 4 * MC; ++i) v[i] = acc[i / MC][i % MC];
+#pragma unroll
+    for (int b = 4, h = 2 * MC; b >= 1; b >>= 1, h >>= 1) {
+        if (h >= 1) {
+            const bool hi = s & b;
+#pragma unroll
+            for (int i = 0; i < h; ++i) {
+                const float send = hi ? v[i] : v[i + h];
+                const float keep = hi ? v[i + h] : v[i];
+                v[i] = keep + __shfl_xor_sync(0xffffffffu, send, b);
+            }
+        } else {
+            v[0] += __shfl_xor_sync(0xffffffffu, v[0], b);
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < (MC > 1 ? MC / 2 : 1); ++i) out[i] = v[i];
+}
+
+// out of sb_reduce to a 128 x MC partial tile
+template <int MC>
+__device__ __forceinline__ void sb_put(float* pt, const float (&out)[MC > 1 ? MC / 2 : 1], int q, int s) {
+    float* d = pt + (4 * q + (s >> 1)) * MC + (MC > 1 ? (s & 1) * (MC / 2) : 0);
+    if constexpr (MC >= 8) {
+#pragma unroll
+        for (int i = 0; i < MC / 2; i += 4)
+            *reinterpret_cast<float4*>(d + i) = make_float4(out[i], out[i + 1], out[i + 2], out[i + 3]);
+    } else {
+#pragma unroll
+        for (int i = 0; i < (MC > 1 ? MC / 2 : 1); ++i) d[i] = out[i];
+    }
 }
 
 // shared memory: y_I of one super-block (SPD_SB_BLOCKS staged 128 x MC blocks)
@@ -244,6 +316,17 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
     int nbar = 0;
     float ra[64], rb[64];
     SbPanel prev{0, 1, 1, 0};  // the previous step's panel update (W = 0: none)
+    // each phase's first tile is loaded before the barrier in front of it: tiles of L
+    // and of the inverses do not change
+    auto first_inverse_tile = [&](int I) {
+        const int nb = min(a.SBB, a.NB - I * a.SBB);
+        if (g >= nb * (nb + 1) / 2) return;
+        int p = 0;
+        while (sb_tri(p + 1, 0) <= g) ++p;
+        const int q = g - sb_tri(p, 0);
+        sb_tile<FWD>(ra, a.X + (long)I * a.S * a.S, a.S, a.S, FWD ? p : q, FWD ? q : p, tq, ts);
+    };
+    first_inverse_tile(FWD ? 0 : a.NS - 1);
     for (int t = 0; t < a.NS; ++t) {
         const int I = FWD ? t : a.NS - 1 - t;
         const int jb0 = I * a.SBB;                    // first 128-block of the super-block
@@ -278,10 +361,10 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
             const int q = task - sb_tri(p, 0);  // q <= p
             // forward: X[b][c] with b = p, c = q; backward: X[c][b]^T with b = q, c = p
             const int b = FWD ? p : q, c = FWD ? q : p;
-            tv_tile<FWD>(ra, XI, a.S, a.S, b, c, tq, ts);
+            if (task != g) sb_tile<FWD>(ra, XI, a.S, a.S, b, c, tq, ts);
             int slot_lo = 0, glo = 0;
             const int ns = prev.W == 0 ? 0 : sb_row_slots(prev, jb0 + c, slot_lo, glo);
-            sb_stage<MC>(YI, a, (long)(jb0 + c) * 128, ns, slot_lo, glo);
+            sb_stage<MC, FWD>(YI, a, (long)(jb0 + c) * 128, ns, slot_lo, glo);
             __syncthreads();
             float acc[4][MC];
 #pragma unroll
@@ -289,14 +372,9 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
 #pragma unroll
                 for (int cc = 0; cc < MC; ++cc) acc[j][cc] = 0.f;
             tv_dot<MC>(acc, ra, YI, ts);
-            tv_reduce8<MC>(acc);
-            if (ts == 0) {
-                float* pt = a.P + (long)task * 128 * MC;
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-#pragma unroll
-                    for (int cc = 0; cc < MC; ++cc) pt[(4 * tq + j) * MC + cc] = acc[j][cc];
-            }
+            float sum[MC > 1 ? MC / 2 : 1];
+            sb_reduce<MC>(acc, sum, ts);
+            sb_put<MC>(a.P + (long)task * 128 * MC, sum, tq, ts);
             __syncthreads();
             // the last tile of block row b to arrive adds the row's partials
             // in c order (forward c = 0..b, backward c = b..nb-1) into y_I[b]
@@ -332,7 +410,6 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
             }
         }
         if (t + 1 == a.NS) break;  // no rows left to update
-        if (!sb_barrier(a, ++nbar, &s_abort)) return;
         // B: units (J, c) of every remaining 128-row block J (forward: below
         // the super-block, backward: above it), in equal ranges over the CTAs
         SbPanel pn;
@@ -340,13 +417,17 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
         pn.nb = nb;
         pn.W = (long)((FWD ? a.NB : jb0) - pn.J0) * nb;
         pn.geff = (int)min((long)G, pn.W);
+        const long u0 = sb_ub(g, pn.W, pn.geff), u1 = g < pn.geff ? sb_ub(g + 1, pn.W, pn.geff) : u0;
         if (g < pn.geff) {
-            const long u0 = sb_ub(g, pn.W, pn.geff), u1 = sb_ub(g + 1, pn.W, pn.geff);
+            sb_tile<FWD>(ra, a.W, a.ldw, a.n, pn.J0 + (int)(u0 / nb), jb0 + (int)(u0 % nb), tq, ts);
+            if (u0 + 1 < u1) sb_prefetch_unit<FWD>(a, pn, jb0, u0 + 1);
+        }
+        if (!sb_barrier(a, ++nbar, &s_abort)) return;
+        if (g < pn.geff) {
             // the blocks of y_I this CTA's units multiply, staged once
             const bool all = (u1 - u0 >= nb) || (u0 / nb != (u1 - 1) / nb);
             const int cs0 = all ? 0 : (int)(u0 % nb), cs1 = all ? nb : (int)((u1 - 1) % nb) + 1;
-            for (long v = u0; v < min(u1, u0 + 2); ++v) sb_prefetch_unit<FWD>(a, pn, jb0, v);
-            sb_stage_range<MC>(YI, a, jb0, cs0, cs1);
+            sb_stage_range<MC, FWD>(YI, a, jb0, cs0, cs1);
             __syncthreads();
             for (long u = u0; u < u1;) {
                 const int J = pn.J0 + (int)(u / nb), ca = (int)(u % nb);
@@ -360,45 +441,40 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
                 // two per trip so that the register buffers alternate: the
                 // next tile's loads are in flight during this tile's products
                 // (tiles two units ahead, across pieces, are prefetched into L2)
-                tv_tile<FWD>(ra, a.W, a.ldw, a.n, J, jb0 + ca, tq, ts);
+                if (u != u0) sb_tile<FWD>(ra, a.W, a.ldw, a.n, J, jb0 + ca, tq, ts);
                 for (int c = ca; c < ce; c += 2) {
                     const long uc = u + (c - ca);
                     if (uc + 2 < u1) sb_prefetch_unit<FWD>(a, pn, jb0, uc + 2);
-                    if (c + 1 < ce) tv_tile<FWD>(rb, a.W, a.ldw, a.n, J, jb0 + c + 1, tq, ts);
+                    if (c + 1 < ce) sb_tile<FWD>(rb, a.W, a.ldw, a.n, J, jb0 + c + 1, tq, ts);
                     tv_dot<MC>(acc, ra, YI + c * YB, ts);
                     if (c + 1 >= ce) break;
                     if (uc + 3 < u1) sb_prefetch_unit<FWD>(a, pn, jb0, uc + 3);
-                    if (c + 2 < ce) tv_tile<FWD>(ra, a.W, a.ldw, a.n, J, jb0 + c + 2, tq, ts);
+                    if (c + 2 < ce) sb_tile<FWD>(ra, a.W, a.ldw, a.n, J, jb0 + c + 2, tq, ts);
                     tv_dot<MC>(acc, rb, YI + (c + 1) * YB, ts);
                 }
-                tv_reduce8<MC>(acc);
-                if (ts == 0) {
-                    if (ca == 0 && ce == nb) {  // the whole row: subtract in place
+                float sum[MC > 1 ? MC / 2 : 1];
+                sb_reduce<MC>(acc, sum, ts);
+                if (ca == 0 && ce == nb) {  // the whole row: subtract in place
+                    const long row = (long)J * 128 + 4 * tq + (ts >> 1);
+                    const int cc0 = MC > 1 ? (ts & 1) * (MC / 2) : 0;
+                    if (row < a.n && (MC > 1 || !(ts & 1))) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const long row = (long)J * 128 + 4 * tq + j;
-#pragma unroll
-                            for (int cc = 0; cc < MC; ++cc)
-                                if (cc < a.mc && row < a.n) {
-                                    float* y = a.Y + (long)(a.c0 + cc) * a.n + row;
-                                    *y = __ldcg(y) - acc[j][cc];
-                                }
-                        }
-                    } else {  // a piece of a shared row: partial slot
-                        float* pt = a.P2 + (long)(2 * g + (u == u0 ? 0 : 1)) * 128 * MC;
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-#pragma unroll
-                            for (int cc = 0; cc < MC; ++cc) pt[(4 * tq + j) * MC + cc] = acc[j][cc];
+                        for (int i = 0; i < (MC > 1 ? MC / 2 : 1); ++i)
+                            if (cc0 + i < a.mc) {
+                                float* y = a.Y + (long)(a.c0 + cc0 + i) * a.n + row;
+                                *y = __ldcg(y) - sum[i];
+                            }
                     }
+                } else {  // a piece of a shared row: partial slot
+                    sb_put<MC>(a.P2 + (long)(2 * g + (u == u0 ? 0 : 1)) * 128 * MC, sum, tq, ts);
                 }
                 u += ce - ca;
             }
         }
-        {   // the next super-block's inverse tiles this CTA will multiply in phase F
+        {   // the next super-block's other inverse tiles this CTA will multiply in phase F
             const int In = FWD ? I + 1 : I - 1;
             const int nbn = min(a.SBB, a.NB - In * a.SBB), ntn = nbn * (nbn + 1) / 2;
-            for (int task = g; task < ntn; task += G) {
+            for (int task = g + G; task < ntn; task += G) {
                 int p = 0;
                 while (sb_tri(p + 1, 0) <= task) ++p;
                 const int q = task - sb_tri(p, 0);
@@ -408,6 +484,7 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
                 else sb_prefetch_tile(XN, a.S, a.S, (long)c * 128, (long)b * 128);
             }
         }
+        first_inverse_tile(FWD ? I + 1 : I - 1);
         prev = pn;
         if (!sb_barrier(a, ++nbar, &s_abort)) return;
     }
