@@ -124,12 +124,14 @@ __device__ __forceinline__ void sb_pending(const SbArgs& a, int ns, int slot_lo,
     }
 }
 
-// 64 tile entries into registers as tv_tile, but with 16-byte loads of whole lines in
-// the forward sweep too: thread (q, s) takes the columns 32 l + 4 s + e (l, e < 4)
-// of its rows, v[j * 16 + 4 l + e], so that eight adjacent lanes read the 128 bytes of
-// a row's line (columns s + 8 l' one by one were 32-byte pieces of four lines a load,
-// four times the L1 passes: PLACEHOLDER).  sb_pos is where row k of the staged
-// right-hand sides goes so that the product finds it at s + 8 (4 l + e).
+// 64 tile entries into registers as tv_tile, in 16-byte loads of whole lines (with
+// pieces of lines the sweeps were bound by the passes through L1: busy 43 and 53 % of
+// the time at n = 8191, m = 32, the float32 units 20 %; forward 258 -> 189 us,
+// backward 313 -> 216, the reductions below included).  Forward, eight adjacent lanes are the slices s of a row quad q:
+// thread (q, s) takes the columns 32 l + 4 s + e (l, e < 4) of its rows, v[j * 16 + 4 l +
+// e]; sb_pos is where row k of the staged right-hand sides goes so that the product
+// finds it at s + 8 (4 l + e).  Backward, a warp is a slice s and its lanes the 32
+// column quads q: a load is one row of the tile.
 template <bool FWD>
 __device__ __forceinline__ int sb_pos(int k) {
     return FWD ? (k & ~31) | ((k & 3) << 3) | ((k >> 2) & 7) : k;
@@ -237,7 +239,52 @@ __device__ __forceinline__ void sb_prefetch_unit(const SbArgs& a, const SbPanel&
     else sb_prefetch_tile(a.W, a.ldw, a.n, (long)K * 128, (long)J * 128);
 }
 
-// Sum over the eight reduction slices (adjacent lanes): each exchange halves the
+// Backward: the slices are the eight warps; each writes its sums to red (in the order
+// in which lanes hold them) and every thread adds the slices of its share, four columns
+// (MC < 4: one) of row 4 q + j at a time, in slice order, and passes it to put(row of
+// the tile, first column, sums).
+template <int MC, typename Put>
+__device__ __forceinline__ void sb_reduce_warps(const float (&acc)[4][MC], float* red, Put put) {
+    constexpr int V = MC >= 4 ? 4 : 1, CV = MC / V;
+    const int q = threadIdx.x & 31, s = threadIdx.x >> 5;
+    __syncthreads();  // the last sums have been read
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+#pragma unroll
+        for (int c = 0; c < CV; ++c) {
+            float* d = red + (((s * 4 + j) * CV + c) * 32 + q) * V;
+            if constexpr (V == 4)
+                *reinterpret_cast<float4*>(d) = make_float4(acc[j][4 * c], acc[j][4 * c + 1], acc[j][4 * c + 2], acc[j][4 * c + 3]);
+            else
+                *d = acc[j][c];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int e0 = 0; e0 < 128 * CV; e0 += 256) {
+        const int e = e0 + threadIdx.x;
+        if (128 * CV < 256 && e >= 128 * CV) break;
+        const int r = e >> 5, j = r / CV, c = r % CV;
+        float t[V];
+#pragma unroll
+        for (int i = 0; i < V; ++i) t[i] = 0.f;
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const float* d = red + (k * 128 * CV + e) * V;
+            if constexpr (V == 4) {
+                const float4 x = *reinterpret_cast<const float4*>(d);
+                t[0] += x.x;
+                t[1] += x.y;
+                t[2] += x.z;
+                t[3] += x.w;
+            } else {
+                t[0] += *d;
+            }
+        }
+        put(4 * (e & 31) + j, c * V, t);
+    }
+}
+
+// Forward: sum over the eight reduction slices (adjacent lanes); each exchange halves the
 // values a lane still holds (7 MC / 2 shuffles instead of 12 MC), so that lane s ends
 // with row j = s / 2 of the quad, columns (s % 2) MC / 2 .. in acc[0][0 ..] (MC = 1: the
 // column, in both lanes of the pair), and the results are written by all lanes.
@@ -278,10 +325,28 @@ __device__ __forceinline__ void sb_put(float* pt, const float (&out)[MC > 1 ? MC
     }
 }
 
-// shared memory: y_I of one super-block (SPD_SB_BLOCKS staged 128 x MC blocks)
+// the slices' sum of acc to a 128 x MC partial tile
+template <int MC, bool FWD>
+__device__ __forceinline__ void sb_store(float* pt, float (&acc)[4][MC], float* red, int q, int s) {
+    if constexpr (FWD) {
+        float sum[MC > 1 ? MC / 2 : 1];
+        sb_reduce<MC>(acc, sum, s);
+        sb_put<MC>(pt, sum, q, s);
+    } else {
+        sb_reduce_warps<MC>(acc, red, [&](int r, int c, auto& t) {
+            if constexpr (MC >= 4)
+                *reinterpret_cast<float4*>(pt + r * MC + c) = make_float4(t[0], t[1], t[2], t[3]);
+            else
+                pt[r * MC + c] = t[0];
+        });
+    }
+}
+
+// shared memory: y_I of one super-block (SPD_SB_BLOCKS staged 128 x MC blocks) and the
+// eight warps' sums of the backward sweep
 template <int MC>
 constexpr size_t trsv_sb_smem() {
-    return (size_t)SPD_SB_BLOCKS * 128 * tv_ys<MC>() * sizeof(float);
+    return (size_t)(SPD_SB_BLOCKS * 128 * tv_ys<MC>() + 8 * 128 * MC) * sizeof(float);
 }
 
 // tile index of the pair (p, q), q <= p, in the order (0,0), (1,0), (1,1), ...
@@ -297,10 +362,11 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* YI = reinterpret_cast<float*>(smem_raw);  // [SBB][128][tv_ys] staged blocks of y_I (F: one)
     constexpr int YB = 128 * tv_ys<MC>();           // floats per staged block
+    float* red = YI + SPD_SB_BLOCKS * YB;           // backward: the warps' sums
     __shared__ int s_abort, s_last;
     if (a.gate && *a.gate == 0) return;  // refinement over (capturable solves)
     const int tid = threadIdx.x;
-    const int tq = tid >> 3, ts = tid & 7;
+    const int tq = FWD ? tid >> 3 : tid & 31, ts = FWD ? tid & 7 : tid >> 5;  // row quad, reduction slice
     const int G = gridDim.x, g = blockIdx.x;
     if (gridDim.y > 1) {
         const int y = blockIdx.y;
@@ -372,9 +438,7 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
 #pragma unroll
                 for (int cc = 0; cc < MC; ++cc) acc[j][cc] = 0.f;
             tv_dot<MC>(acc, ra, YI, ts);
-            float sum[MC > 1 ? MC / 2 : 1];
-            sb_reduce<MC>(acc, sum, ts);
-            sb_put<MC>(a.P + (long)task * 128 * MC, sum, tq, ts);
+            sb_store<MC, FWD>(a.P + (long)task * 128 * MC, acc, red, tq, ts);
             __syncthreads();
             // the last tile of block row b to arrive adds the row's partials
             // in c order (forward c = 0..b, backward c = b..nb-1) into y_I[b]
@@ -452,21 +516,29 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
                     if (c + 2 < ce) sb_tile<FWD>(ra, a.W, a.ldw, a.n, J, jb0 + c + 2, tq, ts);
                     tv_dot<MC>(acc, rb, YI + (c + 1) * YB, ts);
                 }
-                float sum[MC > 1 ? MC / 2 : 1];
-                sb_reduce<MC>(acc, sum, ts);
                 if (ca == 0 && ce == nb) {  // the whole row: subtract in place
-                    const long row = (long)J * 128 + 4 * tq + (ts >> 1);
-                    const int cc0 = MC > 1 ? (ts & 1) * (MC / 2) : 0;
-                    if (row < a.n && (MC > 1 || !(ts & 1))) {
+                    auto sub = [&](int r, int c, float t) {
+                        const long row = (long)J * 128 + r;
+                        if (row < a.n && c < a.mc) {
+                            float* y = a.Y + (long)(a.c0 + c) * a.n + row;
+                            *y = __ldcg(y) - t;
+                        }
+                    };
+                    if constexpr (FWD) {
+                        float sum[MC > 1 ? MC / 2 : 1];
+                        sb_reduce<MC>(acc, sum, ts);
+                        if (MC > 1 || !(ts & 1))
 #pragma unroll
-                        for (int i = 0; i < (MC > 1 ? MC / 2 : 1); ++i)
-                            if (cc0 + i < a.mc) {
-                                float* y = a.Y + (long)(a.c0 + cc0 + i) * a.n + row;
-                                *y = __ldcg(y) - sum[i];
-                            }
+                            for (int i = 0; i < (MC > 1 ? MC / 2 : 1); ++i)
+                                sub(4 * tq + (ts >> 1), (MC > 1 ? (ts & 1) * (MC / 2) : 0) + i, sum[i]);
+                    } else {
+                        sb_reduce_warps<MC>(acc, red, [&](int r, int c, auto& t) {
+#pragma unroll
+                            for (int i = 0; i < (MC >= 4 ? 4 : 1); ++i) sub(r, c + i, t[i]);
+                        });
                     }
                 } else {  // a piece of a shared row: partial slot
-                    sb_put<MC>(a.P2 + (long)(2 * g + (u == u0 ? 0 : 1)) * 128 * MC, sum, tq, ts);
+                    sb_store<MC, FWD>(a.P2 + (long)(2 * g + (u == u0 ? 0 : 1)) * 128 * MC, acc, red, tq, ts);
                 }
                 u += ce - ca;
             }
