@@ -161,6 +161,16 @@ template <typename T> __device__ __forceinline__ T dsqrt(T x);
 template <> __device__ __forceinline__ float dsqrt<float>(float x) { return sqrtf(x); }
 template <> __device__ __forceinline__ double dsqrt<double>(double x) { return sqrt(x); }
 
+// Tile t of the lower triangle, row-major over (i, j <= i).  The root is taken in float32
+// and corrected: a float64 root by every thread delayed each CTA's first loads (n = 16384:
+// k_scale_convert 453 -> 432 us, k_lz_symv_tiles 92 -> 82).
+__device__ __forceinline__ void tri_tile(long t, int& i, int& j) {
+    i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);
+    while ((long)(i + 1) * (i + 2) / 2 <= t) ++i;
+    while ((long)i * (i + 1) / 2 > t) --i;
+    j = (int)(t - (long)i * (i + 1) / 2);
+}
+
 // Bounded spin-wait on a device flag (volatile load).  Returns false after
 // `limit` polls without seeing `want`.
 __device__ __forceinline__ bool spin_until_geq(const volatile int* flag, int want, long limit) {

@@ -150,10 +150,8 @@ static __global__ void __launch_bounds__(256) k_scale_convert(const double* __re
                                                                 long ldw, DevStatus* st) {
     __shared__ T tile[64][65];  // tile[i_local][j_local]
     const long t = blockIdx.x;
-    int bi = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-    while ((long)(bi + 1) * (bi + 2) / 2 <= t) ++bi;
-    while ((long)bi * (bi + 1) / 2 > t) --bi;
-    const int bj = (int)(t - (long)bi * (bi + 1) / 2);
+    int bi, bj;
+    tri_tile(t, bi, bj);
     const int i0 = bi * 64, j0 = bj * 64;
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
     double a[16];

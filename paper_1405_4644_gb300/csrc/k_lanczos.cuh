@@ -26,15 +26,6 @@
 #define LZ_CHUNKS 64    // row chunks of the vector reductions
 #define LZ_MAXK 16      // Lanczos steps at most
 
-// tile t of the lower triangle, row-major over (I, J <= I)
-__device__ __forceinline__ void lz_tile(long t, int& I, int& J) {
-    int i = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
-    while ((long)(i + 1) * (i + 2) / 2 <= t) ++i;
-    while ((long)i * (i + 1) / 2 > t) --i;
-    I = i;
-    J = (int)(t - (long)i * (i + 1) / 2);
-}
-
 // The sixteen row sums of a warp (v[k]: this lane's part of row k) with 16
 // shuffles instead of 5 per row: at each step a lane keeps half of its
 // values, sends the other half to the partner (lane ^ 16, 8, 4, 2) and adds
@@ -83,7 +74,7 @@ __global__ void __launch_bounds__(256, 3) k_lz_symv_tiles(const float* __restric
     __shared__ float ps[LZ_T];
     __shared__ float qs[8][LZ_T];
     int I, J;
-    lz_tile(blockIdx.x, I, J);
+    tri_tile(blockIdx.x, I, J);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int r0 = I * LZ_T, c0 = J * LZ_T;
     if (tid < LZ_T) xs_i[tid] = (r0 + tid < n) ? x[r0 + tid] : 0.f;
