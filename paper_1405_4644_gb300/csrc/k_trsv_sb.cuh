@@ -127,11 +127,11 @@ __device__ __forceinline__ void sb_pending(const SbArgs& a, int ns, int slot_lo,
 // 64 tile entries into registers as tv_tile, in 16-byte loads of whole lines (with
 // pieces of lines the sweeps were bound by the passes through L1: busy 43 and 53 % of
 // the time at n = 8191, m = 32, the float32 units 20 %; forward 258 -> 189 us,
-// backward 313 -> 216, the reductions below included).  Forward, eight adjacent lanes are the slices s of a row quad q:
-// thread (q, s) takes the columns 32 l + 4 s + e (l, e < 4) of its rows, v[j * 16 + 4 l +
-// e]; sb_pos is where row k of the staged right-hand sides goes so that the product
-// finds it at s + 8 (4 l + e).  Backward, a warp is a slice s and its lanes the 32
-// column quads q: a load is one row of the tile.
+// backward 313 -> 216, the reductions below included).  Forward, eight adjacent lanes
+// are the slices s of a row quad q: thread (q, s) takes the columns 32 l + 4 s + e
+// (l, e < 4) of its rows, v[j * 16 + 4 l + e]; sb_pos is where row k of the staged
+// right-hand sides goes so that the product finds it at s + 8 (4 l + e).  Backward, a
+// warp is a slice s and its lanes the 32 column quads q: a load is one row of the tile.
 template <bool FWD>
 __device__ __forceinline__ int sb_pos(int k) {
     return FWD ? (k & ~31) | ((k & 3) << 3) | ((k >> 2) & 7) : k;

@@ -350,10 +350,10 @@ __global__ void __launch_bounds__(256) k_tcr_digits_x(const double* __restrict__
 // instructions a tile hide behind the stream, two blocks' 80 do not), so the 320 and
 // 288 columns of p = 0, 1 are split in two and the others go as one (n = 8191 / 16384,
 // m = 32: one block at a time 373 / 1440 us, two with instructions of their own
-// 308 / 1150, as one 259 / 956; the planes' stream alone 197 / 790).  With
-// one accumulator buffer of 320 columns, the wait for the read-out before the next
-// tile's first product costs the tensor core, not the stream of A, which the ring
-// covers.
+// 308 / 1150, as one 259 / 956; the planes' stream alone 197 / 790).  The
+// accumulators take 320 of the 512 columns, so there is one buffer: its lower half
+// (groups 0 .. 4) is complete after p = 4 and read out during the other products, its
+// upper half during the next tile's products with the lower one (n = 8191 / 16384, m = 32: 259 -> 237 us, 956 -> 860).
 constexpr int TCR_FLUSH = 256;
 template <int CB>
 __global__ void __launch_bounds__(tcr_threads(CB), 1)
@@ -373,8 +373,8 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
     uint64_t* aempty = afull + NA;
     uint64_t* xfull = aempty + NA;
     uint64_t* xempty = xfull + NX;
-    uint64_t* tfull = xempty + NX;  // [2] chunk accumulated (tcgen05.commit)
-    uint64_t* tfree = tfull + 2;    // [2] chunk read out (8 CB epilogue warps)
+    uint64_t* tfull = xempty + NX;  // [2] chunk accumulated (tcgen05.commit), by buffer or (CB = 2) half
+    uint64_t* tfree = tfull + 2;    // [2] chunk read out (8 epilogue warps)
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfree + 2);
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
         }
         for (int s = 0; s < 2; ++s) {
             tc::mbar_init(&tfull[s], 1);
-            tc::mbar_init(&tfree[s], 8 * CB);
+            tc::mbar_init(&tfree[s], 8);
         }
         *abort_flag = 0;
         tc::fence_barrier_init();
@@ -446,6 +446,7 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
             bool ok = true;
             for (int u = 0; u < nitems && ok; ++u) {
                 const int buf = u % NB, sx = u % NX;
+                // CB = 2: the lower half of the columns; the upper one is waited for below
                 if (u >= NB && !tc::mbar_wait(&tfree[buf], (u / NB - 1) & 1u, abort_flag, TCR_WAIT_NS)) break;
                 if (!tc::mbar_wait(&xfull[sx], (u / NX) & 1u, abort_flag, TCR_WAIT_NS)) break;
                 tc::fence_after_sync();
@@ -456,29 +457,46 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
                 // of N = W (10 - p) in all, whose columns are the accumulators
                 // of groups p .. 9 (group g at columns W g)
                 const uint64_t bd = tc::sdesc_kmajor_sw128(tc::smem_u32(sX + sx * XB));
-                for (int p = 0; p < TCR_S; ++p) {
-                    const int sa = ia % NA;
-                    if (!tc::mbar_wait(&afull[sa], (ia / NA) & 1u, abort_flag, TCR_WAIT_NS)) {
-                        ok = false;
-                        break;
-                    }
-                    tc::fence_after_sync();
+                // columns [c0, c0 + N) of A plane p's products
+                auto products = [&](int p, int sa, int c0, int N) {
                     const uint64_t ad = tc::sdesc_kmajor_sw128(tc::smem_u32(sA + sa * TCR_A_BYTES));
-                    const int cols = W * (TCR_S - p), parts = cols > 256 ? 2 : 1, N = cols / parts;
+                    const uint64_t bv = bd + (uint64_t)((c0 - p * W) * 128 >> 4);
                     const uint32_t idesc = tc::idesc_f32acc(1, 128, N);  // bf16 -> f32
-                    for (int v = 0; v < parts; ++v) {
-                        const uint32_t dcol = dbase + (uint32_t)(p * W + v * N);
-                        const uint64_t bv = bd + (uint64_t)(v * N * 128 >> 4);
 #pragma unroll
-                        for (int kk = 0; kk < TCR_BK / 16; ++kk)  // +32 bytes of K = +2 in the address field
-                            tc::mma<0>(dcol, ad + 2 * kk, bv + 2 * kk, idesc, (p > 0 || kk > 0) ? 1u : 0u);
+                    for (int kk = 0; kk < TCR_BK / 16; ++kk)  // +32 bytes of K = +2 in the address field
+                        tc::mma<0>(dbase + (uint32_t)c0, ad + 2 * kk, bv + 2 * kk, idesc, (p > 0 || kk > 0) ? 1u : 0u);
+                };
+                auto landed = [&](int i) {
+                    if (!tc::mbar_wait(&afull[i % NA], (i / NA) & 1u, abort_flag, TCR_WAIT_NS)) return false;
+                    tc::fence_after_sync();
+                    return true;
+                };
+                int p = 0;
+                if constexpr (CB == 2) {
+                    // planes 0 and 1 in two halves (N <= 256), the lower halves first:
+                    // they run while the upper half of the last tile is read out
+                    constexpr int H = TCR_NG * W / 2;
+                    for (; p < 2 && ok; ++p) {
+                        ok = landed(ia + p);
+                        if (ok) products(p, (ia + p) % NA, p * W, H - p * W);
                     }
-                    tc::mma_commit(&aempty[sa]);
-                    ++ia;
+                    if (ok && u >= 1) ok = tc::mbar_wait(&tfree[1], (u - 1) & 1u, abort_flag, TCR_WAIT_NS);
+                    if (!ok) break;
+                    tc::fence_after_sync();
+                    for (p = 0; p < 2; ++p, ++ia) {
+                        products(p, ia % NA, H, H);
+                        tc::mma_commit(&aempty[ia % NA]);
+                    }
+                }
+                for (; p < TCR_S; ++p, ++ia) {
+                    if (!(ok = landed(ia))) break;
+                    products(p, ia % NA, p * W, W * (TCR_S - p));
+                    tc::mma_commit(&aempty[ia % NA]);
+                    if (CB == 2 && p == TCR_NG / 2 - 1) tc::mma_commit(&tfull[0]);  // groups 0 .. 4 are complete
                 }
                 if (!ok) break;
                 tc::mma_commit(&xempty[sx]);
-                tc::mma_commit(&tfull[buf]);
+                tc::mma_commit(&tfull[CB == 2 ? 1 : buf]);
             }
         }
         __syncwarp();
@@ -496,8 +514,8 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
             for (int j = 0; j < EW; ++j) acc[j] = 0;
 #pragma unroll 1
             for (; u < u1; ++u) {
-                const int buf = u % NB;
-                ok = tc::mbar_wait(&tfull[buf], (u / NB) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
+                const int buf = u % NB, bar = CB == 2 ? h >> 1 : buf;
+                ok = tc::mbar_wait(&tfull[bar], (u / NB) & 1u, abort_flag, TCR_WAIT_NS) && !*abort_flag;
                 ok = __all_sync(0xffffffffu, ok);  // tcgen05.ld is warp-collective
                 if (!ok) break;
                 tc::fence_after_sync();
@@ -511,7 +529,7 @@ __global__ void __launch_bounds__(tcr_threads(CB), 1)
                 }
                 tc::fence_before_sync();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(&tfree[buf]);
+                if (lane == 0) tc::mbar_arrive(&tfree[bar]);
             }
             if (!ok) break;
             // accumulator column h EW + j: group / W, column of the group % W
@@ -694,8 +712,8 @@ struct TcrSchedule {
     long T;
 };
 
-// Column blocks per A tile: two from 17 columns on (m = 32: n = 8191 259 us against
-// 373 with one, n = 16384 956 against 1440; 16 columns take 803 there with one).
+// Column blocks per A tile: two from 17 columns on (m = 32: n = 8191 237 us against
+// 373 with one, n = 16384 860 against 1440; 16 columns take 800 there with one).
 
 TcrSchedule tcr_schedule(spd_handle* h, int n, int m) {
     TcrSchedule s;

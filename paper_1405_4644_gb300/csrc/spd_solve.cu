@@ -531,15 +531,15 @@ spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, i
 // about c + a n + (b + (g - 1) d) n^2 us, n in thousands: the chain of phases (its
 // links grow with w), a group's share of the panel products, and what another
 // group adds (it reads the panel again and has its own products).  Coefficients
-// fitted to sweep pairs at n = 2100, 8191 and 16384 (one group of 16: 158, 501,
-// 1225 us; of 8: 113, 349, 830; two groups of 8: 115, 418, 1213; four of 16: 177,
-// 924, 3075 against 557, 1938, 4715 one after another).
+// fitted to spd_factor_solve at n = 2100, 8191 and 16384 (one group of 1: 82, 211,
+// 462 us; one of 8: 99, 286, 653; two of 8: 100, 333, 871; one of 16: 131, 432, 1023;
+// four of 8: 109, 443, 1247; two of 16: 132, 523, 1407).
 void sb_groups(int n, int m, int* w_out, int* per_out) {
     static const struct {
         int w;
         double c, a, b, d;
-    } T[] = {{1, 35, 27.2, 0.48, 0.60}, {2, 37, 27.3, 0.62, 0.75}, {4, 36, 28.3, 0.78, 0.95},
-             {8, 38, 34.5, 0.98, 1.30}, {16, 52, 47.6, 1.66, 2.20}};
+    } T[] = {{1, 49, 14.4, 0.66, 0.34}, {2, 52, 14.3, 0.70, 0.39}, {4, 50, 16.0, 0.76, 0.53},
+             {8, 52, 20.5, 0.99, 0.75}, {16, 55, 33.0, 1.59, 1.35}};
     const double x = n * 1e-3;
     double best = INFINITY;
     for (const auto& t : T) {
