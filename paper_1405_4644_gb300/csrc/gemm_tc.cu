@@ -802,7 +802,8 @@ spd_status tc_gemm_launch(TcGemm* g, cudaStream_t s, int cy0, int cx0, int M, in
     const float scale = g->kind == 4 ? 1.0f / (tc_fp8_scale() * tc_fp8_scale()) : 1.0f;
     // float32 as three bf16 slices: the six slice products of order <= 2 (A
     // slice in bits 4q..4q+1, B slice in bits 4q+2..4q+3 of segment q); the
-    // five small ones into accumulator 0, s0*t0 into accumulator 1
+    // five small ones into accumulator 0, s0*t0 into accumulator 1 (the narrow tiles
+    // have an accumulator for each order)
     int nseg = 1;
     uint32_t segs = 0, accsel = 0;
     if (g->kind == 5) {

@@ -79,3 +79,17 @@ def test_one_super_block(h, n, m):
     # float32 products with an explicit float32 inverse: n^1/2 2^-24 times cond(L) squared
     tol = 8 * n ** 0.5 * 2.0 ** -24 * np.linalg.cond(L) ** 2
     assert np.linalg.norm(Z.cpu().numpy() - want) <= tol * np.linalg.norm(want)
+
+
+@pytest.mark.parametrize("e", [-140, -127, -126, -125, 0, 123, 124, 125, 126])
+def test_conversion_at_the_ends_of_the_exponent_range(h, e):
+    """A diagonal matrix without scaling: its entries reach the leaf by the conversion alone."""
+    n = 70
+    m = np.where(np.arange(n) % 3 == 0, 1.0, np.where(np.arange(n) % 3 == 1, 1.5, 1.9375))  # short: exact as subnormals
+    a = m * 2.0 ** e
+    st, F, _ = spd.spd_factor(h, dev_sym(np.diag(a)), "fp32", flags=0)
+    check(h, st)
+    L, _, _ = factor_L(F)
+    spd.spd_factor_destroy(F)
+    # three roundings of 2^-24 in the conversion (none here), one square root and one product
+    assert np.max(np.abs(np.diag(L) / np.sqrt(a) - 1.0)) <= 2.0 ** -21
