@@ -436,16 +436,21 @@ spd_status factor_once(spd_handle* h, int n, const double* A, int lda, int prec,
         free_factor(F);
         return s;
     };
+    bool use_sb = !(flags & SPD_FACTOR_BLOCK_SWEEPS) && sb_sweeps(F->nblk128);
     {  // the factor's whole device request against the handle's cap
         const size_t nb = (size_t)std::max(F->nblk128, 1);
         size_t req = sizeof(double) * std::max(n, 1);
         if (prec == SPD_PREC_FP64) req += sizeof(double) * (std::max<size_t>(nW, 1) + 4096 * nb);
         else req += sizeof(float) * (std::max<size_t>(nW, 1) + (1 + 4 + 0.25) * 16384 * nb) +
-                    (kind ? mirror_elem(kind) * std::max<size_t>(nW, 1) : 0) +
-                    (sb_sweeps((int)nb) && !(flags & SPD_FACTOR_BLOCK_SWEEPS)
-                         ? sizeof(float) * (size_t)ceil_div((long)nb, SPD_SB_BLOCKS) * SPD_SB_BLOCKS * 128 *
-                               SPD_SB_BLOCKS * 128
-                         : 0);
+                    (kind ? mirror_elem(kind) * std::max<size_t>(nW, 1) : 0);
+        if (use_sb && prec != SPD_PREC_FP64) {
+            const size_t sb = sizeof(float) * (size_t)ceil_div((long)nb, SPD_SB_BLOCKS) * SPD_SB_BLOCKS * 128 *
+                              SPD_SB_BLOCKS * 128;
+            // one super-block's inverse is large beside a small factor: a cap that
+            // leaves no room for it gets the 128-block sweeps
+            if ((int)nb <= SPD_SB_BLOCKS && over_cap(h, req + sb)) use_sb = false;
+            else req += sb;
+        }
         if (over_cap(h, req))
             return fail(set_err(h, SPD_ERR_OOM, "factor of order %d needs %zu bytes, above the handle's memory cap "
                                 "of %zu bytes", n, req, h->mem_cap));
@@ -533,7 +538,7 @@ spd_status factor_once(spd_handle* h, int n, const double* A, int lda, int prec,
             // inverses of the diagonal blocks and of the diagonal super-blocks (for
             // the super-block sweeps): off the factorisation's critical path, all
             // blocks at once
-            if (!(flags & SPD_FACTOR_BLOCK_SWEEPS) && sb_sweeps(F->nblk128)) {
+            if (use_sb) {
                 F->sbb = SPD_SB_BLOCKS;
                 F->nsb = ceil_div(F->nblk128, F->sbb);
                 const size_t S = (size_t)F->sbb * 128;

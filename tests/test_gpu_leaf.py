@@ -93,3 +93,31 @@ def test_conversion_at_the_ends_of_the_exponent_range(h, e):
     spd.spd_factor_destroy(F)
     # three roundings of 2^-24 in the conversion (none here), one square root and one product
     assert np.max(np.abs(np.diag(L) / np.sqrt(a) - 1.0)) <= 2.0 ** -21
+
+
+@pytest.mark.parametrize("n", [200, 1024])
+def test_one_super_block_under_a_memory_cap(h, n):
+    """A cap that holds the factor but not its super-block's inverse: the block sweeps serve."""
+    import torch
+    A = W.gram_shifted(n, seed=n, shift=0.5)
+    At = dev_sym(A)
+    B = torch.from_numpy(W.gaussian_rhs(n, 1, 3).T.copy()).to(At.device).t()
+    nb, ldw = -(-n // 128), -(-n // 64) * 64
+    need = 8 * n + 4 * (n * ldw + 86016 * nb) + 6 * n * ldw  # d, W, the blocks' inverses and couplings, the mirror
+    X = {}
+    try:
+        for cap in (0, need):
+            spd.spd_set_memory_cap(h, cap)
+            st, F, _ = spd.spd_factor(h, At, "fp32")
+            check(h, st)
+            spd.spd_set_memory_cap(h, 0)
+            Z = torch.zeros_like(B)
+            check(h, spd.spd_factor_solve(h, F, B, Z))
+            spd.spd_factor_destroy(F)
+            X[cap] = Z.cpu().numpy()
+    finally:
+        spd.spd_set_memory_cap(h, 0)
+    ref = np.linalg.solve(A, B.cpu().numpy())
+    tol = 8 * n ** 0.5 * 2.0 ** -24 * np.linalg.cond(A)  # as two float32 solves
+    for x in X.values():
+        assert np.linalg.norm(x - ref) <= tol * np.linalg.norm(ref)
