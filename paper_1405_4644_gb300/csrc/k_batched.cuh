@@ -344,7 +344,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batch_chol_ir(BatchArgs a) {
         __syncthreads();
         // factor (A1-A3) by 32-column panels
         const int nb = (n + 31) / 32;
-        for (int kb = 0; kb < nb && !s_bad; ++kb) {
+        // (s_bad is read only behind the barrier after the diagonal block: in the loop's
+        // condition a late warp could meet this block's value and leave the others there)
+        for (int kb = 0; kb < nb; ++kb) {
             const int k0 = kb * 32;
             if (warp == 0) {
                 float av[32];
