@@ -246,6 +246,9 @@ __device__ __forceinline__ double batch_row_dot(const BatchSys& S, const double*
     return (q[0] + q[1]) + (q[2] + q[3]);
 }
 
+// |v| for a maximum that decides convergence: NaN counts as infinity (fmax drops it)
+__device__ __forceinline__ double abs_or_inf(double v) { return v == v ? fabs(v) : INFINITY; }
+
 // The block's sum of s and maxima of m1 and m2, one pass (red: 3 NT / 32 values)
 template <int NT>
 __device__ __forceinline__ void block_sum_max2(double& s, double& m1, double& m2, double* red) {
@@ -269,8 +272,8 @@ __device__ __forceinline__ void block_sum_max2(double& s, double& m1, double& m2
 }
 
 // r = b - A x (float64) for one system; returns berr = ||r||_inf / (anorm
-// ||x||_inf); with want_anorm anorm = ||A||_inf is formed first.  x is complete (a
-// barrier before the call).
+// ||x||_inf), infinity where r is not finite; with want_anorm anorm = ||A||_inf is
+// formed first.  x is complete (a barrier before the call).
 template <int NT>
 __device__ double batch_residual(const BatchSys& S, const double* x, double* r, bool want_anorm, double* red,
                                  double* anorm) {
@@ -279,7 +282,7 @@ __device__ double batch_residual(const BatchSys& S, const double* x, double* r, 
         double a = 0.0;
         const double s = S.B[i] - (want_anorm ? batch_row_dot<true>(S, x, i, a) : batch_row_dot<false>(S, x, i, a));
         r[i] = s;
-        rmax = fmax(rmax, fabs(s));
+        rmax = fmax(rmax, abs_or_inf(s));
         xmax = fmax(xmax, fabs(x[i]));
         amax = fmax(amax, a);
     }
@@ -290,6 +293,7 @@ __device__ double batch_residual(const BatchSys& S, const double* x, double* r, 
         __syncthreads();
     }
     const double an = *anorm;
+    if (rmax == INFINITY) return INFINITY;
     return (an > 0.0 && xmax > 0.0) ? rmax / (an * xmax) : rmax;
 }
 
@@ -532,7 +536,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batch_pcg(BatchArgs a) {
             }
             block_sum_max2<NT>(rho, xmax, rmax, red);  // its barriers also publish ps
             for (; it < a.maxit; ++it) {
-                if (xmax > 0.0 && rmax <= 0.5 * a.tol * s_anorm * xmax) break;
+                // (r = 0: b = 0, or nothing left to reduce; alpha would be 0 / 0.  A maximum
+                // of nothing but NaN is 0 too, and the residual below tells the two apart)
+                if (rmax == 0.0 || (xmax > 0.0 && rmax <= 0.5 * a.tol * s_anorm * xmax)) break;
                 double pq = 0.0;
                 for (int i = tid; i < n; i += NT) {
                     double none;
