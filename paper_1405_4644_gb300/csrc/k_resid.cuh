@@ -20,8 +20,9 @@
 
 // |a| rounded to float32 (half up) by 32-bit integer operations without a branch:
 // a float64 -> float32 conversion runs at the float64 rate, a small fraction of
-// the float32 one; below 2^-126 counts as 0, above float range (and NaN) as
-// infinity
+// the float32 one (and a branch to it for what float32 does not hold cost 70 us of
+// the first residual at n = 16384).  Below 2^-126 counts as 0, above float range and
+// NaN as infinity: k_anorm sums such rows again.
 __device__ __forceinline__ float f64_absf(double a) {
     const uint32_t hi = (uint32_t)__double2hiint(a) & 0x7FFFFFFFu, lo = (uint32_t)__double2loint(a);
     uint32_t f = __funnelshift_l(lo, hi, 3) - 0xC0000000u + ((lo >> 28) & 1u);
@@ -187,8 +188,13 @@ static __global__ void __launch_bounds__(256) k_colnorms(const double* __restric
 // result does not depend on the order; *anorm starts at 0).  NaN rows are left
 // out, as by fmax.  One CTA alone took 83 us for 8 x 16384 sums, 300 for 64 x
 // 8191: its loads' latency, row after row.
+//
+// The partial sums are float32, without the entries below 2^-126.  A row whose sum is
+// infinite (an entry or the sum above float32's range, or a NaN), or below 2^-90, where
+// those entries (n 2^-126 of them) could count, is summed again from A in float64 by
+// its thread: seldom, and then a pass over such rows with sixteen loads in flight each.
 static __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ rowabs, int S, int n,
-                                                double* __restrict__ anorm) {
+                                                const double* __restrict__ A, long lda, double* __restrict__ anorm) {
     __shared__ double red[8];
     const int i = blockIdx.x * 256 + threadIdx.x;
     double s = 0.0;
@@ -202,6 +208,11 @@ static __global__ void __launch_bounds__(256) k_anorm(const float* __restrict__ 
             for (int u = 0; u < 8; ++u) s += (double)v[u];
         }
         for (; k < S; ++k) s += (double)rowabs[(long)k * n + i];
+        if (s < 0x1p-90 || s == INFINITY) {
+            s = 0.0;
+#pragma unroll 16
+            for (int j = 0; j < n; ++j) s += fabs(__ldg(A + (long)j * lda + i));
+        }
     }
     const double best = warp_max(fmax(0.0, s));
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = best;

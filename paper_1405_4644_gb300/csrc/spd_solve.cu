@@ -278,7 +278,7 @@ spd_status resid_run(spd_handle* h, const ResidWs& w, int n, int m, const double
         }
         if (anorm) {
             CUDA_TRY(h, cudaMemsetAsync(anorm, 0, sizeof(double), s));
-            ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.tc->rowabs, w.tc->RS, n, anorm);
+            ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.tc->rowabs, w.tc->RS, n, A, lda, anorm);
             LAUNCH_CHECK(h);
         }
         return SPD_OK;
@@ -317,7 +317,7 @@ spd_status resid_run(spd_handle* h, const ResidWs& w, int n, int m, const double
     }
     if (anorm) {
         CUDA_TRY(h, cudaMemsetAsync(anorm, 0, sizeof(double), s));
-            ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.rowabs, S, n, anorm);
+        ++(h)->launches, k_anorm<<<G, 256, 0, s>>>(w.rowabs, S, n, A, lda, anorm);
         LAUNCH_CHECK(h);
     }
     return SPD_OK;
