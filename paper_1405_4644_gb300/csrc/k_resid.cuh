@@ -259,19 +259,24 @@ struct IrSummary {
     double max_berr;  // max over columns of the backward error
     double max_rel;   // max over columns of ||r||_2 / ||b||_2
     int pending;      // columns that met the rule on a residual not allowed to accept
+    int lost;         // active columns that no sweep brings back (k_ir_check)
 };
 
-// One CTA: update per-column state from colnorms; crit as spd_crit.
+// One CTA: update per-column state from colnorms; crit as spd_crit.  The maxima in
+// colnorms and in anorm leave NaN out (fmax), the 2-norm does not: a column whose
+// 2-norm is NaN has an infinite error by every rule, and so has, by the backward
+// error, every column of a matrix whose norm is infinite.
 static __global__ void k_ir_check(const double* __restrict__ colnorms, const double* __restrict__ anorm,
                            const double* __restrict__ b2, int m, int crit, double tol,
                            IrCol* __restrict__ cols, IrSummary* __restrict__ sum, int count_sweep, int polish,
                            int accept = 1, int restart = 0) {
-    __shared__ int s_active, s_stag, s_pend;
+    __shared__ int s_active, s_stag, s_pend, s_lost;
     __shared__ double s_berr, s_rel;
     if (threadIdx.x == 0) {
         s_active = 0;
         s_stag = 0;
         s_pend = 0;
+        s_lost = 0;
         s_berr = 0.0;
         s_rel = 0.0;
     }
@@ -282,6 +287,9 @@ static __global__ void k_ir_check(const double* __restrict__ colnorms, const dou
         double an = *anorm;
         double berr = (an > 0.0 && xinf > 0.0) ? rinf / (an * xinf) : rinf;
         double rel = (b2[c] > 0.0) ? r2 / b2[c] : r2;
+        const bool nan = r2 != r2, wild = !(an < INFINITY);
+        if (nan || wild) berr = INFINITY;
+        if (nan) rel = r2 = INFINITY;
         double err = (crit == 0) ? berr : (crit == 1 ? rel : r2);
         if (!st.conv) {
             if (count_sweep) st.iters += 1;
@@ -309,6 +317,7 @@ static __global__ void k_ir_check(const double* __restrict__ colnorms, const dou
         }
         cols[c] = st;
         if (!st.conv) atomicAdd(&s_active, 1);
+        if (!st.conv && (nan || (crit == 0 && wild))) atomicAdd(&s_lost, 1);
         if (!st.conv && st.stall >= 2) atomicAdd(&s_stag, 1);
         // max of non-negative doubles through their bit patterns (order-independent)
         atomicMax((unsigned long long*)&s_berr, (unsigned long long)__double_as_longlong(berr));
@@ -319,6 +328,7 @@ static __global__ void k_ir_check(const double* __restrict__ colnorms, const dou
         sum->active = s_active;
         sum->stagnated = s_stag;
         sum->pending = s_pend;
+        sum->lost = s_lost;
         sum->max_berr = s_berr;
         sum->max_rel = s_rel;
     }

@@ -894,6 +894,10 @@ spd_status cg_ir_core(spd_handle* h, CgWs& w, int n, int m, const double* A, lon
         st = read_summary(h, w.sum, &sm);
         if (st != SPD_OK) return st;
         if (sm.active == 0) break;
+        if (sm.lost == sm.active) {
+            *last = sm;
+            return set_err(h, SPD_ERR_NO_CONVERGENCE, "CG refinement: the residual of %d columns is not finite", sm.lost);
+        }
         if (outer >= o.maxit) {
             *last = sm;
             return set_err(h, SPD_ERR_NO_CONVERGENCE, "CG refinement: %d columns above tolerance after %d outer steps",
@@ -1111,6 +1115,10 @@ extern "C" spd_status spd_solve_ir(spd_handle* h, const spd_factor_t* F, int n, 
         st = read_summary(h, w.sum, &sm);
         if (st != SPD_OK) return st;
         if (sm.active == 0) break;
+        if (sm.lost == sm.active) {
+            result = set_err(h, SPD_ERR_NO_CONVERGENCE, "refinement: the residual of %d columns is not finite", sm.lost);
+            break;
+        }
         if (sweeps >= o.maxit) {
             result = set_err(h, SPD_ERR_NO_CONVERGENCE, "refinement: %d columns above tolerance after %d sweeps",
                              sm.active, sweeps);
