@@ -294,7 +294,8 @@ __device__ double batch_residual(const BatchSys& S, const double* x, double* r, 
     }
     const double an = *anorm;
     if (rmax == INFINITY) return INFINITY;
-    return (an > 0.0 && xmax > 0.0) ? rmax / (an * xmax) : rmax;
+    // (x = 0 solves b = 0 only)
+    return (an > 0.0 && xmax > 0.0) ? rmax / (an * xmax) : rmax > 0.0 ? INFINITY : 0.0;
 }
 
 template <int NT>

@@ -285,7 +285,8 @@ static __global__ void k_ir_check(const double* __restrict__ colnorms, const dou
         IrCol st = cols[c];
         double rinf = colnorms[3 * c], r2 = colnorms[3 * c + 1], xinf = colnorms[3 * c + 2];
         double an = *anorm;
-        double berr = (an > 0.0 && xinf > 0.0) ? rinf / (an * xinf) : rinf;
+        // (x = 0 solves b = 0 only)
+        double berr = (an > 0.0 && xinf > 0.0) ? rinf / (an * xinf) : rinf > 0.0 ? INFINITY : 0.0;
         double rel = (b2[c] > 0.0) ? r2 / b2[c] : r2;
         const bool nan = r2 != r2, wild = !(an < INFINITY);
         if (nan || wild) berr = INFINITY;
