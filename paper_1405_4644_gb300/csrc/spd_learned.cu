@@ -57,23 +57,26 @@ void gemm(spd_handle* h, int M, int N, int K, const float* A, long sam, long sak
 }
 
 // The weight gradients: C (M x N, dense) = A B over K = the rows of the batch, in
-// slices of 128 of K (at most GRAD_SLICES) added in order; part holds the slices.
+// slices of 128 of K (at most GRAD_SLICES) added in order; part holds the slices
+// (NULL: one slice, straight to C).
 constexpr int GRAD_SLICES = 32;
 void gemm_grad(spd_handle* h, int M, int N, int K, const float* A, long sam, long sak, const float* B, long sbk,
                long sbn, float* C, float* part) {
-    const int ks = std::max(128, (int)round_up(ceil_div(K, GRAD_SLICES), 16)), Z = ceil_div(K, ks);
+    const int ks = part ? std::max(128, (int)round_up(ceil_div(K, GRAD_SLICES), 16)) : K, Z = ceil_div(K, ks);
     dim3 grid((N + 63) / 64, (M + 63) / 64, Z);
     const long cnt = (long)M * N;
-    ++h->launches, k_gemm_strided<<<grid, 256, 0, h->stream>>>(M, N, K, A, sam, sak, B, sbk, sbn, part, N, 1.f, 0.f, 0,
-                                                               ks, cnt);
-    ++h->launches, k_sum_slices<<<grid_for(cnt, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, cnt, C);
+    ++h->launches, k_gemm_strided<<<grid, 256, 0, h->stream>>>(M, N, K, A, sam, sak, B, sbk, sbn, part ? part : C, N,
+                                                               1.f, 0.f, 0, ks, cnt);
+    if (part)
+        ++h->launches, k_sum_slices<<<grid_for(cnt, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, cnt, C);
 }
 
-// out = column sums of dZ (rows x N), in row chunks added in order
+// out = column sums of dZ (rows x N), in row chunks added in order (part NULL: one)
 void colsum(spd_handle* h, const float* dZ, int rows, int N, float* out, float* part) {
-    const int chunk = std::max(64, ceil_div(rows, 64)), Z = ceil_div(rows, chunk);
-    ++h->launches, k_colsum<<<dim3((N + 127) / 128, Z), 128, 0, h->stream>>>(dZ, rows, N, chunk, part);
-    ++h->launches, k_sum_slices<<<grid_for(N, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, N, out);
+    const int chunk = part ? std::max(64, ceil_div(rows, 64)) : rows, Z = ceil_div(rows, chunk);
+    ++h->launches, k_colsum<<<dim3((N + 127) / 128, Z), 128, 0, h->stream>>>(dZ, rows, N, chunk, part ? part : out);
+    if (part)
+        ++h->launches, k_sum_slices<<<grid_for(N, 256, 8 * h->sms), 256, 0, h->stream>>>(part, Z, N, out);
 }
 
 spd_status ensure_acts(spd_mlp* m, int n) {
@@ -109,7 +112,7 @@ void forward(spd_mlp* m, int n, const float* F) {
 }
 
 // backward pass from dO (n x 33) into m->g
-// part: GRAD_SLICES x the largest weight matrix, and 64 x H for the column sums
+// part (may be NULL): GRAD_SLICES x the largest weight matrix, and 64 x H for the column sums
 size_t backward_part(const spd_mlp* m) {
     return std::max((size_t)GRAD_SLICES * m->H * std::max({m->H, m->O, m->F}), (size_t)64 * std::max(m->H, m->O));
 }
@@ -141,7 +144,7 @@ __global__ void k_sdiag(const double* __restrict__ A, long lda, int n, double* _
 // Q = A P in float64 (A column-major symmetric, P n x p with ld n): the split-K
 // partial sums of the residual (k_resid_partial; bound by the float64 rate), then
 // their sum in order.  A thread per row over all of A kept ceil(n / 256) SMs busy:
-// 3.4 ms at n = 4096, p = 8.
+// 3.4 ms at n = 4096, p = 8; part = NULL does just that, straight into Q.
 __global__ void k_sum_parts64(const double* __restrict__ P, int S, long count, double* __restrict__ Q) {
     for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < count; e += (long)gridDim.x * blockDim.x) {
         double s = 0.0;
@@ -153,18 +156,20 @@ int prod64_splits(const spd_handle* h, int n) {
     return std::max(1, std::min(ceil_div(4 * h->sms, ceil_div(n, RESID_ROWS)), n / (2 * RESID_JT)));
 }
 void prod64(spd_handle* h, const double* A, long lda, int n, const double* P, int p, double* Q, double* part) {
-    const int S = prod64_splits(h, n), jchunk = (int)round_up(ceil_div(n, S), RESID_JT);
+    const int S = part ? prod64_splits(h, n) : 1, jchunk = (int)round_up(ceil_div(n, S), RESID_JT);
     const dim3 grid(ceil_div(n, RESID_ROWS), S);
     cudaStream_t s = h->stream;
+    double* out = part ? part : Q;
     for (int c0 = 0; c0 < p; c0 += 16) {
         const int pc = std::min(16, p - c0);
         ++h->launches;
-        if (pc == 1) k_resid_partial<1><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
-        else if (pc <= 4) k_resid_partial<4><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
-        else if (pc <= 8) k_resid_partial<8><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
-        else k_resid_partial<16><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, part, nullptr);
+        if (pc == 1) k_resid_partial<1><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, out, nullptr);
+        else if (pc <= 4) k_resid_partial<4><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, out, nullptr);
+        else if (pc <= 8) k_resid_partial<8><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, out, nullptr);
+        else k_resid_partial<16><<<grid, RESID_ROWS, 0, s>>>(A, lda, n, P, n, c0, pc, jchunk, p, out, nullptr);
     }
-    ++h->launches, k_sum_parts64<<<grid_for((long)n * p, 256, 8 * h->sms), 256, 0, s>>>(part, S, (long)n * p, Q);
+    if (part)
+        ++h->launches, k_sum_parts64<<<grid_for((long)n * p, 256, 8 * h->sms), 256, 0, s>>>(part, S, (long)n * p, Q);
 }
 
 // PV[c][k] = sum_i Uh_ik V_ic: block (x, c) over rows [256 x, 256 x + 256) as
@@ -283,8 +288,8 @@ spd_status build_core(spd_mlp* m, spd_lowrank* P, int n, int* dbad) {
     spd_handle* h = m->h;
     ++h->launches, k_out_to_dU<<<grid_for(n, 256, 4 * h->sms), 256, 0, h->stream>>>(m->Ob, n, P->dh, P->Uh);
     CUDA_TRY(h, cudaMemsetAsync(dbad, 0, sizeof(int), h->stream));
-    // the Gram term over 128-row chunks on many SMs, then one CTA for the
-    // 32 x 32 core (one float64 division per row, not per row and entry)
+    // the Gram term over CORE_ROWS-row chunks on many SMs, then one CTA for the
+    // 32 x 32 core
     const int G = ceil_div(n, CORE_ROWS);
     double* part = nullptr;
     CUDA_TRY(h, cudaMallocAsync(&part, sizeof(double) * (size_t)G * LR_RANK * LR_RANK, h->stream));
@@ -534,15 +539,20 @@ extern "C" spd_status spd_mlp_loss_grad(spd_mlp* m, int n, const double* A, int 
            o_w = pl.add<double>((size_t)wb_chunks(n) * LR_RANK * p),
            o_sums = pl.add<double>(2 * p + 2), o_coef = pl.add<double>(p), o_dh = pl.add<double>(n),
            o_Uh = pl.add<double>((size_t)n * LR_RANK), o_Lc = pl.add<double>(2 * LR_RANK * LR_RANK),
-           o_bad = pl.add<int>(1), o_parts = pl.add<double>((size_t)prod64_splits(h, n) * np),
-           o_bpart = pl.add<float>(backward_part(m));
-    if ((st = ws_reserve(h, pl.bytes)) != SPD_OK) return st;
+           o_bad = pl.add<int>(1);
+    // the splits' partial sums, left out where they don't fit (n = 4096, p = 8, hidden
+    // 256: 17 MB beside 3)
+    WsPlan full = pl;
+    size_t o_parts = full.add<double>((size_t)prod64_splits(h, n) * np), o_bpart = full.add<float>(backward_part(m));
+    const bool split = (st = ws_reserve(h, full.bytes)) == SPD_OK;
+    if (st == SPD_ERR_OOM) st = ws_reserve(h, pl.bytes);
+    if (st != SPD_OK) return st;
     double *sd = ws_at<double>(h, o_sd), *Y = ws_at<double>(h, o_Y), *Q = ws_at<double>(h, o_Q),
            *E = ws_at<double>(h, o_E), *G = ws_at<double>(h, o_G), *Wv = ws_at<double>(h, o_Wv),
            *Yh = ws_at<double>(h, o_Yh), *Wh = ws_at<double>(h, o_Wh), *PY = ws_at<double>(h, o_PY),
            *PW = ws_at<double>(h, o_PW), *wb = ws_at<double>(h, o_w), *sums = ws_at<double>(h, o_sums),
-           *coef = ws_at<double>(h, o_coef), *parts = ws_at<double>(h, o_parts);
-    float* bpart = ws_at<float>(h, o_bpart);
+           *coef = ws_at<double>(h, o_coef), *parts = split ? ws_at<double>(h, o_parts) : nullptr;
+    float* bpart = split ? ws_at<float>(h, o_bpart) : nullptr;
     spd_lowrank P;
     P.h = h;
     P.n = n;
