@@ -791,8 +791,6 @@ size_t cg_plan(WsPlan& p, spd_handle* h, int n, int m, size_t* o, int* S, int* G
     o[11] = p.add<double>(nm);      // Z
     o[12] = p.add<double>(nm);      // P
     o[13] = p.add<double>(nm);      // Q
-    // part: p^T q, written by k_dot2, the products (32-row blocks) or the band step
-    o[14] = p.add<double>((size_t)std::max(*G2, m <= MV_DOT_MAXM ? ceil_div(n, MV_ROWS) : ceil_div(n, CGB_ROWS)) * m * 2);
     o[15] = p.add<double>(nm);      // Yz (factor preconditioner scratch)
     o[16] = p.add<float>(nm);       // Pf
     o[17] = p.add<IrCol>(m);
@@ -800,7 +798,13 @@ size_t cg_plan(WsPlan& p, spd_handle* h, int n, int m, size_t* o, int* S, int* G
     o[19] = p.add<CgCol>(m);
     o[20] = p.add<int>(m);          // frozen
     o[21] = p.add<int>(1);          // active
-    o[22] = p.add<double>((size_t)(*G2) * m * 2);  // part2: r^T z, r^T r
+    // part: p^T q, written by k_dot2, the products (32-row blocks) or the band step;
+    // part2: r^T z, r^T r.  Both lie in the residual's partial sums (n m doubles and
+    // more), which only a float64 product writes, between the steps' reads and writes
+    // of the two; for n < 4 in its block norms (3 m doubles) and an array of its own.
+    const size_t np = (size_t)std::max(*G2, m <= MV_DOT_MAXM ? ceil_div(n, MV_ROWS) : ceil_div(n, CGB_ROWS)) * m * 2;
+    o[14] = n < 4 ? o[2] : o[0];
+    o[22] = n < 4 ? p.add<double>((size_t)2 * m) : o[0] + sizeof(double) * np;
     return p.bytes;
 }
 

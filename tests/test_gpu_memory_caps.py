@@ -1,10 +1,12 @@
 """Calls under a memory cap that leaves room for what they cannot do without: partial
 sums that only serve speed are left out, and the call is served."""
+import numpy as np
 import pytest
 import torch
 
 import paper_1405_4644_gb300 as spd
 import workloads as W
+from tests.gpu_util import dev_cols, dev_sym, dev_zeros
 from tests.test_gpu_learned_shapes import loss64
 
 pytestmark = pytest.mark.gpu
@@ -45,5 +47,76 @@ def test_training_step(n, p, H):
                 assert abs(L - L64) <= tol * abs(L64)
                 assert float((grad.double() - g64).norm()) <= tol * float(g64.norm())
         spd.spd_mlp_destroy(net)
+    finally:
+        spd.spd_destroy(h)
+
+
+def solver_request(n, m):
+    """spd_solve_ir with the float64 residual: the residual's partial sums, eight vectors of
+    n m and float32 copies, one pair of dot partials per row chunk and column, the
+    columns' state."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    blocks = -(-n // 256)
+    split = min(max(1, (4 * sms + blocks - 1) // blocks), max(1, n // 256))  # float64 kernel
+    best, best_eff = 1, -1.0  # float32-pair kernel
+    for s in range(1, max(1, n // 128) + 1):
+        ctas = blocks * s
+        eff = ctas / (-(-ctas // (2 * sms)) * 2 * sms)
+        if ctas < 4 * sms and s < max(1, n // 128):
+            eff *= 0.5
+        if eff > best_eff + 1e-9:
+            best, best_eff = s, eff
+        if ctas >= 8 * sms:
+            break
+    split = max(split, best)
+    dots = max(1, min(2 * sms, blocks) // m)
+    nm = n * m
+    return [8 * split * nm, 4 * split * n, 8 * 3 * blocks * m, 16 * m, 8 * nm, 24 * m, 8, 8 * m, 8 * m, *[8 * nm] * 5,
+            16 * dots * m, 8 * nm, 4 * nm, 32 * m, 32, 56 * m, 4 * m, 4]
+
+
+SHAPES = [(1, 1), (2, 40), (2, 3), (3, 9), (4, 8), (33, 8), (300, 1), (2000, 8), (2000, 33), (3000, 16)]
+
+
+@pytest.mark.parametrize("n,m", SHAPES)
+def test_refinement(n, m):
+    A = W.gram_shifted(n, seed=n, shift=0.5)
+    Ad, Bd, X = dev_sym(A), dev_cols(W.gaussian_rhs(n, m, 1)), dev_zeros(n, m)
+    h = spd.spd_create(torch.cuda.current_stream())
+    try:
+        st, F, _ = spd.spd_factor(h, Ad, "fp32")
+        assert st == spd.SPD_OK
+        spd.spd_set_memory_cap(h, total(*solver_request(n, m)))
+        st, rep = spd.spd_solve_ir(h, F, Ad, Bd, X, {"resid": "fp64"})
+        assert st == spd.SPD_OK and rep.berr <= 1e-14
+        spd.spd_factor_destroy(F)
+    finally:
+        spd.spd_destroy(h)
+
+
+@pytest.mark.parametrize("kind", ["fp32", "bf16", "fp64", "band", "jacobi"])
+@pytest.mark.parametrize("n,m", SHAPES)
+def test_cg(n, m, kind):
+    # the inner matrix: float32 (rows to a multiple of 64), bf16, a band of half-width 3 or none
+    inner = {"fp32": 4 * n * (-(-n // 64) * 64), "bf16": 2 * n * (-(-n // 64) * 64), "fp64": 0, "band": 4 * 7 * n,
+             "jacobi": 4 * 7 * n}[kind]
+    A = W.gram_shifted(n, seed=n, shift=2.0)
+    if kind in ("band", "jacobi"):
+        i = np.arange(n)
+        A = np.where(np.abs(i[:, None] - i) <= 3, A, 0.0)
+        A[i, i] = 8.0 + i / n
+    Ad, Bd, X = dev_sym(A), dev_cols(W.gaussian_rhs(n, m, 1)), dev_zeros(n, m)
+    extra = [8 * n] if kind == "jacobi" else []
+    opts = {"resid": "fp64", "matvec_cores": "cuda" if kind == "fp32" else "auto"}
+    if kind in ("band", "jacobi"):
+        opts["band"] = 3
+    h = spd.spd_create(torch.cuda.current_stream())
+    try:
+        spd.spd_set_memory_cap(h, total(*solver_request(n, m), inner, *extra))
+        st, rep = spd.spd_cg(h, Ad, Bd, X, kind if kind in ("fp32", "bf16", "fp64") else "fp32",
+                             pc="jacobi" if kind == "jacobi" else "none", opts=opts)
+        assert st == spd.SPD_OK and rep.berr <= 1e-14
+        R = np.abs(Bd.cpu().numpy() - A @ X.cpu().numpy()).max(0)
+        assert np.all(R <= (1e-14 + n * 2.0**-53) * np.abs(A).sum(1).max() * np.abs(X.cpu().numpy()).max(0))
     finally:
         spd.spd_destroy(h)
