@@ -28,13 +28,16 @@ struct spd_batch {
 namespace {
 
 // CTAs of a launch: 512 threads per SM (the kernels' launch bounds), no more than
-// systems
-int batch_ctas(const spd_batch* b, int nt) { return std::max(1, std::min(b->h->sms * (512 / nt), b->count)); }
+// systems, and for Cholesky-IR no more than have scratch
+int batch_ctas(const spd_batch* b, int method, int nt) {
+    const int g = std::max(1, std::min(b->h->sms * (512 / nt), b->count));
+    return method == SPD_BATCH_CHOL_IR ? std::min(g, b->ctas) : g;
+}
 
 template <int NT>
 void launch_batch(spd_batch* b, int method, const BatchArgs& a, cudaStream_t s) {
-    const int ctas = batch_ctas(b, NT);
-    if (method == 0) k_batch_chol_ir<NT><<<ctas, NT, batch_smem_bytes(), s>>>(a);
+    const int ctas = batch_ctas(b, method, NT);
+    if (method == SPD_BATCH_CHOL_IR) k_batch_chol_ir<NT><<<ctas, NT, batch_smem_bytes(), s>>>(a);
     else k_batch_pcg<NT><<<ctas, NT, batch_pcg_smem_bytes(), s>>>(a);
 }
 
@@ -80,13 +83,23 @@ extern "C" spd_status spd_batch_create(spd_handle* h, int count, const int* n, c
     b->h = h;
     b->count = count;
     b->nmax = nmax;
-    b->ctas = std::max(1, std::min(2 * h->sms, count));  // scratch of the largest Cholesky-IR launch
+    // scratch (1 MB per CTA) of the largest Cholesky-IR launch, two CTAs per SM; one per
+    // SM where two are more than the handle's cap or the device has room for
+    const int one = std::max(1, std::min(h->sms, count));
+    const size_t per_cta = sizeof(float) * BLD * BLD;
+    b->ctas = std::max(1, std::min(2 * h->sms, count));
+    if (over_cap(h, per_cta * b->ctas)) b->ctas = one;
     set_batch_attrs();
     cudaError_t e = cudaMalloc(&b->sys, sizeof(BatchSys) * std::max(count, 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->order, sizeof(int) * std::max(count, 1));
     if (e == cudaSuccess) e = cudaMalloc(&b->next, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&b->rep, sizeof(BatchRep) * std::max(count, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&b->scratch, sizeof(float) * (size_t)b->ctas * BLD * BLD);
+    if (e == cudaSuccess) e = cudaMalloc(&b->scratch, per_cta * b->ctas);
+    if (e == cudaErrorMemoryAllocation && !b->scratch && b->rep && b->ctas > one) {
+        cudaGetLastError();
+        b->ctas = one;
+        e = cudaMalloc(&b->scratch, per_cta * b->ctas);
+    }
     if (e == cudaSuccess && count > 0)
         e = cudaMemcpy(b->sys, hs.data(), sizeof(BatchSys) * count, cudaMemcpyHostToDevice);
     if (e == cudaSuccess && count > 0) e = cudaMemcpy(b->order, order.data(), sizeof(int) * count, cudaMemcpyHostToDevice);
@@ -282,7 +295,7 @@ extern "C" spd_status spd_batch_info(const spd_batch* b, int method, int* thread
     if (!b || (method != SPD_BATCH_CHOL_IR && method != SPD_BATCH_PCG_JACOBI)) return SPD_ERR_ARG;
     const int mi = method == SPD_BATCH_CHOL_IR ? 0 : 1;
     if (threads_per_cta) *threads_per_cta = b->threads[mi];
-    if (ctas) *ctas = batch_ctas(b, b->threads[mi] ? b->threads[mi] : 512);
+    if (ctas) *ctas = batch_ctas(b, method, b->threads[mi] ? b->threads[mi] : 512);
     if (tune_ms) {
         tune_ms[0] = b->tune_ms[mi][0];
         tune_ms[1] = b->tune_ms[mi][1];

@@ -120,3 +120,34 @@ def test_cg(n, m, kind):
         assert np.all(R <= (1e-14 + n * 2.0**-53) * np.abs(A).sum(1).max() * np.abs(X.cpu().numpy()).max(0))
     finally:
         spd.spd_destroy(h)
+
+
+def test_batched_plan():
+    """One CTA's scratch per SM, and as many CTAs, where two per SM are over the cap; a plan
+    is never refused for it."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    sizes = [16 + (7 * k) % 100 for k in range(4 * sms)]
+    dA = [torch.from_numpy(W.gram_shifted(n, seed=k, shift=0.5)).cuda() for k, n in enumerate(sizes)]
+    db = [torch.from_numpy(W.rng(k).standard_normal(n)).cuda() for k, n in enumerate(sizes)]
+    want = None
+    for cap, most in [(0, 2 * sms), (sms << 20, sms), (1 << 16, sms)]:
+        h = spd.spd_create(torch.cuda.current_stream())
+        try:
+            spd.spd_set_memory_cap(h, cap)
+            dx = [torch.zeros_like(b) for b in db]
+            free = torch.cuda.mem_get_info()[0]
+            st, plan = spd.spd_batch_create(h, dA, db, dx)
+            assert st == spd.SPD_OK
+            used = free - torch.cuda.mem_get_info()[0]
+            assert used <= (most << 20) + (32 << 20)  # the tables, and the driver's granularity
+            for method in ("chol_ir", "pcg_jacobi"):
+                st, _, sts, berr, _ = spd.spd_batch_solve(plan, method, "fp32", count=len(sizes))
+                assert st == spd.SPD_OK and np.all(berr[:len(sizes)] <= 1e-14)
+                if method == "chol_ir":
+                    assert spd.spd_batch_info(plan, method)["ctas"] <= most
+                    xs = [x.cpu().numpy() for x in dx]
+                    want = want or xs
+                    assert all(np.array_equal(a, b) for a, b in zip(xs, want))
+            spd.spd_batch_destroy(plan)
+        finally:
+            spd.spd_destroy(h)
