@@ -8,8 +8,9 @@
 // backward (I = last, ..., 0):
 //   z_I = X_I^T y_I, then   y_K -= L_IK^T z_I  for every 128-row block K above,
 // i.e. block substitution with the diagonal solve replaced by a product with
-// the inverse.  One persistent cooperative kernel per sweep runs three
-// grid-wide phases per super-block, separated by bounded grid barriers:
+// the inverse.  One persistent cooperative kernel per sweep runs two grid-wide
+// phases per super-block, separated by bounded grid barriers (a factor of one
+// super-block has phase F alone, no barrier, and is launched as an ordinary kernel):
 //   F   the SBB (SBB + 1) / 2 tile products X_I[b][c] r_I[c] (c <= b; for the
 //       backward sweep X_I[c][b]^T r_I[c], c >= b) into partial tiles; the
 //       last tile of block row b to arrive (an atomic count) adds the row's
@@ -342,11 +343,12 @@ __device__ __forceinline__ void sb_store(float* pt, float (&acc)[4][MC], float* 
     }
 }
 
-// shared memory: y_I of one super-block (SPD_SB_BLOCKS staged 128 x MC blocks) and the
-// eight warps' sums of the backward sweep
+// shared memory: y_I of one super-block (SPD_SB_BLOCKS staged 128 x MC blocks; one
+// where there is no panel to update) and the eight warps' sums of the backward sweep
+__host__ __device__ constexpr int sb_staged(int NS) { return NS == 1 ? 1 : SPD_SB_BLOCKS; }
 template <int MC>
-constexpr size_t trsv_sb_smem() {
-    return (size_t)(SPD_SB_BLOCKS * 128 * tv_ys<MC>() + 8 * 128 * MC) * sizeof(float);
+constexpr size_t trsv_sb_smem(int NS) {
+    return (size_t)(sb_staged(NS) * 128 * tv_ys<MC>() + 8 * 128 * MC) * sizeof(float);
 }
 
 // tile index of the pair (p, q), q <= p, in the order (0,0), (1,0), (1,1), ...
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(256, 1) k_trsv_sb(SbArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float* YI = reinterpret_cast<float*>(smem_raw);  // [SBB][128][tv_ys] staged blocks of y_I (F: one)
     constexpr int YB = 128 * tv_ys<MC>();           // floats per staged block
-    float* red = YI + SPD_SB_BLOCKS * YB;           // backward: the warps' sums
+    float* red = YI + sb_staged(a.NS) * YB;         // backward: the warps' sums
     __shared__ int s_abort, s_last;
     if (a.gate && *a.gate == 0) return;  // refinement over (capturable solves)
     const int tid = threadIdx.x;

@@ -473,15 +473,17 @@ namespace {
 // The scratch (partial tiles, partial slots, barrier words) is sized for
 // SB_GROUPS groups of 16 columns whatever this call has, so that it grows with the
 // order alone; the first call on a handle must not be captured.  mc columns: groups
-// of MC, side by side.
+// of MC, side by side.  One super-block has no barriers: its sweeps are ordinary
+// launches of a CTA per tile of the inverse (at most 36 a group), which neither wait
+// for every SM to be free nor for other streams' cooperative launches.
 template <int MC>
 spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, int c0, int mc) {
-    const size_t smem = trsv_sb_smem<MC>();
+    const size_t smem = trsv_sb_smem<MC>(F->nsb);
     auto fwd = k_trsv_sb<MC, true>;
     auto bwd = k_trsv_sb<MC, false>;
     static const bool attr = [&] {  // once per instantiation, thread-safe
-        cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        cudaFuncSetAttribute(bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        cudaFuncSetAttribute(fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsv_sb_smem<MC>(2));
+        cudaFuncSetAttribute(bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)trsv_sb_smem<MC>(2));
         return true;
     }();
     (void)attr;
@@ -489,10 +491,10 @@ spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, i
     // every SM streams the panel updates: one CTA each (its registers fill the SM),
     // shared out among the column groups
     const int ng = ceil_div(mc, MC), slots = std::max(SB_GROUPS, std::min(h->sms, TV_SLOTS));
-    const int G = slots / ng;
+    const int G = F->nsb == 1 ? F->nblk128 * (F->nblk128 + 1) / 2 : slots / ng;
     const size_t pbytes = sizeof(float) * ntile * 128 * 16;                // per group
     const size_t p2bytes = sizeof(float) * 2 * (size_t)G * 128 * MC;       // per group
-    const size_t p2all = sizeof(float) * 2 * (size_t)slots * 128 * 16;  // ng G <= slots
+    const size_t p2all = sizeof(float) * 2 * (size_t)slots * 128 * 16;  // ng G <= slots (one super-block: no slots)
     const size_t zbytes = (size_t)round_up((long)(sizeof(float) * (size_t)n * 16 * SB_GROUPS), 256);
     const int nbar = 2 + F->nsb * F->sbb;  // per group: barrier words, then the block-row tile counts
     const size_t need = SB_GROUPS * pbytes + p2all + zbytes + sizeof(int) * (size_t)nbar * SB_GROUPS;
@@ -520,8 +522,9 @@ spd_status trsv_sb_pass(spd_handle* h, const spd_factor_t* F, float* Y, int n, i
         void* args[] = {&a};
         CUDA_TRY(h, cudaMemsetAsync(bar, 0, sizeof(int) * nbar * ng, h->stream));
         ++h->launches;
-        CUDA_TRY(h, coop_launch(dir == 0 ? (const void*)fwd : (const void*)bwd, dim3(G, ng), dim3(256), args, smem,
-                                h->stream));
+        const void* fn = dir == 0 ? (const void*)fwd : (const void*)bwd;
+        CUDA_TRY(h, F->nsb == 1 ? cudaLaunchKernel(fn, dim3(G, ng), dim3(256), args, smem, h->stream)
+                                : coop_launch(fn, dim3(G, ng), dim3(256), args, smem, h->stream));
     }
     return SPD_OK;
 }
