@@ -43,7 +43,19 @@ static __global__ void k_features(const double* __restrict__ A, long lda, int n,
     }
     s1 = warp_sum(s1) * si;
     s2 = warp_sum(s2) * (si * si);
-    const double mx = warp_max(__longlong_as_double((long long)mb)) * si;
+    double mx = warp_max(__longlong_as_double((long long)mb)) * si;
+    if (si < 1e-140 || si > 1e140) {  // t_j is up to 1 / s_i: its square may have left float64's range
+        s1 = s2 = mx = 0.0;
+        for (int j = lane; j < n; j += 32) {
+            const double v = fabs(A[(long)i * lda + j] * si * sdiag[j]);
+            s1 += v;
+            s2 = fma(v, v, s2);
+            if (j != i) mx = fmax(mx, v);
+        }
+        s1 = warp_sum(s1);
+        s2 = warp_sum(s2);
+        mx = warp_max(mx);
+    }
     if (lane == 0) {
         const double x = coords[2 * i], y = coords[2 * i + 1];
         const double pi = 3.14159265358979323846;
