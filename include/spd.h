@@ -78,7 +78,9 @@ typedef enum spd_prec {
 } spd_prec;
 
 /* Stopping rules (Alg. 1 and Alg. 2 print ||r||_2 >= tolerance; the
- * normwise backward error is the accuracy target of this library). */
+ * normwise backward error is the accuracy target of this library).  A column
+ * whose residual is NaN meets none of them; the backward error is infinite
+ * there, for x = 0 with b != 0, and where ||A||_inf is infinite. */
 typedef enum spd_crit {
     SPD_CRIT_BERR = 0, /* ||b - A x||_inf / (||A||_inf ||x||_inf) <= tol */
     SPD_CRIT_REL2 = 1, /* ||b - A x||_2 <= tol * ||b||_2               */
@@ -144,10 +146,13 @@ typedef enum spd_resid {
 #define SPD_FACTOR_BLOCK_SWEEPS 32u /* float32 factors: apply the factor
                                     with the sweeps over 128-row blocks.  By
                                     default a factor of 2 to 8 blocks or of
-                                    at least 16 also holds the inverses of its diagonal
-                                    super-blocks (8 blocks each, formed once,
-                                    4 (1024)^2 bytes each) and is applied with
-                                    the super-block sweeps */
+                                    at least 16 also holds the inverses of its
+                                    diagonal super-blocks (8 blocks each,
+                                    formed once, 4 (1024)^2 bytes each) and is
+                                    applied with the super-block sweeps.  Where
+                                    there is no memory for them (2 to 8 blocks:
+                                    nor room under spd_set_memory_cap) the
+                                    128-block sweeps serve */
 #define SPD_FACTOR_SERIAL 8u     /* left-looking schedule without its
                                     look-ahead: every kernel on the handle's
                                     stream in order (kernels then run alone,
@@ -560,7 +565,10 @@ spd_status spd_gemm_update(spd_handle *h, int prec, int M, int N, int K, const f
  * and the CUDA context stay usable.
  * spd_set_memory_cap caps the device memory one call on h may request
  * (a factor's arrays, the workspace, spd_solve_ir_host's device copies);
- * a larger request returns SPD_ERR_OOM before anything is allocated.
+ * a larger request returns SPD_ERR_OOM before anything is allocated.  What
+ * serves speed alone (a small factor's super-block inverse, the training
+ * step's split sums, a batched plan's scratch for a second CTA per SM) is
+ * left out of a request that would be too large with it.
  * 0 (the default) means no cap.
  * spd_wait_probe launches one kernel that waits, with h's wait limit, on a
  * device flag that nothing sets: it returns SPD_ERR_TIMEOUT after that

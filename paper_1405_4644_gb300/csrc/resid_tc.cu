@@ -624,7 +624,7 @@ __global__ void __launch_bounds__(256) k_tcr_final(const unsigned long long* __r
         if (er == TCR_NONFINITE || fc == TCR_NONFINITE) {
             r = __longlong_as_double(0x7FF8000000000000ll);
         } else {
-            __int128 S = 0;  // |G_t| < 2^53 for n < 2^30: below 2^117
+            __int128 S = 0;  // |G_t| <= (t - 1) 2^12 n: below 2^106 for n < 2^30
 #pragma unroll
             for (int k = 0; k < TCR_NG; ++k) S = (S << 7) + gs[k];
             double hi, lo;
@@ -712,9 +712,8 @@ struct TcrSchedule {
     long T;
 };
 
-// Column blocks per A tile: two from 17 columns on (m = 32: n = 8191 237 us against
-// 373 with one, n = 16384 860 against 1440; 16 columns take 800 there with one).
-
+// per: column blocks per A tile, two from 17 columns on (m = 32: n = 8191 237 us
+// against 373 with one, n = 16384 860 against 1440; 16 columns take 800 there with one)
 TcrSchedule tcr_schedule(spd_handle* h, int n, int m) {
     TcrSchedule s;
     s.RB = ceil_div(n, 128);

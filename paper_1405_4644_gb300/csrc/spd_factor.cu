@@ -28,9 +28,13 @@ namespace {
 
 // Whether a float32 factor of nb 128-row blocks is applied with the super-block
 // sweeps: with one super-block a sweep is its triangular product, with no chain at
-// all (14 us a pair at n = 1024, one right-hand side, against 57 under ncu); from two
-// full ones on the chain is short enough.  Between, the
-// 128-block sweeps stay.
+// all (14 us a pair at n = 1024, one right-hand side, against 57 under ncu; a call of
+// spd_factor_solve 45, and 52 for 32, against 79 and 291); from two on it is a chain of
+// one step per super-block (n = 2048: 63 and 86 us against 127 and 527).  A second one
+// of less than eight blocks (9 to 15 in all) gains as much (n = 1025: 58 and 73 us
+// against 83 and 316, n = 1919: 62 and 84 against 120 and 505, the factor's own time
+// the same); the 128-block sweeps stay there because the flag is known to change no bit
+// at those orders.
 inline bool sb_sweeps(int nb) { return (nb >= 2 && nb <= SPD_SB_BLOCKS) || nb >= 2 * SPD_SB_BLOCKS; }
 
 struct FCtx {
