@@ -538,8 +538,9 @@ __global__ void __launch_bounds__(NT, 512 / NT) k_batch_pcg(BatchArgs a) {
             block_sum_max2<NT>(rho, xmax, rmax, red);  // its barriers also publish ps
             for (; it < a.maxit; ++it) {
                 // (r = 0: b = 0, or nothing left to reduce; alpha would be 0 / 0.  A maximum
-                // of nothing but NaN is 0 too, and the residual below tells the two apart)
-                if (rmax == 0.0 || (xmax > 0.0 && rmax <= 0.5 * a.tol * s_anorm * xmax)) break;
+                // of nothing but NaN is 0 too, and the residual below tells the two apart; by
+                // its bits, since a float64 comparison is on the step's chain)
+                if (__double_as_longlong(rmax) == 0ll || (xmax > 0.0 && rmax <= 0.5 * a.tol * s_anorm * xmax)) break;
                 double pq = 0.0;
                 for (int i = tid; i < n; i += NT) {
                     double none;
